@@ -40,28 +40,81 @@ struct GView {
 
 __device__ __forceinline__ float wbf(const __nv_bfloat16 *W, int i) { return __bfloat162float(W[i]); }
 
-// features of one graph by one CTA; d1, d2: scratch of n ints (local index)
+// Rows of a warp's 32 nodes (lane: node v if take): every lane walks its own
+// short row; a row above MP_ROW_LANE entries is spread over the lanes, since a
+// hub's row on one thread holds up the whole CTA.
+// f(entry) for every entry
+constexpr int MP_ROW_LANE = 24;
+template <class XT, class F>
+__device__ __forceinline__ void mp_rows(const GView<XT> &G, bool take, int32_t v, F f) {
+  const int lane = threadIdx.x & 31;
+  XT b = 0, e = 0;
+  if (take) {
+    b = G.xadj[v];
+    e = G.xadj[v + 1];
+  }
+  const bool big = e - b > MP_ROW_LANE;
+  if (!big)
+    for (XT q = b; q < e; ++q) f(q);
+  for (unsigned m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1) {
+    const XT b1 = __shfl_sync(0xFFFFFFFFu, b, __ffs(m) - 1), e1 = __shfl_sync(0xFFFFFFFFu, e, __ffs(m) - 1);
+    for (XT q = b1 + lane; q < e1; q += 32) f(q);
+  }
+}
+// weighted degree of each lane's node (whole warp)
+template <class XT>
+__device__ __forceinline__ int64_t mp_wdeg(const GView<XT> &G, bool take, int32_t v) {
+  const int lane = threadIdx.x & 31;
+  XT b = 0, e = 0;
+  if (take) {
+    b = G.xadj[v];
+    e = G.xadj[v + 1];
+  }
+  if (!G.ew) return (int64_t)(e - b);
+  const bool big = e - b > MP_ROW_LANE;
+  int64_t r = 0;
+  if (!big)
+    for (XT q = b; q < e; ++q) r += G.ew[q];
+  for (unsigned m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1) {
+    const int src = __ffs(m) - 1;
+    const XT b1 = __shfl_sync(0xFFFFFFFFu, b, src), e1 = __shfl_sync(0xFFFFFFFFu, e, src);
+    int64_t x = 0;
+    for (XT q = b1 + lane; q < e1; q += 32) x += G.ew[q];
+    x = warp_sum64(x);
+    if (lane == src) r = x;
+  }
+  return r;
+}
+
+// Features of one graph by one CTA; d1, d2: scratch of n ints (local index).
+// The sums are whole numbers below 2^53, so their doubles are exact.
 template <class XT>
 __device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t *d1, int32_t *d2) {
-  __shared__ double s_c, s_w;
-  __shared__ unsigned long long s_md;
+  __shared__ unsigned long long s_c, s_w, s_md;
   int32_t n = G.n;
+  const int lane = threadIdx.x & 31;
+  const int32_t warp0 = threadIdx.x & ~31;  // the warp's first node of a sweep
   if (threadIdx.x == 0) {
     s_c = 0;
     s_w = 0;
     s_md = 0;
   }
   __syncthreads();
-  double lc = 0, lw = 0;
+  int64_t lc = 0, lw = 0;
   unsigned long long md = 0;
-  for (int32_t v = threadIdx.x; v < n; v += blockDim.x) {
+  for (int32_t v0 = warp0; v0 < n; v0 += blockDim.x) {
+    const int32_t v = v0 + lane;
+    const int64_t wd = mp_wdeg(G, v < n, v);
+    if (v >= n) continue;
     lc += G.vw ? G.vw[v] : 1;
-    for (XT e = G.xadj[v]; e < G.xadj[v + 1]; ++e) lw += G.ew ? G.ew[e] : 1;
+    lw += wd;
+    // kept in the node's feature row until it is scaled
+    *reinterpret_cast<int64_t *>(X + (int64_t)v * MF + 6) = wd;
     unsigned long long d = (unsigned long long)(G.xadj[v + 1] - G.xadj[v]);
     md = d > md ? d : md;
   }
-  atomicAdd(&s_c, lc);
-  atomicAdd(&s_w, lw);
+  atomicAdd(&s_c, (unsigned long long)lc);
+  atomicAdd(&s_w, (unsigned long long)lw);
   atomicMax(&s_md, md);
   __syncthreads();
   // anchor a: smallest key, then smallest id
@@ -78,8 +131,9 @@ __device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t 
   for (int32_t v = threadIdx.x; v < n; v += blockDim.x)
     if (key_step(key, (uint64_t)(uint32_t)v) == s_kmin) atomicMin(&s_src, v);
   __syncthreads();
-  // hop distances from a, then from b (farthest from a, smallest id), by
-  // parallel relaxation d(v) = min(d(v), d(u) + 1) to the fixpoint (= BFS)
+  // hop distances from a, then from b (farthest from a, smallest id), level by
+  // level: the nodes of hop `it` mark their unmarked neighbours with it + 1, so
+  // a row is read once per pass (every marker of a node writes the same value)
   for (int pass = 0; pass < 2 && n > 0; ++pass) {
     volatile int32_t *d = pass == 0 ? d1 : d2;
     int32_t src = s_src;
@@ -89,20 +143,20 @@ __device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t 
       s_D[pass] = 0;
     }
     __syncthreads();
-    // at most n + 1 sweeps: every sweep that changes something lowers a distance
-    for (int32_t it = 0; it <= n; ++it) {
-      for (int32_t v = threadIdx.x; v < n; v += blockDim.x) {
-        int32_t dv = d[v], best = dv;
-        for (XT e = G.xadj[v]; e < G.xadj[v + 1]; ++e) {
-          int32_t du = d[G.adj[e] - G.abase];
-          if (du != INT32_MAX && du + 1 < best) best = du + 1;
-        }
-        if (best < dv) {
-          d[v] = best;
-          s_chg[it % 3] = 1;
-        }
+    for (int32_t it = 0; it < n; ++it) {
+      bool any = false;
+      for (int32_t v0 = warp0; v0 < n; v0 += blockDim.x) {
+        const int32_t v = v0 + lane;
+        mp_rows(G, v < n && d[v] == it, v, [&](XT e) {
+          const int32_t u = G.adj[e] - G.abase;
+          if (d[u] == INT32_MAX) {
+            d[u] = it + 1;
+            any = true;
+          }
+        });
       }
-      // flag (it + 1) % 3 was last read two sweeps ago: safe to clear now
+      if (any) s_chg[it % 3] = 1;
+      // flag (it + 1) % 3 was last read two levels ago: safe to clear now
       if (threadIdx.x == 0) s_chg[(it + 1) % 3] = 0;
       __syncthreads();
       if (!s_chg[it % 3]) break;
@@ -121,10 +175,9 @@ __device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t 
     }
   }
   int32_t s_D1 = s_D[0], s_D2 = s_D[1];
-  double meanc = s_c / (n > 0 ? n : 1), meanw = s_w / (n > 0 ? n : 1);
+  double meanc = (double)s_c / (n > 0 ? n : 1), meanw = (double)s_w / (n > 0 ? n : 1);
   for (int32_t v = threadIdx.x; v < n; v += blockDim.x) {
-    double wd = 0;
-    for (XT e = G.xadj[v]; e < G.xadj[v + 1]; ++e) wd += G.ew ? G.ew[e] : 1;
+    const double wd = (double)*reinterpret_cast<const int64_t *>(X + (int64_t)v * MF + 6);
     double deg = (double)(G.xadj[v + 1] - G.xadj[v]);
     uint64_t h = key_step(key, (uint64_t)(uint32_t)v);
     float *x = X + (int64_t)v * MF;
