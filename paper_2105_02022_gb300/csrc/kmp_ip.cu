@@ -29,20 +29,27 @@ namespace kmp {
 
 constexpr int IPT = 256;
 constexpr int IPW = IPT / 32;
-constexpr int IP_WTAB = 512;       // per-warp shared table: degree <= 256
 constexpr int IP_MAXL = 63;
 constexpr int32_t IP_MAX_N = 65535;
-// dynamic shared memory per bipartitioner CTA, at most (words): 184 KB, which
-// with the kernel's 40 KB of static shared memory stays within the 227 KB a
-// CTA may use
-constexpr int32_t IP_DYN_MAX_WORDS = 46000;
-constexpr int32_t IP_DYN_SHARED_WORDS = 18000;  // 72 KB: two CTAs per SM
+constexpr uint16_t IP_NONE = 0xFFFF;  // no node: ids are below IP_MAX_N
+// Dynamic shared memory of a bipartitioner CTA: a hash table per warp (wtab slots
+// of key and weight: rows up to wtab / 2 entries) and behind them the working
+// state of the item's phases (dyn_words).  An item's time is latency, so what
+// counts is how many an SM works on.  A round with more items than SMs: 256
+// slots and 12,800 words, 67 KB in all, three CTAs an SM (with 80 registers a
+// thread).  That holds items of up to 2300 nodes; larger ones work in their
+// scratch, which is still faster than two CTAs an SM that hold 3350 nodes (4096
+// items of 200..4000 nodes: 32.4 against 38.2 ms).  Otherwise the items are on
+// the critical path: one CTA an SM with what it offers.
+struct IPShape {
+  int32_t wtab, dyn_words;
+};
+constexpr IPShape IP_SHAPE3{256, 12800}, IP_SHAPE1{512, 45000};
+constexpr size_t ip_smem(IPShape s) { return 4 * (size_t)(2 * IPW * s.wtab + s.dyn_words); }
 
 struct ItemDesc {
   int64_t vbase;  // first member position
   int64_t ebase;  // first induced edge
-  int64_t sbase;  // scratch region (int32 units)
-  int64_t ssize;
   uint64_t key;
   int32_t n, m;
   int32_t t0, t1, L0, L1;
@@ -56,11 +63,12 @@ struct IPArgs {
   int32_t *queue;         // work counter
   int32_t *oom;           // set when a scratch region was too small
   const int64_t *gx;      // induced CSR offsets over all members (n+1)
-  const int32_t *sadj;    // local neighbour ids
-  const int32_t *sew;
+  const uint16_t *sadj;   // local neighbour ids (an item has at most IP_MAX_N nodes)
+  const int32_t *sew;     // null: unit weights
   const int32_t *svw;
   int32_t *side_out;      // per member position
-  int32_t *scratch;
+  int32_t *scratch;       // a region of slot words per CTA, reused by its items
+  int64_t slot;
   // configuration
   int32_t S, ip_C, ip_lp_rounds, rep_random, rep_bfs, rep_ggg, fm_passes, fm_stop;
   int32_t conv_num, conv_den;
@@ -70,14 +78,22 @@ struct IPArgs {
   int32_t adaptive;  // adaptive portfolio (plain mode only)
   int32_t learned_item;  // learned item mode (W set): start on the item graph, FM there
   SampleSink sink;  // counters null: no recording
-  int32_t dyn_words;  // dynamic shared memory per CTA (int32 words) for FM and portfolio state
+  int32_t wtab;       // slots of a warp's shared hash table
+  int32_t dyn_words;  // words of the phases' working state in shared memory
 };
 
+// A level of an item.  Neighbour ids take 16 bits and unit weights are not
+// stored, so the 2048-node items of a degree-16 mesh take 64 KB each instead of
+// 250: what the resident items read again and again stays in L2.
 struct LG {
   int32_t n, m;
-  int32_t *xadj, *adj, *ew, *vw;
+  int32_t *xadj;
+  uint16_t *adj;
+  int32_t *ew;  // null: unit weights
+  int32_t *vw;
   int32_t maxdeg, maxc;
 };
+__device__ __forceinline__ int32_t lg_w(const LG &g, int32_t q) { return g.ew ? g.ew[q] : 1; }
 
 struct Bump {
   int32_t *base;
@@ -228,23 +244,23 @@ __device__ __forceinline__ int32_t pow2_at_least(int32_t x) {
 
 // ------------------------------------------------------ item clustering
 // rating of node u by one warp; returns (via lane 0) proposal target or -1
-__device__ void item_rate(const LG &g, int32_t u, const int32_t *label, const int32_t *wt, int32_t U,
-                          uint32_t rk_hi, int32_t *skeys, int32_t *svals, int32_t *gkeys,
-                          int32_t *gvals, int32_t *out_t, int32_t *out_g) {
+__device__ void item_rate(const LG &g, int32_t u, const uint16_t *label, const int32_t *wt, int32_t U,
+                          uint32_t rk_hi, uint32_t wtab, int32_t *skeys, int32_t *svals, int32_t *gkeys,
+                          int32_t *gvals, uint16_t *out_t, int32_t *out_g) {
   int lane = threadIdx.x & 31;
   int32_t b = g.xadj[u], e = g.xadj[u + 1], deg = e - b;
   uint32_t cap = 32;
   while ((int64_t)cap < 2ll * deg) cap <<= 1;
   uint32_t mask = cap - 1;
   // shared-memory table unless this node's table does not fit there
-  int32_t *keys = cap <= (uint32_t)IP_WTAB ? skeys : gkeys;
-  int32_t *vals = cap <= (uint32_t)IP_WTAB ? svals : gvals;
+  int32_t *keys = cap <= wtab ? skeys : gkeys;
+  int32_t *vals = cap <= wtab ? svals : gvals;
   for (uint32_t i = lane; i < cap; i += 32) {
     keys[i] = HT_EMPTY;
     vals[i] = 0;
   }
   __syncwarp();
-  for (int32_t q = b + lane; q < e; q += 32) ht_add(keys, vals, mask, label[g.adj[q]], g.ew[q]);
+  for (int32_t q = b + lane; q < e; q += 32) ht_add(keys, vals, mask, label[g.adj[q]], lg_w(g, q));
   __syncwarp();
   int32_t own = label[u], cu = g.vw[u];
   int32_t rown = ht_get(keys, vals, mask, own);
@@ -263,10 +279,10 @@ __device__ void item_rate(const LG &g, int32_t u, const int32_t *label, const in
   if (lane == 0) {
     int32_t rc = (int32_t)(mc >> 32);
     if (mc != 0 && rc > rown) {
-      *out_t = lc;
+      *out_t = (uint16_t)lc;
       *out_g = rc - rown;
     } else {
-      *out_t = -1;
+      *out_t = IP_NONE;
     }
   }
   __syncwarp();
@@ -276,38 +292,35 @@ __device__ void item_rate(const LG &g, int32_t u, const int32_t *label, const in
 // neighbour per lane; u < 0: no node): lanes of a group holding the same
 // label form a peer set whose weight sum is that label's rating.  Same
 // decision as item_rate.
-// loads of one group node: neighbour label and edge weight of this lane,
-// own label and node weight (u < 0: no node)
+// inputs of one group node: neighbour label and edge weight of this lane, own
+// label and node weight (u < 0: no node)
 struct GroupIn {
   int32_t l, x, own, cu;
 };
-template <int G>
-__device__ __forceinline__ GroupIn item_group_load(const LG &g, int32_t u, const int32_t *label) {
-  const int gl = (threadIdx.x & 31) & (G - 1);
-  GroupIn r{-1, 0, -1, 0};
-  if (u >= 0) {
-    int32_t b = g.xadj[u], deg = g.xadj[u + 1] - b;
-    r.own = label[u];
-    r.cu = g.vw[u];
-    if (gl < deg) {
-      r.l = label[g.adj[b + gl]];
-      r.x = g.ew[b + gl];
-    }
-  }
-  return r;
-}
 
 // rating of 32 / G nodes by one warp, G lanes per node (degree <= G, one
 // neighbour per lane): lanes of a group holding the same label form a peer
 // set whose weight sum is that label's rating.  Same decision as item_rate.
 template <int G>
-__device__ __forceinline__ void item_group_rate(const GroupIn &in, int32_t u, const int32_t *wt, int32_t U,
-                                                uint32_t rk_hi, int32_t *pt, int32_t *pg) {
+__device__ __forceinline__ void item_group_rate(const GroupIn &in, bool unit, int32_t u, const int32_t *wt, int32_t U,
+                                                uint32_t rk_hi, uint16_t *pt, int32_t *pg) {
   const int lane = threadIdx.x & 31, gl = lane & (G - 1);
   const unsigned gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int32_t l = in.l;
-  unsigned peers = __match_any_sync(0xFFFFFFFFu, ((uint64_t)(uint32_t)(lane / G) << 32) | (uint32_t)l);
-  int32_t r = __reduce_add_sync(peers, in.x);
+  // as k_rate's groups: the set's size with unit weights, else its peers' weights
+  const unsigned peers = __match_any_sync(0xFFFFFFFFu, l) & gmask;
+  int32_t r;
+  if (unit) {
+    r = __popc(peers);
+  } else {
+    r = in.x;
+    unsigned rest = l < 0 ? 0 : peers & ~(1u << lane);
+    while (__any_sync(0xFFFFFFFFu, rest != 0)) {
+      const int32_t t = __shfl_sync(0xFFFFFFFFu, in.x, rest ? __ffs(rest) - 1 : lane);
+      if (rest) r += t;
+      rest &= rest - 1;
+    }
+  }
   unsigned bown = __ballot_sync(0xFFFFFFFFu, l >= 0 && l == in.own) & gmask;
   int32_t rown = __shfl_sync(0xFFFFFFFFu, r, bown ? __ffs(bown) - 1 : lane);
   if (!bown) rown = 0;
@@ -319,26 +332,34 @@ __device__ __forceinline__ void item_group_rate(const GroupIn &in, int32_t u, co
   if (gl == 0 && u >= 0) {
     int32_t rc = (int32_t)(mc >> 32);
     if (mc != 0 && rc > rown) {
-      pt[u] = lc;
+      pt[u] = (uint16_t)lc;
       pg[u] = rc - rown;
     } else {
-      pt[u] = -1;
+      pt[u] = IP_NONE;
     }
   }
 }
 
 // the nodes sl[lo..hi) rated 32 / G per warp step
 template <int G>
-__device__ __forceinline__ void item_rate_groups(const LG &g, const int32_t *sl, int32_t lo, int32_t hi,
-                                                 const int32_t *label, const int32_t *wt, int32_t U,
-                                                 uint32_t rk_hi, int32_t *pt, int32_t *pg) {
+__device__ __forceinline__ void item_rate_groups(const LG &g, const uint16_t *sl, int32_t lo, int32_t hi,
+                                                 const uint16_t *label, const int32_t *wt, int32_t U,
+                                                 uint32_t rk_hi, uint16_t *pt, int32_t *pg) {
   constexpr int per = 32 / G;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, gl = lane & (G - 1);
   for (int32_t i0 = lo + per * w; i0 < hi; i0 += per * IPW) {
-    int32_t i = i0 + lane / G;
-    int32_t u = i < hi ? sl[i] : -1;
-    GroupIn a = item_group_load<G>(g, u, label);
-    item_group_rate<G>(a, u, wt, U, rk_hi, pt, pg);
+    const int32_t i = i0 + lane / G, u = i < hi ? sl[i] : -1;
+    GroupIn a{-1, 0, -1, 0};
+    if (u >= 0) {
+      const int32_t b = g.xadj[u], deg = g.xadj[u + 1] - b;
+      a.own = label[u];
+      a.cu = g.vw[u];
+      if (gl < deg) {
+        a.l = label[g.adj[b + gl]];
+        a.x = lg_w(g, b + gl);
+      }
+    }
+    item_group_rate<G>(a, g.ew == nullptr, u, wt, U, rk_hi, pt, pg);
   }
 }
 
@@ -386,54 +407,49 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
   // to `label` at the end either way.  The sort space of contested proposals
   // sits in shared memory behind them when a sub-round's proposals fit
   // there, else in the scratch (pl_g, always reserved).
-  int32_t *lab, *wt, *pt, *pg, *sl, *fl, *tsum;
-  uint8_t *act, *act2;  // active flags
+  int32_t *wt, *pg, *tsum;  // tsum: proposed weight per target (kept zero between uses)
+  uint16_t *lab, *pt, *sl, *fl;  // sl: the round's nodes by sub-round; fl: accepted
+                                 // proposals of uncontested targets
+  uint8_t *act, *act2;           // active flags
   uint64_t *pl_s = nullptr;
   int32_t pl_cap = 0;   // entries of pl_s
   uint64_t *pl_g = reinterpret_cast<uint64_t *>(B.take(2ll * P));
-  const int64_t flag_words = (n + 3) / 4;
-  const bool fast = 7ll * n + 2 * flag_words + 2 + 128 <= dyn_words;
-  if (fast) {
-    int32_t *q = dyn;
-    lab = q; q += n;
+  const int32_t id_words = (n + 1) / 2, flag_words = (n + 3) / 4;
+  const int64_t lp_words = 3ll * n + 4ll * id_words + 2ll * flag_words;
+  const bool fast = lp_words + 2 + 128 <= dyn_words;
+  {
+    int32_t *q = fast ? dyn : B.take(lp_words);
     wt = q; q += n;
-    pt = q; q += n;
     pg = q; q += n;
-    sl = q; q += n;
-    fl = q; q += n;
     tsum = q; q += n;
+    lab = reinterpret_cast<uint16_t *>(q); q += id_words;
+    pt = reinterpret_cast<uint16_t *>(q); q += id_words;
+    sl = reinterpret_cast<uint16_t *>(q); q += id_words;
+    fl = reinterpret_cast<uint16_t *>(q); q += id_words;
     act = reinterpret_cast<uint8_t *>(q); q += flag_words;
     act2 = reinterpret_cast<uint8_t *>(q); q += flag_words;
-    q += (q - dyn) & 1;  // 8-byte alignment
-    pl_s = reinterpret_cast<uint64_t *>(q);
-    pl_cap = (int32_t)((dyn_words - (q - dyn)) / 2);
-  } else {
-    lab = label;
-    wt = B.take(n);
-    act = reinterpret_cast<uint8_t *>(B.take(flag_words));
-    act2 = reinterpret_cast<uint8_t *>(B.take(flag_words));
-    pt = B.take(n);
-    pg = B.take(n);
-    sl = B.take(n);    // the round's nodes by sub-round
-    fl = B.take(n);    // accepted proposals of uncontested targets
-    tsum = B.take(n);  // proposed weight per target (kept zero between uses)
+    if (fast) {
+      q += (q - dyn) & 1;  // 8-byte alignment
+      pl_s = reinterpret_cast<uint64_t *>(q);
+      pl_cap = (int32_t)((dyn_words - (q - dyn)) / 2);
+    }
   }
   int32_t *gtab = nullptr;
   uint32_t gcap = 0;
-  if (g.maxdeg > IP_WTAB / 2) {
+  if (g.maxdeg > A.wtab / 2) {
     gcap = 32;
     while ((int64_t)gcap < 2ll * g.maxdeg) gcap <<= 1;
     gtab = B.take(2ll * gcap * IPW);
   }
   if (B.oom) return -1;
   for (int32_t v = threadIdx.x; v < n; v += IPT) {
-    lab[v] = v;
+    lab[v] = (uint16_t)v;
     wt[v] = g.vw[v];
     act[v] = 1;
     tsum[v] = 0;
   }
   __syncthreads();
-  int32_t *mk = wkeys + w * IP_WTAB, *mv = wvals + w * IP_WTAB;
+  int32_t *mk = wkeys + w * A.wtab, *mv = wvals + w * A.wtab;
   int32_t *gk = nullptr, *gv = nullptr;
   if (gtab) {
     gk = gtab + (int64_t)w * 2 * gcap;
@@ -470,7 +486,7 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
       int32_t d = g.xadj[v + 1] - g.xadj[v];
       if (act[v] && d > 0) {
         int32_t x = 3 * (int32_t)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1)) + item_deg_class(d);
-        sl[s_soff[x] + atomicAdd(&s_fill[x], 1)] = v;
+        sl[s_soff[x] + atomicAdd(&s_fill[x], 1)] = (uint16_t)v;
       }
     }
     __syncthreads();
@@ -485,7 +501,7 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
       item_rate_groups<32>(g, sl, m1, m2, lab, wt, U, rk_hi, pt, pg);
       for (int32_t i = m2 + w; i < hi; i += IPW) {
         int32_t u = sl[i];
-        item_rate(g, u, lab, wt, U, rk_hi, mk, mv, gk, gv, &pt[u], &pg[u]);
+        item_rate(g, u, lab, wt, U, rk_hi, (uint32_t)A.wtab, mk, mv, gk, gv, &pt[u], &pg[u]);
       }
       if (threadIdx.x == 0) {
         s_cnt = 0;
@@ -495,16 +511,16 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
       // proposed weight per target
       for (int32_t i = lo + threadIdx.x; i < hi; i += IPT) {
         int32_t u = sl[i], T = pt[u];
-        if (T >= 0) atomicAdd(&tsum[T], g.vw[u]);
+        if (T != IP_NONE) atomicAdd(&tsum[T], g.vw[u]);
       }
       __syncthreads();
       // a target whose proposals all fit takes them all; only the proposals
       // of contested targets need the (target, gain desc, node) order
       for (int32_t i = lo + threadIdx.x; i < hi; i += IPT) {
         int32_t u = sl[i], T = pt[u];
-        if (T < 0) continue;
+        if (T == IP_NONE) continue;
         if ((int64_t)wt[T] + tsum[T] <= U) {
-          fl[atomicAdd(&s_fast, 1)] = u;
+          fl[atomicAdd(&s_fast, 1)] = (uint16_t)u;
         } else {
           int32_t p = atomicAdd(&s_cnt, 1);
           pl[p] = ((uint64_t)(uint32_t)T << 47) | ((uint64_t)(uint32_t)(0x7FFFFFFF - pg[u]) << 16) |
@@ -514,7 +530,7 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
       __syncthreads();
       for (int32_t i = lo + threadIdx.x; i < hi; i += IPT) {
         int32_t T = pt[sl[i]];
-        if (T >= 0) tsum[T] = 0;  // every reader is past the barrier above
+        if (T != IP_NONE) tsum[T] = 0;  // every reader is past the barrier above
       }
       int32_t np = s_cnt, nf = s_fast;
       if (np > 0) {
@@ -559,30 +575,59 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
           __syncthreads();
         }
       }
-      // apply: one warp per accepted move; lane 0 moves the node, the lanes
-      // mark its neighbours active for the next round
+      // apply: every warp takes its share of the accepted moves, a lane each, and
+      // then walks the moved nodes' rows together, an entry per lane, to mark the
+      // neighbours active for the next round (a warp per move cost the latency of
+      // its row 30 times over: 40,000 cycles in the first sub-rounds of a
+      // 2048-node item)
       int32_t mv_local = 0;
-      for (int32_t i = w; i < nf + np; i += IPW) {
-        int32_t u, T;
-        if (i < nf) {
-          u = fl[i];
-          T = pt[u];
-        } else {
-          uint64_t k = pl[i - nf];
-          if (!(k >> 63)) continue;
-          T = (int32_t)((k >> 47) & 0xFFFF);
-          u = (int32_t)(k & 0xFFFF);
+      const int32_t share = (nf + np + IPW - 1) / IPW;
+      const int32_t mend = min((w + 1) * share, nf + np);
+      for (int32_t i0 = w * share; i0 < mend; i0 += 32) {
+        const int32_t i = i0 + lane;
+        int32_t u = -1, T = 0, deg = 0, beg = 0;
+        if (i < mend) {
+          if (i < nf) {
+            u = fl[i];
+            T = pt[u];
+          } else {
+            const uint64_t k = pl[i - nf];
+            if (k >> 63) {
+              T = (int32_t)((k >> 47) & 0xFFFF);
+              u = (int32_t)(k & 0xFFFF);
+            }
+          }
         }
-        if (lane == 0) {
-          int32_t own = lab[u], c = g.vw[u];
-          lab[u] = T;
+        if (u >= 0) {
+          const int32_t own = lab[u], c = g.vw[u];
+          lab[u] = (uint16_t)T;
           atomicAdd(&wt[T], c);
           atomicSub(&wt[own], c);
           ++mv_local;
+          beg = g.xadj[u];
+          deg = g.xadj[u + 1] - beg;
         }
-        for (int32_t q = g.xadj[u] + lane; q < g.xadj[u + 1]; q += 32) act2[g.adj[q]] = 1;
+        int32_t inc = deg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+          if (lane >= o) inc += t;
+        }
+        const int32_t tot = __shfl_sync(0xFFFFFFFFu, inc, 31), shift = beg - (inc - deg);
+        for (int32_t e0 = 0; e0 < tot; e0 += 32) {
+          const int32_t e = e0 + lane;
+          int32_t j = 0;  // moves whose rows end at or before entry e
+#pragma unroll
+          for (int st = 16; st > 0; st >>= 1) {
+            const int32_t t = __shfl_sync(0xFFFFFFFFu, inc, j + st - 1);
+            if (t <= e) j += st;
+          }
+          const int32_t q = __shfl_sync(0xFFFFFFFFu, shift, j & 31) + e;
+          if (e < tot) act2[g.adj[q]] = 1;
+        }
       }
-      if (mv_local) atomicAdd(&s_moved, mv_local);
+      mv_local = warp_sum32(mv_local);
+      if (lane == 0 && mv_local) atomicAdd(&s_moved, mv_local);
       __syncthreads();
     }
     int32_t moved = s_moved;
@@ -597,25 +642,25 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
   for (int32_t v = threadIdx.x; v < n; v += IPT) iw[v] = (g.xadj[v + 1] == g.xadj[v]) ? g.vw[v] : 0;
   __syncthreads();
   block_scan_excl<int32_t>(iw, iw, n);
-  int32_t *first = sl;
+  int32_t *first = tsum;
   for (int32_t v = threadIdx.x; v < n; v += IPT) first[v] = INT32_MAX;
   __syncthreads();
   for (int32_t v = threadIdx.x; v < n; v += IPT) {
     if (g.xadj[v + 1] != g.xadj[v]) continue;
     int64_t P0 = iw[v], c = g.vw[v];
     int64_t q = P0 / U, qe = (P0 + c - 1) / U;
-    if (q == qe) atomicMin(&first[q], lab[v]);
+    if (q == qe) atomicMin(&first[q], (int32_t)lab[v]);
   }
   __syncthreads();
   for (int32_t v = threadIdx.x; v < n; v += IPT) {
     if (g.xadj[v + 1] != g.xadj[v]) continue;
     int64_t P0 = iw[v], c = g.vw[v];
     int64_t q = P0 / U, qe = (P0 + c - 1) / U;
-    if (q == qe) lab[v] = first[q];
+    if (q == qe) lab[v] = (uint16_t)first[q];
   }
   __syncthreads();
   // count clusters
-  int32_t *used = pt;
+  uint16_t *used = pt;
   for (int32_t v = threadIdx.x; v < n; v += IPT) used[v] = 0;
   __syncthreads();
   for (int32_t v = threadIdx.x; v < n; v += IPT) used[lab[v]] = 1;
@@ -623,16 +668,14 @@ __device__ int32_t item_cluster(const IPArgs &A, const LG &g, int32_t U, uint64_
   int64_t c = 0;
   for (int32_t v = threadIdx.x; v < n; v += IPT) c += used[v];
   int32_t nc = (int32_t)block_sum64(c);
-  if (fast) {
-    for (int32_t v = threadIdx.x; v < n; v += IPT) label[v] = lab[v];
-    __syncthreads();
-  }
+  for (int32_t v = threadIdx.x; v < n; v += IPT) label[v] = lab[v];
+  __syncthreads();
   B.top = mark;
   return nc;
 }
 
 // contraction of one item level; fills *out (arrays allocated from B)
-__device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, LG *out, Bump &B,
+__device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, LG *out, Bump &B, int32_t wtab,
                               int32_t *wkeys, int32_t *wvals) {
   int32_t n = g.n;
   int32_t *cid = B.take(n + 1);
@@ -651,13 +694,14 @@ __device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, L
   for (int32_t v = threadIdx.x; v < n; v += IPT)
     for (int32_t q = g.xadj[v]; q < g.xadj[v + 1]; ++q) cnt += (map[v] != map[g.adj[q]]);
   int32_t np = (int32_t)block_sum64(cnt);
-  int32_t *cadj = B.take(np);
+  uint16_t *cadj = reinterpret_cast<uint16_t *>(B.take((np + 1) / 2));
   int32_t *cew = B.take(np);
   int64_t mark = B.top;
   // members grouped by coarse node; members' total degree per coarse node
   int32_t *moff = B.take(nc + 1), *mcur = B.take(nc), *members = B.take(n);
   int32_t *ub = B.take(nc + 1), *toff = B.take(nc + 1), *rowlen = B.take(nc + 1);
-  int32_t *tadj = B.take(g.m > 0 ? g.m : 1), *tw = B.take(g.m > 0 ? g.m : 1);
+  uint16_t *tadj = reinterpret_cast<uint16_t *>(B.take((g.m + 2) / 2));
+  int32_t *tw = B.take(g.m > 0 ? g.m : 1);
   if (B.oom) return;
   for (int32_t x = threadIdx.x; x <= nc; x += IPT) {
     if (x < nc) {
@@ -689,7 +733,7 @@ __device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, L
   int32_t gcap = 32;
   while (gcap < 2 * dmax) gcap <<= 1;
   int32_t lcap = pow2_at_least(dmax > 1 ? dmax : 2);
-  int32_t *gtab = gcap > IP_WTAB ? B.take(2ll * gcap * IPW) : nullptr;
+  int32_t *gtab = gcap > wtab ? B.take(2ll * gcap * IPW) : nullptr;
   uint64_t *lbuf = reinterpret_cast<uint64_t *>(B.take(2ll * lcap * IPW));
   __syncthreads();
   if (B.oom) return;
@@ -700,8 +744,8 @@ __device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, L
     int32_t d = ub[x] < nc ? ub[x] : nc;
     uint32_t cap = 32;
     while ((int32_t)cap < 2 * d) cap <<= 1;
-    int32_t *K = cap <= (uint32_t)IP_WTAB ? wkeys + w * IP_WTAB : gtab + (int64_t)w * 2 * gcap;
-    int32_t *V = cap <= (uint32_t)IP_WTAB ? wvals + w * IP_WTAB : K + gcap;
+    int32_t *K = cap <= (uint32_t)wtab ? wkeys + w * wtab : gtab + (int64_t)w * 2 * gcap;
+    int32_t *V = cap <= (uint32_t)wtab ? wvals + w * wtab : K + gcap;
     for (uint32_t i = lane; i < cap; i += 32) {
       K[i] = HT_EMPTY;
       V[i] = 0;
@@ -736,7 +780,7 @@ __device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, L
         if (e < tot) {
           int32_t q = bj + (e - ej);
           int32_t y = map[g.adj[q]];
-          if (y != x) ht_add(K, V, cap - 1, y, g.ew[q]);
+          if (y != x) ht_add(K, V, cap - 1, y, lg_w(g, q));
         }
       }
     }
@@ -754,7 +798,7 @@ __device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, L
     __syncwarp();
     warp_bitonic_u64(L, P);
     for (int32_t i = lane; i < c; i += 32) {
-      tadj[toff[x] + i] = (int32_t)(L[i] >> 32);
+      tadj[toff[x] + i] = (uint16_t)(L[i] >> 32);
       tw[toff[x] + i] = (int32_t)(uint32_t)L[i];
     }
     if (lane == 0) rowlen[x] = c;
@@ -781,16 +825,58 @@ __device__ void item_contract(const LG &g, const int32_t *label, int32_t *map, L
 }
 
 // ------------------------------------------------------------ warp FM
-// FM state: gains, locks, the move log, and per side the selection key of
-// every node of that side that may still move (0 otherwise), so that finding
-// the top of a side is a branch-free max over one array
-struct FMBuf {
-  int32_t *gain, *locked, *moves;
-  uint64_t *key0, *key1;
+// A pass of 2-way FM is a chain of steps on one warp, each a scan for the tops
+// of both sides and an update of one row's gains, so its time is the latency of
+// what a step does in turn.  Its state is small enough for shared memory at
+// every level that occurs in large numbers (6.1 bytes a node, 14.1 with row
+// offsets and node weights): a 32-bit key a node; a bit a node for its side at
+// the start of the pass (a move locks, so sides change once, at the end of the
+// pass, by the kept moves); the move log in 16 bits.
+//
+// The key holds gain and id: ((gain + bias) << idbits | largest id - id), as
+// such on side 0, negated on side 1, 0 once locked (the next pass computes a
+// locked node's gain anew).  So the tops of both sides, gain descending and id
+// ascending, are the largest and the smallest key; and a move changes every
+// unlocked neighbour's key by the same signed amount whichever side it is on.
+// Where id and the largest weighted degree do not fit 31 bits together
+// (idbits < 0) the key is the plain gain, FM_LOCKED once locked, and the scan
+// reads the sides.
+constexpr int32_t FM_LOCKED = INT32_MIN;  // below every gain: those fit 31 bits and a sign
+struct FMState {
+  int32_t *key;     // fm_pad(n) words, 16-byte aligned; locked from n on
+  uint32_t *bits;   // fm_pad(n) / 32 words: sides
+  uint16_t *moves;  // n node ids (IP_MAX_N)
+  // the level's graph; row offsets, node weights and entries in shared memory
+  // where they fit
+  const int32_t *xadj, *vw;
+  const uint16_t *adj;
+  const int32_t *ew;  // null: unit weights
+  // word offsets of the state, of the row offsets (the node weights behind them)
+  // and of the edge weights (neighbour ids behind them) in the CTA's dynamic
+  // shared memory; -1: not there
+  int32_t off, goff, eoff;
 };
+__host__ __device__ __forceinline__ int32_t fm_pad(int32_t n) { return (n + 127) & ~127; }
+__host__ __device__ __forceinline__ int64_t fm_words(int32_t n) { return (int64_t)fm_pad(n) / 32 * 49; }
+__device__ __forceinline__ FMState fm_state(int32_t *p, const LG &g) {
+  const int32_t np = fm_pad(g.n);
+  uint32_t *bits = reinterpret_cast<uint32_t *>(p + np);
+  return FMState{p, bits, reinterpret_cast<uint16_t *>(bits + np / 32), g.xadj, g.vw, g.adj, g.ew, -1, -1, -1};
+}
+__device__ __forceinline__ int32_t *align16(int32_t *p) {
+  return reinterpret_cast<int32_t *>((reinterpret_cast<uintptr_t>(p) + 15) & ~(uintptr_t)15);
+}
+__device__ __forceinline__ int32_t fm_side(const uint32_t *bits, int32_t v) { return (bits[v >> 5] >> (v & 31)) & 1; }
 
-__device__ __forceinline__ uint64_t fm_key(int32_t gain, int32_t v) {
-  return ((uint64_t)((uint32_t)gain ^ 0x80000000u) << 32) | (0xFFFFFFFFu - (uint32_t)v);
+// bits of a node id in the key: n <= 2^idbits, and gains within +-maxwd leave
+// 1 <= (gain + bias) < 2^(31 - idbits) with bias = maxwd + 1; -1 if they do not
+__device__ __forceinline__ int32_t fm_idbits(int32_t n, int32_t maxwd) {
+  const int32_t b = 32 - __clz(n > 1 ? n - 1 : 1);
+  return 2ll * maxwd + 2 < (1ll << (31 - b)) ? b : -1;
+}
+__device__ __forceinline__ int32_t fm_key(int32_t gain, int32_t v, int32_t side, int32_t idbits, int32_t bias) {
+  const int32_t k = ((gain + bias) << idbits) | ((1 << idbits) - 1 - v);
+  return side ? -k : k;
 }
 
 __device__ __forceinline__ bool fm_less(int32_t ia, int64_t oa, int64_t ca, int32_t ib, int64_t ob,
@@ -800,204 +886,368 @@ __device__ __forceinline__ bool fm_less(int32_t ia, int64_t oa, int64_t ca, int3
   return ca < cb;
 }
 
-// 2-way FM by one warp (same decisions as the oracle); returns the final cut
-// the moves of one FM pass by one warp, from gains and locks already set:
-// repeatedly the better feasible top of the two sides (gain desc, id asc),
-// until no unlocked node is left or fm_stop moves bring no new best; then
-// the pass is rolled back to its best prefix.  Returns the kept moves (0: the
-// pass found nothing better) and updates cut.
-__device__ int32_t fm_pass_moves(const IPArgs &A, const LG &g, int32_t *side, int64_t L0, int64_t L1,
-                                 FMBuf fb, int64_t W0, int64_t W1, int64_t &cut) {
-  int lane = threadIdx.x & 31;
-  int32_t n = g.n;
-  auto mk = [&](int32_t &inf, int64_t &ov) {
-    int64_t o0 = W0 - L0, o1 = W1 - L1;
-    int64_t o = o0 > o1 ? o0 : o1;
-    inf = o > 0;
-    ov = inf ? o : 0;
-  };
-  int32_t binf;
-  int64_t bov;
-  mk(binf, bov);
-  int64_t bcut = cut;
+// The moves of one FM pass by one warp, from keys already set: repeatedly the
+// better feasible top of the two sides (gain desc, id asc), until no unlocked
+// node is left or fm_stop moves bring no new best (overload, then cut); then
+// the pass keeps its best prefix.  Returns the kept moves (0: the pass found
+// nothing better) and updates the sides, the side weights and the cut.
+//
+// One warp on its own issues a dependent instruction every few cycles, so a
+// step costs what its instructions count: the shared arrays are addressed as
+// offsets into the CTA's shared memory (32-bit addresses; GRAPH as in FMState),
+// the sums are 32-bit (caps clamped to the total weight, which is below 2^31),
+// the room left on each side stands for both weights, and only the better
+// side's top is looked up unless it does not fit.
+// Measured a step in place: 780 cycles with all of a level of up to 256 nodes in
+// shared memory (about 1900 with 64-bit selection keys reduced by shuffles), 2200
+// for 2048 nodes with the entries in L2 (3800).
+template <int GRAPH>
+__device__ __forceinline__ int32_t fm_pass_packed(int32_t fm_stop, int32_t n, const FMState F, int32_t idbits,
+                                                  int32_t bias, int32_t L0, int32_t L1, int32_t &W0, int32_t &W1,
+                                                  int32_t &cut) {
+  extern __shared__ __align__(16) int32_t ipdyn[];
+  constexpr unsigned ALL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  const int32_t np = fm_pad(n), idmask = (1 << idbits) - 1, total = W0 + W1;
+  int32_t *const key = GRAPH ? ipdyn + F.off : F.key;
+  uint32_t *const bits = GRAPH ? reinterpret_cast<uint32_t *>(ipdyn + F.off + np) : F.bits;
+  uint16_t *const moves = GRAPH ? reinterpret_cast<uint16_t *>(ipdyn + F.off + np + np / 32) : F.moves;
+  const int32_t *const xadj = GRAPH ? ipdyn + F.goff : F.xadj;
+  const int32_t *const vw = GRAPH ? ipdyn + F.goff + n + 1 : F.vw;
+  const bool unit = F.ew == nullptr;
+  const int32_t *const ew = GRAPH == 2 ? ipdyn + F.eoff : F.ew;
+  const uint16_t *const adj =
+      GRAPH == 2 ? reinterpret_cast<const uint16_t *>(ipdyn + F.eoff + (unit ? 0 : xadj[n])) : F.adj;
+  int32_t r0 = min(L0, total) - W0, r1 = min(L1, total) - W1;  // room left
+  int32_t c = cut, br0 = r0, bcut = c, bmin = min(min(r0, r1), 0);
   int32_t best_step = 0, nsteps = 0;
   for (;;) {
-    uint64_t t0 = 0, t1 = 0;  // (gain biased, ~id): larger is better; 0 = none
+    const int4 k0 = *reinterpret_cast<const int4 *>(key + 4 * lane);
+    int32_t hi = max(max(max(k0.x, k0.y), max(k0.z, k0.w)), 0);
+    int32_t lo = min(min(min(k0.x, k0.y), min(k0.z, k0.w)), 0);
 #pragma unroll 4
-    for (int32_t v = lane; v < n; v += 32) {
-      uint64_t a = fb.key0[v], b = fb.key1[v];
-      t0 = a > t0 ? a : t0;
-      t1 = b > t1 ? b : t1;
+    for (int32_t v = 4 * lane + 128; v < np; v += 128) {
+      const int4 k = *reinterpret_cast<const int4 *>(key + v);
+      hi = max(hi, max(max(k.x, k.y), max(k.z, k.w)));
+      lo = min(lo, min(min(k.x, k.y), min(k.z, k.w)));
     }
-    t0 = group_max64<32>(t0);
-    t1 = group_max64<32>(t1);
-    if (t0 == 0 && t1 == 0) break;
-    int32_t v0 = t0 ? (int32_t)(0xFFFFFFFFu - (uint32_t)t0) : -1;
-    int32_t v1 = t1 ? (int32_t)(0xFFFFFFFFu - (uint32_t)t1) : -1;
-    // both candidates' weights and row bounds in one round of loads
-    int32_t c0 = 0, c1 = 0, b0 = 0, e0 = 0, b1 = 0, e1 = 0;
-    if (v0 >= 0) {
-      c0 = g.vw[v0];
-      b0 = g.xadj[v0];
-      e0 = g.xadj[v0 + 1];
-    }
-    if (v1 >= 0) {
-      c1 = g.vw[v1];
-      b1 = g.xadj[v1];
-      e1 = g.xadj[v1 + 1];
-    }
-    bool f0 = v0 >= 0 && W1 + c0 <= L1;
-    bool f1 = v1 >= 0 && W0 + c1 <= L0;
-    int32_t v;
-    if (f0 && f1) v = (t0 > t1) ? v0 : v1;
-    else if (f0) v = v0;
-    else if (f1) v = v1;
-    else {
-      if (lane == 0) {
-        if (v0 >= 0) {
-          fb.locked[v0] = 1;
-          fb.key0[v0] = 0;
-        }
-        if (v1 >= 0) {
-          fb.locked[v1] = 1;
-          fb.key1[v1] = 0;
-        }
+    const int32_t m0 = __reduce_max_sync(ALL, hi), m1 = -__reduce_min_sync(ALL, lo);
+    if ((m0 | m1) == 0) break;
+    bool from0 = m0 > m1;
+    int32_t m = from0 ? m0 : m1, v = idmask - (m & idmask);
+    int32_t cv = vw[v], qb = xadj[v], qe = xadj[v + 1];
+    if (cv > (from0 ? r1 : r0)) {  // the other side's top
+      const int32_t o = from0 ? m1 : m0, u = idmask - (o & idmask);
+      bool fits = false;
+      if (o) {
+        cv = vw[u];
+        fits = cv <= (from0 ? r0 : r1);
       }
-      __syncwarp();
-      continue;
+      if (!fits) {
+        if (lane == 0) {
+          key[v] = 0;
+          if (o) key[u] = 0;
+        }
+        __syncwarp();
+        continue;
+      }
+      from0 = !from0;
+      m = o;
+      v = u;
+      qb = xadj[v];
+      qe = xadj[v + 1];
     }
-    int32_t from = side[v], to = 1 - from;
-    int32_t gv = fb.gain[v];
-    __syncwarp();
+    const int32_t sg = from0 ? 1 << (idbits + 1) : -(1 << (idbits + 1));
+    for (int32_t q = qb + lane; q < qe; q += 32) {
+      const int32_t x = adj[q], d = (unit ? 1 : ew[q]) * sg, k = key[x];
+      if (k) key[x] = k + d;
+    }
     if (lane == 0) {
-      side[v] = to;
-      fb.locked[v] = 1;
-      fb.key0[v] = 0;
-      fb.key1[v] = 0;
-    }
-    const bool is0 = v == v0;
-    int32_t c = is0 ? c0 : c1;
-    if (from == 0) { W0 -= c; W1 += c; } else { W1 -= c; W0 += c; }
-    cut -= gv;
-    const int32_t qe = is0 ? e0 : e1;
-    for (int32_t q = (is0 ? b0 : b1) + lane; q < qe; q += 32) {
-      int32_t x = g.adj[q];
-      int32_t sx = side[x];
-      int32_t gx = fb.gain[x] + (sx == to ? -2 * g.ew[q] : 2 * g.ew[q]);
-      fb.gain[x] = gx;
-      if (!fb.locked[x]) {
-        if (sx == 0) fb.key0[x] = fm_key(gx, x);
-        else fb.key1[x] = fm_key(gx, x);
-      }
+      key[v] = 0;
+      moves[nsteps] = (uint16_t)v;
     }
     __syncwarp();
-    if (lane == 0) {
-      fb.gain[v] = -gv;
-      fb.moves[nsteps] = v;
-    }
     ++nsteps;
-    __syncwarp();
-    int32_t inf;
-    int64_t ov;
-    mk(inf, ov);
-    if (fm_less(inf, ov, cut, binf, bov, bcut)) {
-      binf = inf;
-      bov = ov;
-      bcut = cut;
+    const int32_t d = from0 ? cv : -cv;
+    r0 += d;
+    r1 -= d;
+    c += bias - (m >> idbits);
+    const int32_t mn = min(min(r0, r1), 0);
+    if (mn > bmin || (mn == bmin && c < bcut)) {
+      bmin = mn;
+      bcut = c;
+      br0 = r0;
       best_step = nsteps;
     }
-    if (nsteps - best_step >= A.fm_stop) break;
+    if (nsteps - best_step >= fm_stop) break;
   }
-  for (int32_t i = best_step + lane; i < nsteps; i += 32) side[fb.moves[i]] ^= 1;
+  for (int32_t i = lane; i < best_step; i += 32) {
+    const int32_t v = moves[i];
+    atomicXor(&bits[v >> 5], 1u << (v & 31));
+  }
   __syncwarp();
+  W0 = min(L0, total) - br0;
+  W1 = total - W0;
   cut = bcut;
   return best_step;
 }
 
-__device__ int64_t warp_fm(const IPArgs &A, const LG &g, int32_t *side, int64_t L0, int64_t L1,
-                           FMBuf fb) {
-  int lane = threadIdx.x & 31;
-  int32_t n = g.n;
-  int64_t cut = 0;
-  for (int32_t v = lane; v < n; v += 32)
-    for (int32_t q = g.xadj[v]; q < g.xadj[v + 1]; ++q)
-      if (side[g.adj[q]] != side[v]) cut += g.ew[q];
-  cut = warp_sum64(cut) / 2;
-  for (int32_t pass = 0; pass < A.fm_passes; ++pass) {
-    int64_t W0 = 0, W1 = 0;
+// the same pass from plain gains, for levels whose keys do not pack
+__device__ __noinline__ int32_t fm_pass_plain(int32_t fm_stop, int32_t n, const FMState F, int64_t L0, int64_t L1,
+                                              int32_t &W0, int32_t &W1, int32_t &cut) {
+  constexpr unsigned ALL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  int64_t w0 = W0, w1 = W1, bw0 = w0;
+  const int64_t total = w0 + w1;
+  auto overload = [&]() -> int64_t { return max(max(w0 - L0, w1 - L1), (int64_t)0); };
+  int64_t bov = overload();
+  int32_t c = cut, bcut = c, best_step = 0, nsteps = 0;
+  for (;;) {
+    int32_t g0 = FM_LOCKED, g1 = FM_LOCKED;
+    uint32_t i0 = ~0u, i1 = ~0u;
     for (int32_t v = lane; v < n; v += 32) {
-      if (side[v] == 0) W0 += g.vw[v];
-      else W1 += g.vw[v];
-      int32_t gsum = 0;
-      for (int32_t q = g.xadj[v]; q < g.xadj[v + 1]; ++q)
-        gsum += (side[g.adj[q]] != side[v]) ? g.ew[q] : -g.ew[q];
-      fb.gain[v] = gsum;
-      fb.locked[v] = 0;
-      fb.key0[v] = side[v] == 0 ? fm_key(gsum, v) : 0;
-      fb.key1[v] = side[v] == 0 ? 0 : fm_key(gsum, v);
+      const int32_t x = F.key[v];
+      if (!fm_side(F.bits, v)) {
+        if (x > g0) {
+          g0 = x;
+          i0 = (uint32_t)v;
+        }
+      } else if (x > g1) {
+        g1 = x;
+        i1 = (uint32_t)v;
+      }
     }
-    W0 = warp_sum64(W0);
-    W1 = warp_sum64(W1);
+    const int32_t m0 = __reduce_max_sync(ALL, g0), m1 = __reduce_max_sync(ALL, g1);
+    if (m0 == FM_LOCKED && m1 == FM_LOCKED) break;
+    const int32_t v0 = (int32_t)__reduce_min_sync(ALL, g0 == m0 ? i0 : ~0u);  // -1: no unlocked node
+    const int32_t v1 = (int32_t)__reduce_min_sync(ALL, g1 == m1 ? i1 : ~0u);
+    const bool f0 = v0 >= 0 && w1 + F.vw[v0] <= L1;
+    const bool f1 = v1 >= 0 && w0 + F.vw[v1] <= L0;
+    if (!f0 && !f1) {
+      if (lane == 0) {
+        if (v0 >= 0) F.key[v0] = FM_LOCKED;
+        if (v1 >= 0) F.key[v1] = FM_LOCKED;
+      }
+      __syncwarp();
+      continue;
+    }
+    const bool from0 = f0 && (!f1 || m0 > m1 || (m0 == m1 && v0 < v1));
+    const int32_t v = from0 ? v0 : v1, to = from0 ? 1 : 0;
+    for (int32_t q = F.xadj[v] + lane; q < F.xadj[v + 1]; q += 32) {
+      const int32_t x = F.adj[q], d = 2 * (F.ew ? F.ew[q] : 1), k = F.key[x];
+      if (k != FM_LOCKED) F.key[x] = fm_side(F.bits, x) == to ? k - d : k + d;
+    }
+    if (lane == 0) {
+      F.key[v] = FM_LOCKED;
+      F.moves[nsteps] = (uint16_t)v;
+    }
     __syncwarp();
-    if (fm_pass_moves(A, g, side, L0, L1, fb, W0, W1, cut) == 0) break;
+    ++nsteps;
+    w0 += from0 ? -(int64_t)F.vw[v] : F.vw[v];
+    w1 = total - w0;
+    c -= from0 ? m0 : m1;
+    const int64_t ov = overload();
+    if (ov < bov || (ov == bov && c < bcut)) {
+      bov = ov;
+      bcut = c;
+      bw0 = w0;
+      best_step = nsteps;
+    }
+    if (nsteps - best_step >= fm_stop) break;
+  }
+  for (int32_t i = lane; i < best_step; i += 32) {
+    const int32_t v = F.moves[i];
+    atomicXor(&F.bits[v >> 5], 1u << (v & 31));
+  }
+  __syncwarp();
+  W0 = (int32_t)bw0;
+  W1 = (int32_t)(total - bw0);
+  cut = bcut;
+  return best_step;
+}
+
+__device__ __forceinline__ int32_t pass_moves(int32_t fm_stop, int32_t n, const FMState F, int32_t idbits,
+                                              int32_t bias, int32_t L0, int32_t L1, int32_t &W0, int32_t &W1,
+                                              int32_t &cut) {
+  if (idbits < 0) return fm_pass_plain(fm_stop, n, F, L0, L1, W0, W1, cut);
+  if (F.eoff >= 0) return fm_pass_packed<2>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+  if (F.off >= 0) return fm_pass_packed<1>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+  return fm_pass_packed<0>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+}
+
+// 2-way FM by one warp (same decisions as the oracle) from the sides in
+// F.bits, which it improves; returns the final cut, W0 and W1 the side weights
+__device__ int32_t warp_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, const FMState F, int32_t &W0,
+                           int32_t &W1) {
+  const int lane = threadIdx.x & 31;
+  int32_t cut = 0, idbits = 0, bias = 0;
+  W0 = W1 = 0;
+  for (int32_t pass = 0; pass < A.fm_passes || pass == 0; ++pass) {
+    int64_t lcut = 0;
+    int32_t maxwd = 0;
+    for (int32_t v = lane; v < n; v += 32) {
+      const int32_t sv = fm_side(F.bits, v);
+      int32_t ext = 0, in = 0;
+      for (int32_t q = F.xadj[v]; q < F.xadj[v + 1]; ++q) {
+        const int32_t wq = F.ew ? F.ew[q] : 1;
+        if (fm_side(F.bits, F.adj[q]) != sv) ext += wq;
+        else in += wq;
+      }
+      const int32_t gs = ext - in;
+      if (pass == 0) {
+        lcut += ext;
+        maxwd = max(maxwd, ext + in);
+        if (sv == 0) W0 += F.vw[v];
+        else W1 += F.vw[v];
+      }
+      F.key[v] = pass == 0 || idbits < 0 ? gs : fm_key(gs, v, sv, idbits, bias);
+    }
+    if (pass == 0) {
+      cut = (int32_t)(warp_sum64(lcut) / 2);
+      W0 = warp_sum32(W0);
+      W1 = warp_sum32(W1);
+      if (A.fm_passes == 0) break;
+      maxwd = __reduce_max_sync(0xFFFFFFFFu, maxwd);
+      idbits = L0 < 0 || L1 < 0 ? -1 : fm_idbits(n, maxwd);
+      bias = maxwd + 1;
+      for (int32_t v = lane; v < fm_pad(n); v += 32) {
+        if (v >= n) F.key[v] = idbits < 0 ? FM_LOCKED : 0;
+        else if (idbits >= 0) F.key[v] = fm_key(F.key[v], v, fm_side(F.bits, v), idbits, bias);
+      }
+    }
+    __syncwarp();
+    if (pass_moves(A.fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut) == 0) break;
   }
   return cut;
 }
 
-// the same FM with the whole CTA: cut, gains and weights of every pass by all
-// warps (a half-warp per node, its 16 lanes over the row), the moves by warp 0
-__device__ int64_t cta_fm(const IPArgs &A, const LG &g, int32_t *side, int64_t L0, int64_t L1, FMBuf fb) {
-  __shared__ int64_t s_cut;
+// the same FM with the whole CTA: cut, keys and weights by all warps (a
+// half-warp per node and four nodes at a time, so the loads of four rows are in
+// flight together), the moves by warp 0
+__device__ void cta_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, const FMState F) {
   __shared__ int32_t s_kept;
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int hl = lane & 15, hf = lane >> 4;
-  int32_t n = g.n;
-  int64_t c = 0;
-  for (int32_t v = 2 * w + hf; v < n; v += 2 * IPW) {
-    int32_t sv = side[v];
-    for (int32_t q = g.xadj[v] + hl; q < g.xadj[v + 1]; q += 16)
-      if (side[g.adj[q]] != sv) c += g.ew[q];
-  }
-  int64_t cut = block_sum64(c) / 2;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int hl = lane & 15, h = 2 * w + (lane >> 4);
+  constexpr int ROWS = 4, STEP = 2 * IPW;  // half-warps
+  int64_t lcut = 0, lw0 = 0, lw1 = 0;
+  int32_t cut = 0, W0 = 0, W1 = 0, idbits = 0, bias = 0;  // warp 0's from the second pass on
   for (int32_t pass = 0; pass < A.fm_passes; ++pass) {
-    int64_t W0 = 0, W1 = 0;
-    for (int32_t v = threadIdx.x; v < n; v += IPT) {
-      if (side[v] == 0) W0 += g.vw[v];
-      else W1 += g.vw[v];
-    }
-    for (int32_t v0 = 2 * w; v0 < n; v0 += 2 * IPW) {
-      const int32_t v = v0 + hf;
-      int32_t sv = 0, gs = 0;
-      if (v < n) {
-        sv = side[v];
-        for (int32_t q = g.xadj[v] + hl; q < g.xadj[v + 1]; q += 16)
-          gs += (side[g.adj[q]] != sv) ? g.ew[q] : -g.ew[q];
+    int32_t maxwd = 0;
+    for (int32_t v0 = h; v0 - h < n; v0 += ROWS * STEP) {
+      int32_t b[ROWS], e[ROWS], x[ROWS], wt[ROWS];
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        const int32_t v = v0 + r * STEP;
+        b[r] = v < n ? F.xadj[v] : 0;
+        e[r] = v < n ? F.xadj[v + 1] : 0;
       }
 #pragma unroll
-      for (int m = 8; m > 0; m >>= 1) gs += __shfl_xor_sync(0xFFFFFFFFu, gs, m);  // within the half
-      if (hl == 0 && v < n) {
-        fb.gain[v] = gs;
-        fb.locked[v] = 0;
-        fb.key0[v] = sv == 0 ? fm_key(gs, v) : 0;
-        fb.key1[v] = sv == 0 ? 0 : fm_key(gs, v);
+      for (int r = 0; r < ROWS; ++r) {
+        x[r] = -1;
+        wt[r] = 0;
+        if (b[r] + hl < e[r]) {
+          x[r] = F.adj[b[r] + hl];
+          wt[r] = F.ew ? F.ew[b[r] + hl] : 1;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) {
+        const int32_t v = v0 + r * STEP;
+        const int32_t sv = v < n ? fm_side(F.bits, v) : 0;
+        int32_t ext = 0, wd = wt[r];
+        if (x[r] >= 0 && fm_side(F.bits, x[r]) != sv) ext = wt[r];
+        for (int32_t q = b[r] + 16 + hl; q < e[r]; q += 16) {
+          const int32_t wq = F.ew ? F.ew[q] : 1;
+          wd += wq;
+          if (fm_side(F.bits, F.adj[q]) != sv) ext += wq;
+        }
+        if (pass == 0) lcut += ext;
+        int32_t gs = 2 * ext - wd;  // external less internal
+#pragma unroll
+        for (int m = 8; m > 0; m >>= 1) gs += __shfl_xor_sync(0xFFFFFFFFu, gs, m);  // within the half
+        if (pass == 0) {
+#pragma unroll
+          for (int m = 8; m > 0; m >>= 1) wd += __shfl_xor_sync(0xFFFFFFFFu, wd, m);
+          maxwd = max(maxwd, wd);
+          if (hl == 0 && v < n) {
+            if (sv == 0) lw0 += F.vw[v];
+            else lw1 += F.vw[v];
+          }
+        }
+        if (hl == 0 && v < n) F.key[v] = pass == 0 || idbits < 0 ? gs : fm_key(gs, v, sv, idbits, bias);
       }
     }
-    W0 = block_sum64(W0);  // its barriers also publish the gains
-    W1 = block_sum64(W1);
-    if (w == 0) {
-      int32_t kept = fm_pass_moves(A, g, side, L0, L1, fb, W0, W1, cut);
-      if (lane == 0) {
-        s_kept = kept;
-        s_cut = cut;
+    if (pass == 0) {
+      cut = (int32_t)(block_sum64(lcut) / 2);
+      W0 = (int32_t)block_sum64(lw0);
+      W1 = (int32_t)block_sum64(lw1);
+      maxwd = block_max32(maxwd);
+      idbits = L0 < 0 || L1 < 0 ? -1 : fm_idbits(n, maxwd);
+      bias = maxwd + 1;
+      for (int32_t v = threadIdx.x; v < fm_pad(n); v += IPT) {
+        if (v >= n) F.key[v] = idbits < 0 ? FM_LOCKED : 0;
+        else if (idbits >= 0) F.key[v] = fm_key(F.key[v], v, fm_side(F.bits, v), idbits, bias);
       }
+    }
+    __syncthreads();  // the keys are complete
+    if (w == 0) {
+      const int32_t kept = pass_moves(A.fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+      if (lane == 0) s_kept = kept;
     }
     __syncthreads();
-    cut = s_cut;
-    int32_t kept = s_kept;
+    const int32_t kept = s_kept;
     __syncthreads();
     if (kept == 0) break;
   }
-  return cut;
+}
+
+// sides of a level (given by side(v)) into its bits, by all threads
+template <class F>
+__device__ __forceinline__ void cta_set_bits(uint32_t *bits, int32_t n, F side) {
+  for (int32_t v = threadIdx.x; v < fm_pad(n); v += IPT) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, v < n && side(v) != 0);
+    if ((threadIdx.x & 31) == 0) bits[v >> 5] = m;
+  }
+}
+
+// words of a level's row offsets and node weights, and of its entries
+__device__ __forceinline__ int64_t fm_graph_words(const LG &g) { return 2ll * g.n + 1; }
+__device__ __forceinline__ int64_t fm_entry_words(const LG &g) { return (g.ew ? (int64_t)g.m : 0) + (g.m + 1) / 2; }
+
+// the level's graph at word `at` of the dynamic shared memory, its entries too
+// when they end within `words`; complete after the caller's next barrier
+__device__ void cta_fm_graph(const LG &g, FMState &F, int32_t *dyn, int32_t at, int32_t words) {
+  int32_t *x = dyn + at, *vw = x + g.n + 1;
+  for (int32_t v = threadIdx.x; v <= g.n; v += IPT) {
+    x[v] = g.xadj[v];
+    if (v < g.n) vw[v] = g.vw[v];
+  }
+  F.xadj = x;
+  F.vw = vw;
+  F.goff = at;
+  const int32_t eo = at + (int32_t)fm_graph_words(g);
+  if (eo + fm_entry_words(g) > words) return;
+  int32_t *ew = dyn + eo;
+  uint16_t *adj = reinterpret_cast<uint16_t *>(ew + (g.ew ? g.m : 0));
+  for (int32_t q = threadIdx.x; q < g.m; q += IPT) {
+    adj[q] = g.adj[q];
+    if (g.ew) ew[q] = g.ew[q];
+  }
+  F.adj = adj;
+  if (g.ew) F.ew = ew;
+  F.eoff = eo;
+}
+
+// FM state of a level: in shared memory (dyn) when it fits there with the row
+// offsets and node weights, and with the entries too when those fit as well;
+// else in the item's scratch (glob, 16-byte aligned)
+__device__ FMState cta_fm_state(const LG &g, int32_t *dyn, int32_t dyn_words, int32_t *glob) {
+  const int64_t st = fm_words(g.n);
+  if (st + fm_graph_words(g) > dyn_words) return fm_state(glob, g);
+  FMState F = fm_state(dyn, g);
+  F.off = 0;
+  cta_fm_graph(g, F, dyn, (int32_t)st, dyn_words);
+  return F;
 }
 
 // portfolio initial bipartition by one warp: algo 0 random, 1 BFS, 2 GGG
@@ -1061,7 +1311,7 @@ __device__ void warp_initial(int algo, const LG &g, int32_t t0, uint64_t key, in
   } else {
     for (int32_t v = lane; v < n; v += 32) {
       int32_t s = 0;
-      for (int32_t q = g.xadj[v]; q < g.xadj[v + 1]; ++q) s -= g.ew[q];
+      for (int32_t q = g.xadj[v]; q < g.xadj[v + 1]; ++q) s -= lg_w(g, q);
       gain[v] = s;
     }
     __syncwarp();
@@ -1071,7 +1321,7 @@ __device__ void warp_initial(int algo, const LG &g, int32_t t0, uint64_t key, in
       if (v >= 0) {
         if (lane == 0) side[v] = 0;
         W0 += g.vw[v];
-        for (int32_t q = g.xadj[v] + lane; q < g.xadj[v + 1]; q += 32) gain[g.adj[q]] += 2 * g.ew[q];
+        for (int32_t q = g.xadj[v] + lane; q < g.xadj[v + 1]; q += 32) gain[g.adj[q]] += 2 * lg_w(g, q);
         __syncwarp();
       }
       uint64_t best = 0;
@@ -1127,7 +1377,7 @@ __device__ void record_sample(const SampleSink &K, const LG &h, const int32_t *s
     }
     for (int32_t e = threadIdx.x; e < h.m; e += IPT) {
       K.adj[s_eb + e] = h.adj[e];
-      K.ew[s_eb + e] = h.ew[e];
+      K.ew[s_eb + e] = lg_w(h, e);
     }
   }
   __syncthreads();
@@ -1139,7 +1389,7 @@ __device__ void record_sample(const SampleSink &K, const LG &h, const int32_t *s
 // side_out; 0: a cap is broken (the caller runs the plain method); -1: the
 // item's scratch is too small.
 __device__ int item_learned(const IPArgs &A, const ItemDesc &D, const LG &g, Bump &B, int32_t *dyn) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int w = threadIdx.x >> 5;
   const int32_t n = g.n;
   const int32_t P = pow2_at_least(n > 1 ? n : 2);
   float *X = reinterpret_cast<float *>(B.take((int64_t)n * MF));
@@ -1149,41 +1399,30 @@ __device__ int item_learned(const IPArgs &A, const ItemDesc &D, const LG &g, Bum
   int32_t *side = B.take(n);
   uint64_t *oh = reinterpret_cast<uint64_t *>(B.take(2ll * P));
   int32_t *ov = B.take(P);
-  int32_t *fmbuf = B.take(7ll * n + 2);
+  int32_t *fmbuf = align16(B.take(fm_words(n) + 4));
   if (B.oom) return -1;
-  GView<int32_t> G{n, g.xadj, g.adj, 0, g.vw, g.ew};
+  GView<int32_t, uint16_t> G{n, g.xadj, g.adj, 0, g.vw, g.ew};
   mp_features(G, key_step(D.key, DOM_LEARNED), X, d1, d2);
   mp_forward_cta(G, A.W, X, scr, sc);
   __syncthreads();
   if (w == 0) warp_initial(3, g, D.t0, 0, side, oh, ov, nullptr, nullptr, nullptr, sc);
   __syncthreads();
-  const int64_t c0 = level_cap(D.L0, D.t0, g.maxc), c1 = level_cap(D.L1, D.t1, g.maxc);
-  // FM's state (sides, gains, locks, moves) in shared memory when it fits
-  const bool in_smem = 8ll * n + 2 <= A.dyn_words;
-  int32_t *fs = in_smem ? dyn : side;
-  if (in_smem) {
-    for (int32_t v = threadIdx.x; v < n; v += IPT) fs[v] = side[v];
-    __syncthreads();
-  }
-  {
-    uint64_t *k0 = reinterpret_cast<uint64_t *>(dyn + 4ll * n + 2 - ((4ll * n) & 1));
-    FMBuf sb{dyn + n, dyn + 2ll * n, dyn + 3ll * n, k0, k0 + n};
-    FMBuf fb{fmbuf, fmbuf + n, fmbuf + 2ll * n, reinterpret_cast<uint64_t *>(fmbuf + 3ll * n + (n & 1)),
-             reinterpret_cast<uint64_t *>(fmbuf + 3ll * n + (n & 1)) + n};
-    cta_fm(A, g, fs, c0, c1, in_smem ? sb : fb);
-  }
+  const int32_t c0 = level_cap(D.L0, D.t0, g.maxc), c1 = level_cap(D.L1, D.t1, g.maxc);
+  const FMState F = cta_fm_state(g, dyn, A.dyn_words, fmbuf);
+  cta_set_bits(F.bits, n, [&](int32_t v) { return side[v]; });
+  __syncthreads();
+  cta_fm(A, n, c0, c1, F);
   __syncthreads();
   int64_t W0 = 0, W1 = 0;
   for (int32_t v = threadIdx.x; v < n; v += IPT) {
-    if (fs[v] == 0) W0 += g.vw[v];
+    if (fm_side(F.bits, v) == 0) W0 += g.vw[v];
     else W1 += g.vw[v];
   }
   W0 = block_sum64(W0);
   W1 = block_sum64(W1);
   if (W0 > c0 || W1 > c1) return 0;
-  for (int32_t v = threadIdx.x; v < n; v += IPT) A.side_out[D.vbase + v] = fs[v];
+  for (int32_t v = threadIdx.x; v < n; v += IPT) A.side_out[D.vbase + v] = fm_side(F.bits, v);
   __syncthreads();
-  (void)lane;
   return 1;
 }
 
@@ -1201,7 +1440,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   const ItemDesc D = A.items[it];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (D.n == 0) return;
-  Bump B{A.scratch + D.sbase, D.ssize, 0, false};
+  Bump B{A.scratch + (int64_t)blockIdx.x * A.slot, A.slot, 0, false};
   int32_t n0 = D.n;
   int32_t *x0 = B.take(n0 + 1);
   if (B.oom) {
@@ -1225,8 +1464,8 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
     g0.n = n0;
     g0.m = D.m;
     g0.xadj = x0;
-    g0.adj = const_cast<int32_t *>(A.sadj + eb);
-    g0.ew = const_cast<int32_t *>(A.sew + eb);
+    g0.adj = const_cast<uint16_t *>(A.sadj + eb);
+    g0.ew = A.sew ? const_cast<int32_t *>(A.sew + eb) : nullptr;
     g0.vw = const_cast<int32_t *>(A.svw + D.vbase);
     g0.maxdeg = md;
     g0.maxc = mc;
@@ -1260,7 +1499,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
     if (nc == g.n) break;
     int32_t *map = B.take(g.n);
     LG c;
-    item_contract(g, label, map, &c, B, wkeys, wvals);
+    item_contract(g, label, map, &c, B, A.wtab, wkeys, wvals);
     if (B.oom) break;
     int32_t cmd = 0, cmc = 0;
     for (int32_t x = threadIdx.x; x < c.n; x += IPT) {
@@ -1288,9 +1527,24 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   int32_t nH = h.n;
   int32_t PH = pow2_at_least(nH > 1 ? nH : 2);
   int32_t hL0 = level_cap(D.L0, D.t0, h.maxc), hL1 = level_cap(D.L1, D.t1, h.maxc);
-  int64_t per_warp = 12ll * nH + 3ll * PH + 16;  // even: keeps every warp's 64-bit areas aligned
-  // the portfolio's working state lives in shared memory when it fits
-  int32_t *wbuf = per_warp * IPW <= A.dyn_words ? dyn : B.take(per_warp * IPW);
+  // per warp: FM state, the best sides, the start's side, order (64-bit key and
+  // id), visited marks and queue; the coarsest graph itself once for all warps
+  const int64_t per_warp = (fm_words(nH) + fm_pad(nH) / 32 + 3ll * PH + 3ll * nH + 3) & ~3ll;
+  // in shared memory when it fits
+  const bool pf_smem = per_warp * IPW + fm_graph_words(h) <= A.dyn_words;
+  int32_t *wbuf = pf_smem ? dyn : align16(B.take(per_warp * IPW + 4));
+  FMState FH{};
+  FH.goff = FH.eoff = -1;
+  if (pf_smem) {
+    FH.adj = h.adj;
+    FH.ew = h.ew;
+    cta_fm_graph(h, FH, dyn, (int32_t)per_warp * IPW, A.dyn_words);
+    h.xadj = const_cast<int32_t *>(FH.xadj);
+    h.vw = const_cast<int32_t *>(FH.vw);
+    h.adj = const_cast<uint16_t *>(FH.adj);
+    h.ew = const_cast<int32_t *>(FH.ew);
+    __syncthreads();
+  }
   int32_t *fin = B.take(nH);
   if (B.oom) {
     if (threadIdx.x == 0) atomicExch(A.oom, 1);
@@ -1307,7 +1561,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
       if (threadIdx.x == 0) atomicExch(A.oom, 1);
       return;
     }
-    GView<int32_t> G{nH, h.xadj, h.adj, 0, h.vw, h.ew};
+    GView<int32_t, uint16_t> G{nH, h.xadj, h.adj, 0, h.vw, h.ew};
     mp_features(G, key_step(D.key, DOM_LEARNED), X, d1, d2);
     mp_forward_cta(G, A.W, X, scr, sc);
     score = sc;
@@ -1315,14 +1569,16 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   __shared__ int32_t s_bw;
   {
     int32_t *base = wbuf + per_warp * w;
-    int32_t *side = base;
-    int32_t *best = side + nH;
-    int32_t *gain = best + nH;
-    int32_t *locked = gain + nH;
-    int32_t *moves = locked + nH;
-    int32_t *queue = moves + nH;
-    int32_t *ov = queue + nH;
-    uint64_t *oh = reinterpret_cast<uint64_t *>(ov + PH);  // offset 6 nH + PH: even
+    FMState F = fm_state(base, h);
+    if (pf_smem) {
+      F.off = (int32_t)per_warp * w;
+      F.goff = FH.goff;
+      F.eoff = FH.eoff;
+    }
+    uint32_t *best = reinterpret_cast<uint32_t *>(base + fm_words(nH));
+    uint64_t *oh = reinterpret_cast<uint64_t *>(best + fm_pad(nH) / 32);  // even offset
+    int32_t *ov = reinterpret_cast<int32_t *>(oh + PH);
+    int32_t *side = ov + PH, *vis = side + nH, *queue = vis + nH;
     int32_t reps[3] = {A.rep_random, A.rep_bfs, A.rep_ggg};
     uint64_t doms[3] = {DOM_RANDOM, DOM_BFS, DOM_GGG};
     // candidates in order: [learned], the first `first[a]` repetitions of each
@@ -1402,17 +1658,15 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
           if (phase == 1) r += first[a];
         }
         uint64_t key = a == 3 ? 0 : key_step(key_step(D.key, doms[a]), (uint64_t)r);
-        warp_initial(a, h, D.t0, key, side, oh, ov, gain, locked, queue, score);
-        FMBuf fb{gain, locked, moves, oh + PH, oh + PH + nH};
-        int64_t cut = warp_fm(A, h, side, hL0, hL1, fb);
-        int64_t W0 = 0, W1 = 0;
-        for (int32_t v = lane; v < nH; v += 32) {
-          if (side[v] == 0) W0 += h.vw[v];
-          else W1 += h.vw[v];
+        warp_initial(a, h, D.t0, key, side, oh, ov, F.key, vis, queue, score);
+        for (int32_t v = lane; v < fm_pad(nH); v += 32) {
+          const unsigned m = __ballot_sync(0xFFFFFFFFu, v < nH && side[v] != 0);
+          if (lane == 0) F.bits[v >> 5] = m;
         }
-        W0 = warp_sum64(W0);
-        W1 = warp_sum64(W1);
-        int64_t o0 = W0 - hL0, o1 = W1 - hL1;
+        __syncwarp();
+        int32_t W0, W1;
+        const int64_t cut = warp_fm(A, nH, hL0, hL1, F, W0, W1);
+        int64_t o0 = (int64_t)W0 - hL0, o1 = (int64_t)W1 - hL1;
         int64_t o = o0 > o1 ? o0 : o1;
         int32_t inf = o > 0;
         int64_t ovv = inf ? o : 0;
@@ -1427,7 +1681,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
           bov = ovv;
           bcut = cut;
           brep = phase == 0 ? q : R0 + q;
-          for (int32_t v = lane; v < nH; v += 32) best[v] = side[v];
+          for (int32_t x = lane; x < fm_pad(nH) / 32; x += 32) best[x] = F.bits[x];
         }
         __syncwarp();
       }
@@ -1459,20 +1713,18 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
     }
   }
   {
-    int32_t *bsrc = wbuf + per_warp * s_bw + nH;
-    for (int32_t v = threadIdx.x; v < nH; v += IPT) fin[v] = bsrc[v];
+    const uint32_t *bsrc = reinterpret_cast<const uint32_t *>(wbuf + per_warp * s_bw + fm_words(nH));
+    for (int32_t v = threadIdx.x; v < nH; v += IPT) fin[v] = fm_side(bsrc, v);
   }
   __syncthreads();
   if (A.sink.counters && !A.sink.item_level) record_sample(A.sink, h, fin, D.key);
   // 3. uncoarsen with FM on every level (warp 0)
   int32_t *cur = fin;
-  int32_t *fmbuf = B.take(7ll * n0 + 2);
+  int32_t *fmbuf = align16(B.take(fm_words(n0) + 4));
   if (B.oom) {
     if (threadIdx.x == 0) atomicExch(A.oom, 1);
     return;
   }
-  FMBuf fb{fmbuf, fmbuf + n0, fmbuf + 2ll * n0, reinterpret_cast<uint64_t *>(fmbuf + 3ll * n0 + (n0 & 1)),
-           reinterpret_cast<uint64_t *>(fmbuf + 3ll * n0 + (n0 & 1)) + n0};
   for (int32_t l = nl - 2; l >= 0; --l) {
     LG g = lv[l];
     int32_t *fine = B.take(g.n);
@@ -1481,22 +1733,13 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
       return;
     }
     const int32_t *map = maps[l];
-    // FM's state (sides, gains, locks, moves) in shared memory when it fits:
-    // every FM step scans all nodes
-    bool in_smem = 8ll * g.n + 2 <= A.dyn_words;
-    int32_t *fs = in_smem ? dyn : fine;
-    for (int32_t v = threadIdx.x; v < g.n; v += IPT) fs[v] = cur[map[v]];
+    const FMState F = cta_fm_state(g, dyn, A.dyn_words, fmbuf);
+    cta_set_bits(F.bits, g.n, [&](int32_t v) { return cur[map[v]]; });
     __syncthreads();
-    {
-      uint64_t *k0 = reinterpret_cast<uint64_t *>(dyn + 4ll * g.n + 2 - ((4ll * g.n) & 1));
-      FMBuf sb{dyn + g.n, dyn + 2ll * g.n, dyn + 3ll * g.n, k0, k0 + g.n};
-      cta_fm(A, g, fs, level_cap(D.L0, D.t0, g.maxc), level_cap(D.L1, D.t1, g.maxc), in_smem ? sb : fb);
-    }
+    cta_fm(A, g.n, level_cap(D.L0, D.t0, g.maxc), level_cap(D.L1, D.t1, g.maxc), F);
     __syncthreads();
-    if (in_smem) {
-      for (int32_t v = threadIdx.x; v < g.n; v += IPT) fine[v] = fs[v];
-      __syncthreads();
-    }
+    for (int32_t v = threadIdx.x; v < g.n; v += IPT) fine[v] = fm_side(F.bits, v);
+    __syncthreads();
     cur = fine;
   }
   for (int32_t v = threadIdx.x; v < n0; v += IPT) A.side_out[D.vbase + v] = cur[v];
@@ -1504,11 +1747,10 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   if (A.sink.counters && A.sink.item_level) record_sample(A.sink, lv[0], cur, D.key);
 }
 
-__global__ void __launch_bounds__(IPT) k_ip_items(IPArgs A) {
-  __shared__ int32_t wkeys[IPW * IP_WTAB];
-  __shared__ int32_t wvals[IPW * IP_WTAB];
+__global__ void __launch_bounds__(IPT, 3) k_ip_items(const __grid_constant__ IPArgs A) {
   __shared__ int32_t s_it;
-  extern __shared__ __align__(16) int32_t ipdyn[];
+  extern __shared__ __align__(16) int32_t ipdyn[];  // working state, then the warps' tables
+  int32_t *wkeys = ipdyn + A.dyn_words, *wvals = wkeys + IPW * A.wtab;
   for (;;) {
     if (threadIdx.x == 0) s_it = atomicAdd(A.queue, 1);
     __syncthreads();
@@ -1571,7 +1813,7 @@ __global__ void k_local_ids(int32_t n, const int32_t *members, const int32_t *pa
 
 __global__ void k_fill_sub(int32_t n, const int64_t *xadj, const int32_t *adj, const int32_t *vw,
                            const int32_t *ew, const int32_t *part, const int32_t *members,
-                           const int32_t *loc, const int64_t *gx, int32_t *sadj, int32_t *sew,
+                           const int32_t *loc, const int64_t *gx, uint16_t *sadj, int32_t *sew,
                            int32_t *svw) {
   // a warp per row, order-preserving compaction of the entries inside the block
   int lane = threadIdx.x & 31;
@@ -1593,8 +1835,8 @@ __global__ void k_fill_sub(int32_t n, const int64_t *xadj, const int32_t *adj, c
       unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
       if (keep) {
         int64_t p = o + __popc(bal & ((1u << lane) - 1u));
-        sadj[p] = loc[u];
-        sew[p] = ew ? ew[q] : 1;
+        sadj[p] = (uint16_t)loc[u];
+        if (ew) sew[p] = ew[q];
       }
       o += __popc(bal);
     }
@@ -1671,8 +1913,10 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
   k_set_last<<<1, 1, 0, s>>>(gx, n, etot);
   KMP_LAUNCHED("set_last");
   int64_t E = read1(etot.p);
-  DBuf<int32_t> sadj(E), sew(E), svw(n);
-  k_fill_sub<<<grid, 256, 0, s>>>(n, g.xadj, g.adj, g.vw, g.ew, part, members, loc, gx, sadj, sew, svw);
+  DBuf<uint16_t> sadj(E);
+  DBuf<int32_t> sew, svw(n);
+  if (g.ew) sew.alloc(E);
+  k_fill_sub<<<grid, 256, 0, s>>>(n, g.xadj, g.adj, g.vw, g.ew, part, members, loc, gx, sadj, sew.p, svw);
   KMP_LAUNCHED("fill_sub");
   std::vector<int32_t> hcount(nblocks + 1), hoff(nblocks + 1);
   std::vector<unsigned long long> hw(nblocks), he(nblocks);
@@ -1720,18 +1964,23 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
     to_dev(dorder.p, order.data(), order.size());
     bool learned = cfg.learned && proposer().W;
     int64_t mult = 1;
+    // one wave of CTAs that take items from the queue; each has one scratch
+    // region, sized for the largest item and reused, so that what the CTAs touch
+    // stays in L2 (a region per item spread 8192 items of 2048 nodes over 36 GB)
+    int64_t maxn = 0;
+    for (auto &d : items) maxn = std::max<int64_t>(maxn, d.n);
+    const int per_sm = std::min<int>(C.tune.ip_blocks_per_sm, 3);
+    const int gridip = (int)std::min<int64_t>((int64_t)items.size(), (int64_t)C.sms * per_sm);
     for (int attempt = 0; attempt < 6; ++attempt, mult *= 4) {
-      int64_t total = 0;
+      int64_t slot = 0;
       for (auto &d : items) {
         int64_t nP = next_pow2((uint64_t)std::max(d.n, 2));
         int64_t mP = next_pow2((uint64_t)std::max(d.m, 2));
-        d.sbase = total;
-        d.ssize = mult * (104ll * d.n + 64ll * nP + 16ll * d.m + 8ll * mP + 2048 +
-                          (learned ? (int64_t)(2 * MF + 3 * MH + 4) * d.n + 64 : 0));
-        total += d.ssize;
+        slot = std::max<int64_t>(slot, mult * (104ll * d.n + 64ll * nP + 16ll * d.m + 8ll * mP + 2048 +
+                                      (learned ? (int64_t)(2 * MF + 3 * MH + 4) * d.n + 64 : 0)));
       }
       DBuf<ItemDesc> ditems(items.size());
-      DBuf<int32_t> scratch(total);
+      DBuf<int32_t> scratch(slot * gridip);
       to_dev(ditems.p, items.data(), items.size());
       q.zero();
       IPArgs A;
@@ -1742,10 +1991,11 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
       A.oom = q.p + 1;
       A.gx = gx;
       A.sadj = sadj;
-      A.sew = sew;
+      A.sew = sew.p;
       A.svw = svw;
       A.side_out = side;
       A.scratch = scratch;
+      A.slot = slot;
       A.S = cfg.subrounds;
       A.ip_C = cfg.ip_C;
       A.ip_lp_rounds = cfg.ip_lp_rounds;
@@ -1763,25 +2013,21 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
       A.adaptive = (cfg.adaptive && !A.W) ? 1 : 0;
       A.learned_item = (cfg.learned == 2 && A.W) ? 1 : 0;
       A.sink = sample_sink();
-      // dynamic shared memory: the LP working arrays (7.5 words a node plus
-      // sort space) and then the FM state (8 words a node) of the largest item of the round,
-      // at least 16 KB (the portfolio of small coarsest graphs), at most what
-      // the SM offers next to the kernel's static shared memory when the round
-      // has no more items than SMs (its items are then on the critical path,
-      // one CTA per SM), else at most 72 KB (two CTAs per SM); an item that
-      // does not fit works in its global scratch
-      int64_t maxn = 0;
-      for (auto &d : items) maxn = std::max<int64_t>(maxn, d.n);
-      int32_t cap_words = (int64_t)items.size() <= C.sms ? IP_DYN_MAX_WORDS : IP_DYN_SHARED_WORDS;
-      A.dyn_words = (int32_t)std::min<int64_t>(std::max<int64_t>(8 * maxn + 2 + 2 * maxn / 4, 4096), cap_words);
-      size_t dyn_bytes = (size_t)A.dyn_words * sizeof(int32_t);
+      // working state: the LP arrays (5.5 words a node and the sort space of a
+      // sub-round's contested proposals), then FM's (3.6 words a node, the entries
+      // where they fit) of the largest item, at least 16 KB (the portfolio of small
+      // coarsest graphs); see IPShape
+      const int64_t want = std::max<int64_t>(6 * maxn + maxn / 8 + 256, 4096);
+      const IPShape shape = (int64_t)items.size() <= C.sms ? IP_SHAPE1 : IP_SHAPE3;
+      A.wtab = shape.wtab;
+      A.dyn_words = (int32_t)std::min<int64_t>((want + 3) & ~3ll, shape.dyn_words);
+      const size_t dyn_bytes = ip_smem(IPShape{A.wtab, A.dyn_words});
       static bool attr_set = false;
       if (!attr_set) {
         KMP_CUDA(cudaFuncSetAttribute(k_ip_items, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      IP_DYN_MAX_WORDS * (int)sizeof(int32_t)));
+                                      (int)ip_smem(IP_SHAPE1)));
         attr_set = true;
       }
-      int gridip = (int)std::min<int64_t>((int64_t)items.size(), (int64_t)C.sms * C.tune.ip_blocks_per_sm);
       k_ip_items<<<gridip, IPT, dyn_bytes, s>>>(A);
       KMP_LAUNCHED("ip_items");
       int32_t oom = 0;

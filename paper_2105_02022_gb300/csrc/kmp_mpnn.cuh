@@ -28,11 +28,11 @@ constexpr int P_W1S = 0, P_W1N = P_W1S + MH * MF, P_B1 = P_W1N + MH * MF, P_W2S 
 
 // a graph seen through local node ids 0..n-1: row v is [xadj[v], xadj[v+1])
 // of the edge arrays; a neighbour's local id is adj[e] - abase
-template <class XT>
+template <class XT, class AT = int32_t>
 struct GView {
   int32_t n;
   const XT *xadj;
-  const int32_t *adj;
+  const AT *adj;
   int32_t abase;
   const int32_t *vw;  // local index, nullable
   const int32_t *ew;  // edge index, nullable
@@ -45,8 +45,8 @@ __device__ __forceinline__ float wbf(const __nv_bfloat16 *W, int i) { return __b
 // hub's row on one thread holds up the whole CTA.
 // f(entry) for every entry
 constexpr int MP_ROW_LANE = 24;
-template <class XT, class F>
-__device__ __forceinline__ void mp_rows(const GView<XT> &G, bool take, int32_t v, F f) {
+template <class XT, class AT, class F>
+__device__ __forceinline__ void mp_rows(const GView<XT, AT> &G, bool take, int32_t v, F f) {
   const int lane = threadIdx.x & 31;
   XT b = 0, e = 0;
   if (take) {
@@ -62,8 +62,8 @@ __device__ __forceinline__ void mp_rows(const GView<XT> &G, bool take, int32_t v
   }
 }
 // weighted degree of each lane's node (whole warp)
-template <class XT>
-__device__ __forceinline__ int64_t mp_wdeg(const GView<XT> &G, bool take, int32_t v) {
+template <class XT, class AT>
+__device__ __forceinline__ int64_t mp_wdeg(const GView<XT, AT> &G, bool take, int32_t v) {
   const int lane = threadIdx.x & 31;
   XT b = 0, e = 0;
   if (take) {
@@ -88,8 +88,8 @@ __device__ __forceinline__ int64_t mp_wdeg(const GView<XT> &G, bool take, int32_
 
 // Features of one graph by one CTA; d1, d2: scratch of n ints (local index).
 // The sums are whole numbers below 2^53, so their doubles are exact.
-template <class XT>
-__device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t *d1, int32_t *d2) {
+template <class XT, class AT>
+__device__ void mp_features(const GView<XT, AT> &G, uint64_t key, float *X, int32_t *d1, int32_t *d2) {
   __shared__ unsigned long long s_c, s_w, s_md;
   int32_t n = G.n;
   const int lane = threadIdx.x & 31;
@@ -148,7 +148,7 @@ __device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t 
       for (int32_t v0 = warp0; v0 < n; v0 += blockDim.x) {
         const int32_t v = v0 + lane;
         mp_rows(G, v < n && d[v] == it, v, [&](XT e) {
-          const int32_t u = G.adj[e] - G.abase;
+          const int32_t u = (int32_t)G.adj[e] - G.abase;
           if (d[u] == INT32_MAX) {
             d[u] = it + 1;
             any = true;
@@ -194,13 +194,13 @@ __device__ void mp_features(const GView<XT> &G, uint64_t key, float *X, int32_t 
 }
 
 // neighbour mean of channel c of node v (d channels per node)
-template <class XT>
-__device__ __forceinline__ float mp_nbr_mean(const GView<XT> &G, const float *H, int d, int32_t v, int c) {
+template <class XT, class AT>
+__device__ __forceinline__ float mp_nbr_mean(const GView<XT, AT> &G, const float *H, int d, int32_t v, int c) {
   float s = 0.f, ws = 0.f;
   for (XT e = G.xadj[v]; e < G.xadj[v + 1]; ++e) {
     float w = G.ew ? (float)G.ew[e] : 1.f;
     ws += w;
-    s = __fmaf_rn(w, H[(int64_t)(G.adj[e] - G.abase) * d + c], s);
+    s = __fmaf_rn(w, H[(int64_t)((int32_t)G.adj[e] - G.abase) * d + c], s);
   }
   return ws > 0.f ? s / ws : 0.f;
 }
@@ -223,8 +223,8 @@ __device__ __forceinline__ float mp_readout(const __nv_bfloat16 *W, const float 
 }
 
 // forward of one graph by one CTA (inference): scores S[n]; scratch: n*(MF + 3*MH) floats
-template <class XT>
-__device__ void mp_forward_cta(const GView<XT> &G, const __nv_bfloat16 *W, const float *X, float *scr,
+template <class XT, class AT>
+__device__ void mp_forward_cta(const GView<XT, AT> &G, const __nv_bfloat16 *W, const float *X, float *scr,
                                float *S) {
   int32_t n = G.n;
   float *M0 = scr, *H1 = M0 + (int64_t)n * MF, *M1 = H1 + (int64_t)n * MH, *H2 = M1 + (int64_t)n * MH;
