@@ -6,16 +6,21 @@
 // GPU layout: coarse ids = exclusive scan of "label used" flags (ascending
 // label); members grouped by a counting sort.  A coarse node whose members'
 // total degree is <= 512 is aggregated by one warp in a shared-memory hash
-// table (four bins by size: 64, 128, 256, 512) and sorted by a warp bitonic
-// network; one whose total degree is <= 8192 by one CTA in a shared-memory
-// table sized for it (three bins: 2048, 4096, 8192), ordered by a bitmap rank
-// or a block bitonic network; larger rows are aggregated by all their
-// members' warps in parallel into global tables, and the distinct entries of
-// all large rows are ordered by one GPU-wide key-value radix sort of
-// (row, neighbour).  Rows go to temporary space at upper-bound offsets; a
+// table (four bins by size: 64, 128, 256, 512), one whose total degree is
+// <= 8192 by one CTA in a table sized for it (three bins: 2048, 4096, 8192);
+// larger rows are aggregated by all their members' warps in parallel into
+// global tables.  A row is put in order by the cheapest way that its ids allow:
+// the rank in a bitmap of its id span; buckets of equal id ranges; a bitonic
+// network where ids crowd into few buckets (and for the shortest rows).  The
+// longest rows go through one counting sort by (row, high neighbour bits) and a
+// bitmap per segment.  Rows go to temporary space at upper-bound offsets; a
 // prefix sum of the row lengths then places them into the final CSR.
+// R-MAT 2^24 with its level-0 clusters, whole contraction: 74.0 ms with networks
+// for all rows whose ids span far (66 steps an entry at 2048 entries), 33.3 now.
 // Also: projection (Algorithm 1), cut and block weights (Section 2), and the
 // per-graph facts the other kernels need (max degree, isolated nodes, weights).
+#include <climits>
+
 #include "kmp_internal.cuh"
 
 namespace kmp {
@@ -71,12 +76,46 @@ __global__ void k_members(int32_t n, const int32_t *map, const int32_t *moff, in
   }
 }
 
-// split coarse nodes by row class: list c holds its rows at lists + c * nc
-__global__ void k_split_ub(int32_t nc, const unsigned long long *cub, int32_t *lists, int32_t *counts) {
-  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nc;
-       x += (int64_t)gridDim.x * blockDim.x) {
-    int c = row_class(cub[x]);
-    lists[(int64_t)c * nc + atomicAdd(&counts[c], 1)] = (int32_t)x;
+// Split coarse nodes by row class: list c holds its rows at lists + c * nc (in any
+// order).  A CTA counts a tile's classes in shared memory and claims each class's
+// places with one atomic: one atomic a row on eight counters made this the
+// longest kernel of a mesh level (1.2 M rows: 117 us, 12 now).
+constexpr int SPLIT_PER = 8;
+__global__ void __launch_bounds__(256) k_split_ub(int32_t nc, const unsigned long long *cub, int32_t *lists,
+                                                  int32_t *counts) {
+  __shared__ int32_t cnt[NCLASS], base[NCLASS];
+  const int lane = threadIdx.x & 31;
+  for (int64_t t0 = (int64_t)blockIdx.x * 256 * SPLIT_PER; t0 < nc; t0 += (int64_t)gridDim.x * 256 * SPLIT_PER) {
+    if (threadIdx.x < NCLASS) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    int32_t cls[SPLIT_PER], rank[SPLIT_PER];
+#pragma unroll
+    for (int r = 0; r < SPLIT_PER; ++r) {
+      const int64_t x = t0 + r * 256 + threadIdx.x;
+      cls[r] = x < nc ? row_class(cub[x]) : -1;
+    }
+#pragma unroll
+    for (int r = 0; r < SPLIT_PER; ++r) {
+      rank[r] = 0;
+#pragma unroll
+      for (int c = 0; c < NCLASS; ++c) {
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, cls[r] == c);
+        if (m == 0) continue;
+        int32_t at = 0;
+        if (lane == 0) at = atomicAdd(&cnt[c], __popc(m));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0);
+        if (cls[r] == c) rank[r] = at + __popc(m & ((1u << lane) - 1u));
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < NCLASS && cnt[threadIdx.x] > 0)
+      base[threadIdx.x] = atomicAdd(&counts[threadIdx.x], cnt[threadIdx.x]);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SPLIT_PER; ++r)
+      if (cls[r] >= 0)
+        lists[(int64_t)cls[r] * nc + base[cls[r]] + rank[r]] = (int32_t)(t0 + r * 256 + threadIdx.x);
+    __syncthreads();
   }
 }
 
@@ -109,6 +148,100 @@ __device__ __forceinline__ void bitonic(uint64_t *a, uint32_t P, uint32_t t, uin
   }
 }
 
+// Order of `cnt` entries (neighbour << 32 | weight, neighbours distinct) by
+// neighbour through buckets of equal id ranges, about one entry each: L is
+// counted by bucket (H: nb + 1 counters), scattered to M in bucket order, and an
+// entry's place is its bucket's start plus the smaller entries of its bucket.
+// That is a few shared-memory steps an entry, where a bitonic network of 2^p
+// takes p (p + 1) / 2.  Ids that crowd into a bucket would make the last step
+// quadratic: false (nothing but H and M touched) when one holds more than
+// BUCKET_MAX, and the caller sorts by the network.  All threads of the group
+// (a warp, or a CTA with s_wsum / s_max) call it; out(place, entry) writes.
+constexpr int32_t BUCKET_MAX = 32;
+template <int NT>
+__device__ __forceinline__ int32_t block_scan_excl(int32_t v, int32_t *s_wsum /* NT / 32 */);
+__device__ __forceinline__ int bucket_shift(int32_t ymin, int32_t ymax, int32_t nb) {
+  const int sh = (32 - __clz((ymax - ymin) | 1)) - (31 - __clz(nb));
+  return sh > 0 ? sh : 0;
+}
+template <class F>
+__device__ __forceinline__ bool bucket_order_warp(const uint64_t *L, int32_t cnt, int32_t ymin, int32_t ymax, int32_t nb,
+                                                  int32_t *H, uint64_t *M, F out) {
+  const int lane = threadIdx.x & 31;
+  const int sh = bucket_shift(ymin, ymax, nb);
+  for (int32_t j = lane; j < nb; j += 32) H[j] = 0;
+  __syncwarp();
+  for (int32_t j = lane; j < cnt; j += 32) atomicAdd(&H[((int32_t)(L[j] >> 32) - ymin) >> sh], 1);
+  __syncwarp();
+  int32_t run = 0, top = 0;
+  for (int32_t j0 = 0; j0 < nb; j0 += 32) {
+    const int32_t h = j0 + lane < nb ? H[j0 + lane] : 0;
+    top = max(top, h);
+    int32_t inc = h;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (j0 + lane < nb) H[j0 + lane] = run + inc - h;
+    run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+  }
+  if (__reduce_max_sync(0xFFFFFFFFu, top) > BUCKET_MAX) return false;
+  __syncwarp();
+  for (int32_t j = lane; j < cnt; j += 32) {
+    const uint64_t e = L[j];
+    M[atomicAdd(&H[((int32_t)(e >> 32) - ymin) >> sh], 1)] = e;
+  }
+  __syncwarp();  // H[b] is the end of bucket b now
+  for (int32_t j = lane; j < cnt; j += 32) {
+    const uint64_t e = M[j];
+    const int32_t b = ((int32_t)(e >> 32) - ymin) >> sh, lo = b > 0 ? H[b - 1] : 0, hi = H[b];
+    int32_t r = lo;
+    for (int32_t q = lo; q < hi; ++q) r += M[q] < e;
+    out(r, e);
+  }
+  return true;
+}
+template <int NT, class F>
+__device__ __forceinline__ bool bucket_order_cta(const uint64_t *L, int32_t cnt, int32_t ymin, int32_t ymax, int32_t nb,
+                                                 int32_t *H, uint64_t *M, int32_t *s_wsum, int32_t *s_max, F out) {
+  const int tid = threadIdx.x;
+  const int sh = bucket_shift(ymin, ymax, nb);
+  for (int32_t j = tid; j < nb; j += NT) H[j] = 0;
+  if (tid == 0) *s_max = 0;
+  __syncthreads();
+  for (int32_t j = tid; j < cnt; j += NT) atomicAdd(&H[((int32_t)(L[j] >> 32) - ymin) >> sh], 1);
+  __syncthreads();
+  const int32_t seg = (nb + NT - 1) / NT, a = min(tid * seg, nb), b = min(a + seg, nb);
+  int32_t loc = 0, top = 0;
+  for (int32_t j = a; j < b; ++j) {
+    loc += H[j];
+    top = max(top, H[j]);
+  }
+  if (top > BUCKET_MAX) *s_max = 1;
+  int32_t base = block_scan_excl<NT>(loc, s_wsum);
+  for (int32_t j = a; j < b; ++j) {
+    const int32_t h = H[j];
+    H[j] = base;
+    base += h;
+  }
+  __syncthreads();
+  if (*s_max) return false;
+  for (int32_t j = tid; j < cnt; j += NT) {
+    const uint64_t e = L[j];
+    M[atomicAdd(&H[((int32_t)(e >> 32) - ymin) >> sh], 1)] = e;
+  }
+  __syncthreads();
+  for (int32_t j = tid; j < cnt; j += NT) {
+    const uint64_t e = M[j];
+    const int32_t k = ((int32_t)(e >> 32) - ymin) >> sh, lo = k > 0 ? H[k - 1] : 0, hi = H[k];
+    int32_t r = lo;
+    for (int32_t q = lo; q < hi; ++q) r += M[q] < e;
+    out(r, e);
+  }
+  return true;
+}
+
 // warp path: one coarse node per warp for rows whose members' total degree
 // ub is at most TABW / 2.  The table packs (neighbour << 32 | weight) per slot
 // (key and weight updated as the two 32-bit halves), is sized to the power of
@@ -122,6 +255,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_aggregate_warp(
     const int32_t *adj, const int32_t *ew, const int32_t *map, const int32_t *members,
     const int32_t *moff, const int64_t *toff, int32_t *tadj, int32_t *tw, int32_t *cdeg) {
   __shared__ uint64_t tab[WARPS][TABW];
+  __shared__ int32_t hist[TABW >= 256 ? WARPS : 1][TABW >= 256 ? TABW / 2 : 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint64_t *T = tab[w];
   int32_t *H = reinterpret_cast<int32_t *>(T);  // H[2 j] weight, H[2 j + 1] key of slot j
@@ -190,13 +324,32 @@ __global__ void __launch_bounds__(WARPS * 32) k_aggregate_warp(
     }
     uint32_t P = 1;
     while (P < (uint32_t)cnt) P <<= 1;
-    for (uint32_t j = cnt + lane; j < P; j += 32) T[j] = ~0ull;
-    __syncwarp();
-    bitonic<false>(T, P, lane, 32);
     const int64_t o = toff[x];
-    for (int32_t j = lane; j < cnt; j += 32) {
-      tadj[o + j] = (int32_t)(T[j] >> 32);
-      tw[o + j] = (int32_t)(uint32_t)T[j];
+    bool done = false;
+    if (TABW >= 256 && P >= 64) {
+      // the entries fill at most half of the table: the other half is the scatter space
+      int32_t ymin = INT32_MAX, ymax = 0;
+      for (int32_t j = lane; j < cnt; j += 32) {
+        const int32_t y = (int32_t)(T[j] >> 32);
+        ymin = min(ymin, y);
+        ymax = max(ymax, y);
+      }
+      ymin = __reduce_min_sync(0xFFFFFFFFu, ymin);
+      ymax = __reduce_max_sync(0xFFFFFFFFu, ymax);
+      done = bucket_order_warp(T, cnt, ymin, ymax, (int32_t)P, hist[w], T + TABW / 2, [&](int32_t r, uint64_t e) {
+        tadj[o + r] = (int32_t)(e >> 32);
+        tw[o + r] = (int32_t)(uint32_t)e;
+      });
+      __syncwarp();
+    }
+    if (!done) {
+      for (uint32_t j = cnt + lane; j < P; j += 32) T[j] = ~0ull;
+      __syncwarp();
+      bitonic<false>(T, P, lane, 32);
+      for (int32_t j = lane; j < cnt; j += 32) {
+        tadj[o + j] = (int32_t)(T[j] >> 32);
+        tw[o + j] = (int32_t)(uint32_t)T[j];
+      }
     }
     if (lane == 0) cdeg[x] = cnt;
     __syncwarp();
@@ -207,8 +360,9 @@ template <int TABW, int WARPS>
 void launch_aggregate_warp(const int32_t *list, int32_t nrows, const unsigned long long *cub, const Graph &g,
                            const int32_t *map, const int32_t *members, const int32_t *moff,
                            const int64_t *toff, int32_t *tadj, int32_t *tw, int32_t *cdeg) {
-  static_assert(TABW >= 64 && TABW * WARPS * sizeof(uint64_t) <= 48 * 1024, "bin shape");
-  constexpr int per_sm_smem = (int)((227u << 10) / (TABW * WARPS * sizeof(uint64_t) + 1024));
+  constexpr size_t bytes = (size_t)TABW * WARPS * sizeof(uint64_t) + (TABW >= 256 ? TABW / 2 * WARPS * sizeof(int32_t) : 4);
+  static_assert(TABW >= 64 && bytes <= 48 * 1024, "bin shape");
+  constexpr int per_sm_smem = (int)((227u << 10) / (bytes + 1024));
   constexpr int per_sm = per_sm_smem < 64 / WARPS ? per_sm_smem : 64 / WARPS;
   k_aggregate_warp<TABW, WARPS><<<grid_for(nrows, WARPS, per_sm), WARPS * 32, 0, ctx().stream>>>(
       list, nrows, cub, g.xadj, g.adj, g.ew, map, members, moff, toff, tadj, tw, cdeg);
@@ -266,7 +420,7 @@ __global__ void __launch_bounds__(NT) k_aggregate_cta(
   uint64_t *L = reinterpret_cast<uint64_t *>(cta_smem);      // TAB / 2 sort entries
   int32_t *K = reinterpret_cast<int32_t *>(L + TAB / 2);     // TAB keys
   int32_t *V = K + TAB;                                       // TAB weights
-  __shared__ int32_t s_cnt, s_ymin, s_ymax;
+  __shared__ int32_t s_cnt, s_ymin, s_ymax, s_max;
   __shared__ int32_t s_pre[NT + 1];
   __shared__ int64_t s_b[NT];
   __shared__ int32_t s_wsum[NT / 32];
@@ -362,7 +516,11 @@ __global__ void __launch_bounds__(NT) k_aggregate_cta(
         tadj[o + r] = y;
         tw[o + r] = (int32_t)(uint32_t)ent;
       }
-    } else {
+    } else if (!bucket_order_cta<NT>(L, cnt, ymin, s_ymax, (int32_t)P, K, reinterpret_cast<uint64_t *>(V), s_wsum, &s_max,
+                                     [&](int32_t r, uint64_t e) {
+                                       tadj[o + r] = (int32_t)(e >> 32);
+                                       tw[o + r] = (int32_t)(uint32_t)e;
+                                     })) {
       for (uint32_t j = cnt + tid; j < P; j += NT) L[j] = ~0ull;
       __syncthreads();
       bitonic<true>(L, P, tid, NT);
@@ -493,7 +651,7 @@ __global__ void __launch_bounds__(256) k_large_compact(int64_t LT, const int32_t
 }
 
 // large rows by their distinct entries: up to SORT_S (one CTA of 256 threads
-// sorts in shared memory), up to SORT_L (1024 threads), more (radix sort)
+// orders them in shared memory), up to SORT_L (1024 threads), more (segments)
 constexpr int32_t SORT_S = 2048;
 constexpr int32_t SORT_L = 16384;
 __global__ void k_large_split(const int32_t *rows, const int32_t *nrows, const int32_t *cdeg, int32_t cap,
@@ -506,35 +664,79 @@ __global__ void k_large_split(const int32_t *rows, const int32_t *nrows, const i
   }
 }
 
-// one CTA per row: (neighbour << 32 | weight) sorted in shared memory; the
-// neighbours of a row are distinct, so the order is by neighbour
+// One CTA per row: the row's entries go through buckets of equal id ranges
+// (bucket_order_cta's way) straight from global memory: counted, scattered to
+// shared memory in bucket order, placed by rank.  A row whose ids crowd into a
+// bucket is sorted by a bitonic network.
 template <int P, int NT>
-__global__ void __launch_bounds__(NT) k_large_sort_smem(const int32_t *rows, int32_t nrows, const int64_t *toff,
-                                                        const int32_t *cdeg, int32_t *tadj, int32_t *tw) {
-  extern __shared__ uint64_t srt[];  // P entries
-  const uint32_t tid = threadIdx.x;
+__global__ void __launch_bounds__(NT) k_large_sort_smem(int32_t nc, const int32_t *rows, int32_t nrows,
+                                                        const int64_t *toff, const int32_t *cdeg, int32_t *tadj,
+                                                        int32_t *tw) {
+  extern __shared__ uint64_t srt[];  // P entries, P / 2 counters
+  __shared__ int32_t s_wsum[NT / 32], s_max;
+  int32_t *H = reinterpret_cast<int32_t *>(srt + P);
+  const int32_t tid = threadIdx.x;
   for (int64_t i = blockIdx.x; i < nrows; i += gridDim.x) {
     const int32_t x = rows[i];
     const int64_t o = toff[x];
     const int32_t d = cdeg[x];
-    uint32_t Q = 32;
-    while ((int32_t)Q < d) Q <<= 1;
-    for (uint32_t j = tid; j < Q; j += NT)
-      srt[j] = (int32_t)j < d ? ((uint64_t)(uint32_t)tadj[o + j] << 32) | (uint32_t)tw[o + j] : ~0ull;
+    int32_t Q = 64;
+    while (Q < d) Q <<= 1;
+    const int32_t nb = Q / 2;
+    const int sh = bucket_shift(0, nc, nb);
+    for (int32_t j = tid; j < nb; j += NT) H[j] = 0;
+    if (tid == 0) s_max = 0;
     __syncthreads();
-    bitonic<true>(srt, Q, tid, NT);
-    for (uint32_t j = tid; (int32_t)j < d; j += NT) {
-      tadj[o + j] = (int32_t)(srt[j] >> 32);
-      tw[o + j] = (int32_t)(uint32_t)srt[j];
+#pragma unroll 4
+    for (int32_t j = tid; j < d; j += NT) atomicAdd(&H[tadj[o + j] >> sh], 1);
+    __syncthreads();
+    const int32_t seg = (nb + NT - 1) / NT, a = min(tid * seg, nb), b = min(a + seg, nb);
+    int32_t loc = 0, top = 0;
+    for (int32_t j = a; j < b; ++j) {
+      loc += H[j];
+      top = max(top, H[j]);
     }
-    __syncthreads();  // the next row reuses the array
+    if (top > BUCKET_MAX) s_max = 1;
+    int32_t base = block_scan_excl<NT>(loc, s_wsum);
+    for (int32_t j = a; j < b; ++j) {
+      const int32_t h = H[j];
+      H[j] = base;
+      base += h;
+    }
+    __syncthreads();
+    if (!s_max) {
+#pragma unroll 4
+      for (int32_t j = tid; j < d; j += NT) {
+        const int32_t y = tadj[o + j];
+        srt[atomicAdd(&H[y >> sh], 1)] = ((uint64_t)(uint32_t)y << 32) | (uint32_t)tw[o + j];
+      }
+      __syncthreads();
+      for (int32_t j = tid; j < d; j += NT) {
+        const uint64_t e = srt[j];
+        const int32_t k = (int32_t)(e >> 32) >> sh, lo = k > 0 ? H[k - 1] : 0, hi = H[k];
+        int32_t r = lo;
+        for (int32_t q = lo; q < hi; ++q) r += srt[q] < e;
+        tadj[o + r] = (int32_t)(e >> 32);
+        tw[o + r] = (int32_t)(uint32_t)e;
+      }
+    } else {
+      for (int32_t j = tid; j < Q; j += NT)
+        srt[j] = j < d ? ((uint64_t)(uint32_t)tadj[o + j] << 32) | (uint32_t)tw[o + j] : ~0ull;
+      __syncthreads();
+      bitonic<true>(srt, Q, tid, NT);
+      for (int32_t j = tid; j < d; j += NT) {
+        tadj[o + j] = (int32_t)(srt[j] >> 32);
+        tw[o + j] = (int32_t)(uint32_t)srt[j];
+      }
+    }
+    __syncthreads();  // the next row reuses the arrays
   }
 }
 
 template <int P, int NT>
-void launch_large_sort_smem(const int32_t *rows, int32_t nrows, const int64_t *toff, const int32_t *cdeg,
+void launch_large_sort_smem(int32_t nc, const int32_t *rows, int32_t nrows, const int64_t *toff, const int32_t *cdeg,
                             int32_t *tadj, int32_t *tw) {
-  constexpr size_t bytes = (size_t)P * sizeof(uint64_t);
+  constexpr size_t bytes = (size_t)P * sizeof(uint64_t) + (size_t)P / 2 * sizeof(int32_t);
   static bool attr = false;
   if (!attr) {
     KMP_CUDA(cudaFuncSetAttribute(k_large_sort_smem<P, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -545,107 +747,101 @@ void launch_large_sort_smem(const int32_t *rows, int32_t nrows, const int64_t *t
   if (per_sm < 1) per_sm = 1;
   if (per_sm > 2048 / NT) per_sm = 2048 / NT;
   int blocks = std::min<int64_t>(nrows, (int64_t)ctx().sms * per_sm);
-  k_large_sort_smem<P, NT><<<blocks, NT, bytes, ctx().stream>>>(rows, nrows, toff, cdeg, tadj, tw);
+  k_large_sort_smem<P, NT><<<blocks, NT, bytes, ctx().stream>>>(nc, rows, nrows, toff, cdeg, tadj, tw);
   KMP_LAUNCHED("large_sort_smem");
 }
 
-// rows too long for shared memory: their entries as (rank << bits | neighbour,
-// weight), a warp per row, at the row's offset among them
-__global__ void k_large_gather(const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
-                               const int32_t *tadj, const int32_t *tw, const int32_t *cdeg, int bits,
-                               uint64_t *ek, int32_t *ev) {
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = gw; r < nrows; r += nw) {
-    const int32_t x = rows[r], d = cdeg[x];
-    const int64_t o = toff[x], b = boff[r];
-    for (int32_t j = lane; j < d; j += 32) {
-      ek[b + j] = ((uint64_t)r << bits) | (uint64_t)(uint32_t)tadj[o + j];
-      ev[b + j] = tw[o + j];
-    }
-  }
-}
-
-// The longer rows' entries (rank r << bits | neighbour) are ordered by a
-// counting sort on (r, neighbour >> SEG_LO): every such segment holds at most
-// 2^SEG_LO distinct neighbours of one row, and one CTA then sorts it in shared
-// memory by the low bits.
+// The longest rows (rank r, entries [boff[r], boff[r + 1]) of all of them) are
+// ordered by a counting sort on (r, neighbour >> SEG_LO): such a segment holds
+// distinct neighbours within 2^SEG_LO ids, so a bitmap of the segment and its
+// popcount prefix give every entry's place.  Entries are taken one a thread,
+// whatever the rows' lengths (a warp a row took 8.5 of the 73 ms that
+// contracting R-MAT 2^24 takes), read from the temporary rows, scattered once,
+// and written back in place.
 constexpr int SEG_LO = 14;
-static_assert((1 << SEG_LO) == SORT_L, "a segment fits the larger shared-memory sort");
-__global__ void k_seg_hist(int64_t N, const uint64_t *ek, int bits, int32_t *hist) {
-  const int hb = bits - SEG_LO;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t k = ek[i];
-    atomicAdd(&hist[((k >> bits) << hb) | ((k & ((1ull << bits) - 1ull)) >> SEG_LO)], 1);
+__device__ __forceinline__ int32_t row_of(const int64_t *boff, int32_t nrows, int64_t i) {
+  int32_t lo = 0, hi = nrows - 1;  // last row with boff[row] <= i
+  while (lo < hi) {
+    const int32_t mid = (lo + hi + 1) >> 1;
+    if (boff[mid] <= i) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+__global__ void k_seg_hist(int64_t N, const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
+                           const int32_t *tadj, int hb, int32_t *hist) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r = row_of(boff, nrows, i);
+    atomicAdd(&hist[((int64_t)r << hb) | (tadj[toff[rows[r]] + (i - boff[r])] >> SEG_LO)], 1);
   }
 }
-__global__ void k_seg_scatter(int64_t N, const uint64_t *ek, const int32_t *ev, int bits, const int32_t *off,
-                              int32_t *cur, uint64_t *ek2, int32_t *ev2) {
-  const int hb = bits - SEG_LO;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t k = ek[i];
-    const int64_t x = (int64_t)(((k >> bits) << hb) | ((k & ((1ull << bits) - 1ull)) >> SEG_LO));
+__global__ void k_seg_scatter(int64_t N, const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
+                              const int32_t *tadj, const int32_t *tw, int hb, const int32_t *off, int32_t *cur,
+                              int32_t *ek, int32_t *ev) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r = row_of(boff, nrows, i);
+    const int64_t q = toff[rows[r]] + (i - boff[r]);
+    const int32_t y = tadj[q];
+    const int64_t x = ((int64_t)r << hb) | (y >> SEG_LO);
     const int64_t p = (int64_t)off[x] + atomicAdd(&cur[x], 1);
-    ek2[p] = k;
-    ev2[p] = ev[i];
+    ek[p] = y;
+    ev[p] = tw[q];
   }
 }
-// non-empty segments by size: up to SORT_S entries (list 0) and up to SORT_L (list 1)
-__global__ void k_seg_split(int64_t X, const int32_t *hist, int32_t *lists, int32_t *counts, int64_t cap) {
-  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < X;
-       x += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t len = hist[x];
-    if (len == 0) continue;
-    const int c = len <= SORT_S ? 0 : 1;
-    lists[(int64_t)c * cap + atomicAdd(&counts[c], 1)] = (int32_t)x;
-  }
-}
-// one CTA per segment: (low SEG_LO bits << 32 | weight) sorted in shared memory
-template <int P, int NT>
-__global__ void __launch_bounds__(NT) k_seg_sort(const int32_t *segs, int32_t nseg, const int32_t *off,
-                                                 const int32_t *hist, uint64_t *ek, int32_t *ev) {
-  extern __shared__ uint64_t srt[];  // P entries
-  const uint32_t tid = threadIdx.x;
-  const uint64_t lo_mask = (1ull << SEG_LO) - 1ull;
-  for (int64_t i = blockIdx.x; i < nseg; i += gridDim.x) {
-    const int32_t x = segs[i];
-    const int64_t o = off[x];
+// one CTA per non-empty segment
+__global__ void __launch_bounds__(256) k_seg_place(int64_t X, const int32_t *hist, const int32_t *off, int hb,
+                                                   const int32_t *ek, const int32_t *ev, const int32_t *rows,
+                                                   const int64_t *boff, const int64_t *toff, int32_t *tadj,
+                                                   int32_t *tw) {
+  constexpr int W = 1 << (SEG_LO - 5), PER = W / 256;
+  __shared__ uint32_t bm[W];
+  __shared__ int32_t pf[W];
+  __shared__ int32_t s_wsum[8];
+  const int tid = threadIdx.x;
+  for (int64_t x = blockIdx.x; x < X; x += gridDim.x) {
     const int32_t d = hist[x];
-    const uint64_t hi = ek[o] & ~lo_mask;
-    uint32_t Q = 32;
-    while ((int32_t)Q < d) Q <<= 1;
-    for (uint32_t j = tid; j < Q; j += NT)
-      srt[j] = (int32_t)j < d ? ((ek[o + j] & lo_mask) << 32) | (uint32_t)ev[o + j] : ~0ull;
+    if (d == 0) continue;
+    const int64_t o = off[x];
+    const int32_t r = (int32_t)(x >> hb);
+    const int64_t to = toff[rows[r]] + (o - boff[r]);
+#pragma unroll
+    for (int u = 0; u < PER; ++u) bm[tid * PER + u] = 0;
     __syncthreads();
-    bitonic<true>(srt, Q, tid, NT);
-    for (uint32_t j = tid; (int32_t)j < d; j += NT) {
-      ek[o + j] = hi | (srt[j] >> 32);
-      ev[o + j] = (int32_t)(uint32_t)srt[j];
+    for (int32_t j = tid; j < d; j += 256) {
+      const int32_t y = ek[o + j] & ((1 << SEG_LO) - 1);
+      atomicOr(&bm[y >> 5], 1u << (y & 31));
     }
-    __syncthreads();  // the next segment reuses the array
+    __syncthreads();
+    int32_t loc = 0;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) loc += __popc(bm[tid * PER + u]);
+    int32_t base = block_scan_excl<256>(loc, s_wsum);
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      pf[tid * PER + u] = base;
+      base += __popc(bm[tid * PER + u]);
+    }
+    __syncthreads();
+    for (int32_t j = tid; j < d; j += 256) {
+      const int32_t y = ek[o + j], l = y & ((1 << SEG_LO) - 1);
+      const int64_t p = to + pf[l >> 5] + __popc(bm[l >> 5] & ((1u << (l & 31)) - 1u));
+      tadj[p] = y;
+      tw[p] = ev[o + j];
+    }
+    __syncthreads();  // the next segment reuses the bitmap
   }
 }
-template <int P, int NT>
-void launch_seg_sort(const int32_t *segs, int32_t nseg, const int32_t *off, const int32_t *hist, uint64_t *ek,
-                     int32_t *ev) {
-  constexpr size_t bytes = (size_t)P * sizeof(uint64_t);
-  static bool attr = false;
-  if (!attr) {
-    KMP_CUDA(cudaFuncSetAttribute(k_seg_sort<P, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    attr = true;
+// entries as (rank << bits | neighbour, weight) and back, for the radix sort
+// that serves coarse graphs whose segment counters would not fit int32
+__global__ void k_large_gather(int64_t N, const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
+                               const int32_t *tadj, const int32_t *tw, int bits, uint64_t *ek, int32_t *ev) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r = row_of(boff, nrows, i);
+    const int64_t q = toff[rows[r]] + (i - boff[r]);
+    ek[i] = ((uint64_t)r << bits) | (uint64_t)(uint32_t)tadj[q];
+    ev[i] = tw[q];
   }
-  int per_sm = (int)((227u << 10) / (bytes + 1024));
-  if (per_sm < 1) per_sm = 1;
-  if (per_sm > 2048 / NT) per_sm = 2048 / NT;
-  int blocks = std::min<int64_t>(nseg, (int64_t)ctx().sms * per_sm);
-  k_seg_sort<P, NT><<<blocks, NT, bytes, ctx().stream>>>(segs, nseg, off, hist, ek, ev);
-  KMP_LAUNCHED("seg_sort");
 }
-
-// sorted entries back into their rows (rank r's entries fill [boff[r], boff[r + 1]))
 __global__ void k_large_place(int64_t N, const uint64_t *ek, const int32_t *ev, int bits, const int32_t *rows,
                               const int64_t *boff, const int64_t *toff, int32_t *tadj, int32_t *tw) {
   const uint64_t mask = (1ull << bits) - 1ull;
@@ -787,7 +983,7 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
   cdeg.zero();
   DBuf<int32_t> lists((int64_t)NCLASS * nc), counts(NCLASS);
   counts.zero();
-  k_split_ub<<<gridc, 256, 0, s>>>(nc, cub, lists, counts);
+  k_split_ub<<<grid_for(nc, 256 * SPLIT_PER), 256, 0, s>>>(nc, cub, lists, counts);
   KMP_LAUNCHED("split_ub");
   int32_t hc[NCLASS];
   to_host(hc, counts.p, NCLASS);
@@ -804,9 +1000,8 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
   if (hc[CLS_GLOBAL] > 0) {
     // large rows: every member inserts in parallel into its coarse node's global
     // table; each row's distinct entries are compacted into its temporary row
-    // and sorted there by neighbour: in shared memory by one CTA per row when
-    // they fit; the longer rows' entries by a key-value radix sort of (row
-    // rank, neighbour's high bits) and then per segment in shared memory
+    // and put in order there: in shared memory by one CTA per row when they fit,
+    // the longer rows by segments
     int bits = 1;
     while ((1ll << bits) < (int64_t)nc) ++bits;
     DBuf<int64_t> tsz(nc), ltoff(nc), ltot(1);
@@ -842,8 +1037,8 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
     KMP_LAUNCHED("large_split");
     int32_t sc[3];
     to_host(sc, scounts.p, 3);
-    if (sc[0] > 0) launch_large_sort_smem<SORT_S, 256>(slists.p, sc[0], toff, cdeg, tadj, tw);
-    if (sc[1] > 0) launch_large_sort_smem<SORT_L, 1024>(slists.p + nlarge, sc[1], toff, cdeg, tadj, tw);
+    if (sc[0] > 0) launch_large_sort_smem<SORT_S, 256>(nc, slists.p, sc[0], toff, cdeg, tadj, tw);
+    if (sc[1] > 0) launch_large_sort_smem<SORT_L, 1024>(nc, slists.p + nlarge, sc[1], toff, cdeg, tadj, tw);
     if (sc[2] > 0) {
       const int32_t nbig = sc[2];
       const int32_t *brows = slists.p + 2ll * nlarge;
@@ -852,44 +1047,35 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
       KMP_LAUNCHED("gather_deg");
       scan_excl_i64(bdeg, boff, nbig, btot);
       const int64_t NE = read1(btot.p);
-      DBuf<uint64_t> ek(NE), ektmp(NE);
-      DBuf<int32_t> ev(NE), evtmp(NE);
-      k_large_gather<<<grid_for((int64_t)nbig * 32, 256), 256, 0, s>>>(brows, nbig, boff, toff, tadj, tw, cdeg,
-                                                                      bits, ek, ev);
-      KMP_LAUNCHED("large_gather");
-      // counting sort by (rank, neighbour >> SEG_LO), then every segment by the
-      // low bits in shared memory (a row above SORT_L entries has more than
-      // 2^SEG_LO distinct neighbours, so bits > SEG_LO here)
+      // (a row above SORT_L entries has more than 2^SEG_LO distinct neighbours, so
+      // bits > SEG_LO here)
       const int hb = bits - SEG_LO;
       const int64_t X = (int64_t)nbig << hb;
+      const int gridN = grid_for(NE, 256);
       if (X > (int64_t)INT32_MAX / 2) {
         // counters beyond int32 indexing (coarse graphs near 2^31 nodes): one
         // key-value radix sort of (rank, neighbour) instead
+        DBuf<uint64_t> ek(NE), ektmp(NE);
+        DBuf<int32_t> ev(NE), evtmp(NE);
         int rbits = 1;
         while ((1ll << rbits) < (int64_t)nbig) ++rbits;
+        k_large_gather<<<gridN, 256, 0, s>>>(NE, brows, nbig, boff, toff, tadj, tw, bits, ek, ev);
+        KMP_LAUNCHED("large_gather");
         radix_sort_kv(ek, ev, ektmp, evtmp, NE, rbits + bits);
-        KMP_CUDA(cudaMemcpyAsync(ektmp, ek, NE * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-        KMP_CUDA(cudaMemcpyAsync(evtmp, ev, NE * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+        k_large_place<<<gridN, 256, 0, s>>>(NE, ek, ev, bits, brows, boff, toff, tadj, tw);
+        KMP_LAUNCHED("large_place");
       } else {
-        DBuf<int32_t> hist(X), off(X), cur(X), htot(1);
+        DBuf<int32_t> ek(NE), ev(NE), hist(X), off(X), cur(X), htot(1);
         hist.zero();
         cur.zero();
-        k_seg_hist<<<grid_for(NE, 256), 256, 0, s>>>(NE, ek, bits, hist);
+        k_seg_hist<<<gridN, 256, 0, s>>>(NE, brows, nbig, boff, toff, tadj, hb, hist);
         KMP_LAUNCHED("seg_hist");
         scan_excl_i32(hist, off, X, htot);
-        k_seg_scatter<<<grid_for(NE, 256), 256, 0, s>>>(NE, ek, ev, bits, off, cur, ektmp, evtmp);
+        k_seg_scatter<<<gridN, 256, 0, s>>>(NE, brows, nbig, boff, toff, tadj, tw, hb, off, cur, ek, ev);
         KMP_LAUNCHED("seg_scatter");
-        DBuf<int32_t> slists(2 * X), scnt(2);
-        scnt.zero();
-        k_seg_split<<<grid_for(X, 256), 256, 0, s>>>(X, hist, slists, scnt, X);
-        KMP_LAUNCHED("seg_split");
-        int32_t sc2[2];
-        to_host(sc2, scnt.p, 2);
-        if (sc2[0] > 0) launch_seg_sort<SORT_S, 256>(slists.p, sc2[0], off, hist, ektmp, evtmp);
-        if (sc2[1] > 0) launch_seg_sort<SORT_L, 1024>(slists.p + X, sc2[1], off, hist, ektmp, evtmp);
+        k_seg_place<<<grid_for(X, 1), 256, 0, s>>>(X, hist, off, hb, ek, ev, brows, boff, toff, tadj, tw);
+        KMP_LAUNCHED("seg_place");
       }
-      k_large_place<<<grid_for(NE, 256), 256, 0, s>>>(NE, ektmp, evtmp, bits, brows, boff, toff, tadj, tw);
-      KMP_LAUNCHED("large_place");
     }
   }
   DBuf<int64_t> mtot(1);
