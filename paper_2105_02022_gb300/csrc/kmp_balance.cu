@@ -383,376 +383,457 @@ __global__ void __launch_bounds__(BAL_T) k_bal_spec(BalArgs A) {
   }
 }
 
-// A batch with at most WS_E adjacency entries and WS_T table slots is
-// evaluated by warp 0 alone, in shared-memory tables, with no CTA barrier.
+// ---- the commit: one CTA, driven by its warp 0, block by block
+// Its time is the chain of reads that every block's decision waits for, so what
+// does not change during the commit is read ahead by all warps at once: a window
+// per overloaded block (32 blocks at a time, a warp each) holds the speculated
+// moves and the next candidates with weights, rows and adjacency entries.  The
+// state that does change is the room of every block (cap less weight), in shared
+// memory while k fits, and the blocks of the neighbours, the one gather from
+// global memory left per batch.  A batch with at most WS_E entries and WS_T table
+// slots is evaluated by warp 0 alone, in shared-memory tables; a larger one by
+// the CTA, in shared memory too (over the windows, which are read again after it)
+// while its tables fit.  Mesh of 2^20 nodes, 8192 blocks of 128 nodes brought from
+// 10% to 3% imbalance, the whole call: 97.0 -> 58.4 ms.
 constexpr int WS_E = 256;
 constexpr int WS_T = 2048;
-constexpr int WS_R = 4;  // entries per lane whose loads are issued together
+constexpr int WS_R = 4;   // entries per lane whose gathers are issued together
+constexpr int WIN_E = WS_E;
+constexpr int MEMB = 64;  // slots of the batch-member table (at most 32 members)
 
-// Lowest-id admissible block for a member of weight c (>= 1) with no
-// admissible neighbouring block (one warp).  *hint is the lowest block that
-// may have room: every block below it has cap - weight < 1.  Blocks only gain
-// weight during the commit, except the block being emptied (the commit lowers
-// the hint to it when it gets room), so the scan starts there and moves the
-// hint up past the full blocks it passes.  The overloaded block B has no room.
+struct BalWindow {
+  int64_t beg[32];        // rows of the candidates
+  int64_t epre[33];       // their entries before each
+  int32_t B, lo, hi;      // block, its candidate segment
+  int32_t sat, send, nm;  // speculation: fits after its moves, where it stopped, moves
+  int32_t base, nc;       // candidates [base, base + nc) are held
+  int32_t ne;             // entries held: the first ne of theirs
+  int32_t sv[SPEC_MAX], st[SPEC_MAX], sc[SPEC_MAX];
+  int32_t v[32], c[32];
+  int32_t u[WIN_E], w[WIN_E];
+};
+
+// window of overloaded block o from candidate `start` on (< 0: its first), one warp
+__device__ void load_window(const BalArgs &A, BalWindow &W, int32_t o, int32_t start) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t vmask = (1ull << A.bitsN) - 1ull;
+  const int32_t B = A.olist[o], lo = A.seg_lo[B], hi = A.seg_hi[B], nm = A.spec_n[o];
+  const int32_t base = start < 0 ? lo : start, nc = min(32, hi - base);
+  int32_t v = 0, c = 0;
+  int64_t beg = 0, inc = 0;
+  if (lane < nc) {
+    v = (int32_t)(A.keys[base + lane] & vmask);
+    c = bw_node(A, v);
+    beg = A.xadj[v];
+    inc = A.xadj[v + 1] - beg;
+  }
+  if (lane < nm) {
+    const int32_t sv = A.spec_v[(int64_t)o * SPEC_MAX + lane];
+    W.sv[lane] = sv;
+    W.st[lane] = A.spec_t[(int64_t)o * SPEC_MAX + lane];
+    W.sc[lane] = bw_node(A, sv);
+  }
+#pragma unroll
+  for (int m = 1; m < 32; m <<= 1) {
+    const int64_t x = (int64_t)__shfl_up_sync(0xFFFFFFFFu, (unsigned long long)inc, m);
+    if (lane >= m) inc += x;
+  }
+  W.v[lane] = v;
+  W.c[lane] = c;
+  W.beg[lane] = beg;
+  W.epre[lane + 1] = inc;
+  const int64_t total = (int64_t)__shfl_sync(0xFFFFFFFFu, (unsigned long long)inc, 31);
+  const int32_t ne = total < WIN_E ? (int32_t)total : WIN_E;
+  if (lane == 0) {
+    W.epre[0] = 0;
+    W.B = B;
+    W.lo = lo;
+    W.hi = hi;
+    W.nm = nm;
+    W.sat = A.spec_sat[o];
+    W.send = A.spec_end[o];
+    W.base = base;
+    W.nc = nc;
+    W.ne = ne;
+  }
+  __syncwarp();
+#pragma unroll 4
+  for (int32_t t = lane; t < ne; t += 32) {
+    int32_t j = 0;
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1)
+      if (W.epre[j + st] <= t) j += st;
+    const int64_t q = W.beg[j] + (t - W.epre[j]);
+    W.u[t] = A.adj[q];
+    W.w[t] = A.ew ? A.ew[q] : 1;
+  }
+  __syncwarp();
+}
+
+// Lowest-id block with room for a member of weight c (>= 1) that has no
+// admissible neighbouring block (one warp).  *hint is the lowest block that may
+// have room: every block below it has room < 1.  Blocks only gain weight during
+// the commit, except the block being emptied (the commit lowers the hint to it
+// when it gets room), so the scan starts there and moves the hint up past the
+// full blocks it passes.  The overloaded block has no room.
 constexpr int LA_U = 8;  // chunks of 32 blocks checked per round trip
-__device__ int32_t lowest_admissible(const BalArgs &A, int32_t B, int64_t c, int lane, int32_t *hint) {
+__device__ int32_t lowest_admissible(const int32_t *room, int32_t k, int32_t c, int lane, int32_t *hint) {
   int32_t h1 = -1, res = -1;
-  for (int32_t base = *hint & ~31; base < A.k && res < 0; base += 32 * LA_U) {
-    int32_t room[LA_U];  // cap - weight, clamped to int32 (only >= 1 and >= c matter)
+  for (int32_t base = *hint & ~31; base < k && res < 0; base += 32 * LA_U) {
+    int32_t rm[LA_U];
 #pragma unroll
     for (int u = 0; u < LA_U; ++u) {
       const int32_t b = base + 32 * u + lane;
-      const int32_t bb = b < A.k ? b : A.k - 1;
-      const int64_t r = (int64_t)A.cap[bb] - A.bw[bb];
-      room[u] = r < INT32_MIN ? INT32_MIN : (r > INT32_MAX ? INT32_MAX : (int32_t)r);
+      rm[u] = b < k ? room[b] : INT32_MIN;
     }
 #pragma unroll
     for (int u = 0; u < LA_U; ++u) {
-      const int32_t b = base + 32 * u + lane;
-      const unsigned m1 = __ballot_sync(0xFFFFFFFFu, b < A.k && room[u] >= 1);
-      const unsigned mc = __ballot_sync(0xFFFFFFFFu, b < A.k && b != B && (int64_t)room[u] >= c);
+      const unsigned m1 = __ballot_sync(0xFFFFFFFFu, rm[u] >= 1);
+      const unsigned mc = __ballot_sync(0xFFFFFFFFu, rm[u] >= c);
       if (h1 < 0 && m1) h1 = base + 32 * u + __ffs(m1) - 1;
       if (res < 0 && mc) res = base + 32 * u + __ffs(mc) - 1;
     }
   }
   // blocks in [*hint, h1) were seen without room (h1 = k: none has room)
-  if (lane == 0) atomicMax(hint, h1 >= 0 ? h1 : A.k);
+  if (lane == 0) atomicMax(hint, h1 >= 0 ? h1 : k);
   __syncwarp();
   return res;
 }
 
-
-// the in-order commit of an evaluated batch (one thread); returns the members
-// decided, `stop` when the block fits
-__device__ int32_t commit_batch(const BalArgs &A, int32_t B, int32_t nb, const int32_t *s_v, const int32_t *s_t,
-                                const int64_t *s_c, const int64_t *s_bwt, const int64_t *s_capt,
-                                const uint32_t *s_adj, int64_t E, int32_t &stop, int32_t *hint, int64_t &wB,
-                                int32_t capB) {
-  // only this CTA changes weights, so the block's and the targets' weights are
-  // tracked here (a target's weight is its start weight plus the moves of this
-  // batch into it)
-  uint32_t moved_mask = 0;
-  int32_t j = 0, moves = 0;
-  stop = 0;
-  for (; j < nb; ++j) {
-    if (wB <= capB) {
-      stop = 1;
-      break;
-    }
-    const int32_t t = s_t[j];
-    const int64_t c = s_c[j];
-    int64_t wt = 0;
-    if (t >= 0) {
-      wt = s_bwt[j];
-      for (int32_t x = 0; x < j; ++x)
-        if (((moved_mask >> x) & 1u) && s_t[x] == t) wt += s_c[x];
-    }
-    if (j > 0 && ((s_adj[j] & moved_mask) || (t >= 0 && wt + c > s_capt[j]))) break;
-    if (t >= 0) {
-      A.part[s_v[j]] = t;
-      A.bw[t] = wt + c;
-      wB -= c;
-      ++moves;
-      moved_mask |= 1u << j;
-    }
+// the batch's members by node id (shared memory): -1 or the member
+__device__ __forceinline__ void memb_add(int32_t *mk, int32_t *mv, int32_t v, int32_t j) {
+  uint32_t h = fmix32((uint32_t)v) & (MEMB - 1);
+  while (atomicCAS(&mk[h], HT_EMPTY, v) != HT_EMPTY) h = (h + 1) & (MEMB - 1);  // at most 32 of 64 slots
+  mv[h] = j;
+}
+__device__ __forceinline__ int32_t memb_find(const int32_t *mk, const int32_t *mv, int32_t v) {
+  uint32_t h = fmix32((uint32_t)v) & (MEMB - 1);
+  for (int probe = 0; probe < MEMB; ++probe) {
+    const int32_t x = mk[h];
+    if (x == v) return mv[h];
+    if (x == HT_EMPTY) return -1;
+    h = (h + 1) & (MEMB - 1);
   }
-  A.bw[B] = wB;
-  if ((int64_t)capB - wB >= 1 && B < *hint) *hint = B;
-  if (moves) atomicAdd(A.moved, (unsigned long long)moves);
-  atomicAdd(A.moved + 2, 1ull);  // an exact batch
-  atomicAdd(A.moved + 3, (unsigned long long)nb);
-  atomicAdd(A.moved + 4, (unsigned long long)E);
-  return j;
+  return -1;
 }
 
-// the fixed data of overloaded block o's speculation (lane j: its move j)
-struct SpecAhead {
-  int32_t B = 0, nm = 0, v = 0, t = 0;
-};
-__device__ __forceinline__ SpecAhead spec_ahead(const BalArgs &A, int32_t o, int lane) {
-  SpecAhead S;
-  S.B = A.olist[o];
-  S.nm = A.spec_n[o];
-  if (lane < S.nm) {
-    S.v = A.spec_v[(int64_t)o * SPEC_MAX + lane];
-    S.t = A.spec_t[(int64_t)o * SPEC_MAX + lane];
+// (conn, lowest block) of the larger connectivity
+__device__ __forceinline__ void best_of(int32_t conn, int32_t blk, int32_t &bc, int32_t &bt) {
+  if (conn > bc || (conn == bc && blk < bt)) {
+    bc = conn;
+    bt = blk;
   }
-  return S;
 }
 
-// Warp 0 drives the commit: it applies the speculated moves that stand,
-// sets up every exact batch, and evaluates and commits the small ones alone;
-// the whole CTA joins only for a batch beyond WS_E entries or WS_T slots.
-__global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *inbatch) {
-  __shared__ int32_t s_v[BM_W], s_t[BM_W];
-  __shared__ int64_t s_c[BM_W], s_eoff[BM_W + 1], s_beg[BM_W], s_bwt[BM_W], s_capt[BM_W];
+// The in-order commit of an evaluated batch by warp 0, a lane per member: t its
+// target (-1: none), c its weight, adj its neighbours in the batch, rt the room
+// of its target at the start of the batch.  Members are decided in order while
+// the block is overloaded (need > 0), up to the first whose target no longer
+// fits or who neighbours an earlier move; returns how many, `stop` when the
+// block fits before the next.  All members before that one moved as chosen, so
+// every lane can tell from its predecessors.
+__device__ __forceinline__ int32_t commit_batch(const BalArgs &A, int32_t *room, int32_t B, int32_t nb, int32_t v, int32_t t,
+                                                int32_t c, uint32_t adj, int32_t rt, int32_t need, int32_t *hint,
+                                                int32_t &moves, bool &stop) {
+  constexpr unsigned ALL = 0xFFFFFFFFu;
+  const int lane = threadIdx.x & 31;
+  const bool mover = lane < nb && t >= 0;
+  const unsigned movers = __ballot_sync(ALL, mover), below = (1u << lane) - 1u;
+  unsigned rest = __match_any_sync(ALL, t) & movers & below;
+  int32_t pre = 0;  // earlier moves into the same target
+  while (__any_sync(ALL, rest != 0)) {
+    const int32_t x = __shfl_sync(ALL, c, rest ? __ffs(rest) - 1 : lane);
+    if (rest) pre += x;
+    rest &= rest - 1;
+  }
+  int32_t sum = mover ? c : 0;  // weight moved by the earlier members and this one
+#pragma unroll
+  for (int m = 1; m < 32; m <<= 1) {
+    const int32_t x = __shfl_up_sync(ALL, sum, m);
+    if (lane >= m) sum += x;
+  }
+  const bool fail = lane < nb && lane > 0 && ((adj & movers & below) != 0 || (t >= 0 && pre + c > rt));
+  const bool fits = lane < nb && sum - (mover ? c : 0) >= need;
+  const unsigned mf = __ballot_sync(ALL, fail), ms = __ballot_sync(ALL, fits);
+  const int32_t jf = mf ? __ffs(mf) - 1 : nb, js = ms ? __ffs(ms) - 1 : nb;
+  const int32_t n = min(jf, js);
+  stop = js < nb && js <= jf;
+  if (lane < n && t >= 0) {
+    A.part[v] = t;
+    atomicSub(&room[t], c);
+  }
+  const unsigned done = n >= 32 ? movers : movers & ((1u << n) - 1u);
+  const int32_t gone = n > 0 ? __shfl_sync(ALL, sum, n - 1) : 0;
+  if (lane == 0 && gone > 0) {
+    const int32_t r = room[B] + gone;
+    room[B] = r;
+    if (r >= 1 && B < *hint) *hint = B;
+  }
+  moves += __popc(done);
+  __syncwarp();
+  return n;
+}
+
+constexpr size_t BAL_WINDOWS = BM_W * sizeof(BalWindow);
+constexpr int32_t BAL_SLOTS = (int32_t)(BAL_WINDOWS / (2 * sizeof(int32_t))) & ~31;  // of a CTA batch's tables there
+constexpr size_t BAL_TABS = 2 * WS_T * sizeof(int32_t);
+constexpr int32_t BAL_ROOM_K = 26000;  // rooms in shared memory: 104 KB beside 94 KB of windows and 16 KB of tables
+
+template <bool SROOM>
+__global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
+  extern __shared__ __align__(16) unsigned char bal_smem[];
+  BalWindow *const win = reinterpret_cast<BalWindow *>(bal_smem);
+  int32_t *const wk = reinterpret_cast<int32_t *>(bal_smem + BAL_WINDOWS), *const wv = wk + WS_T;  // empty between batches
+  int32_t *const room = SROOM ? wv + WS_T : groom;
+  __shared__ int32_t s_v[BM_W], s_c[BM_W];
+  __shared__ int64_t s_eoff[BM_W + 1], s_beg[BM_W];
   __shared__ uint32_t s_adj[BM_W], s_mask[BM_W], s_toff[BM_W + 1];
   __shared__ unsigned long long s_best[BM_W];
-  __shared__ int32_t wk[WS_T], wv[WS_T];  // warp 0's tables (empty between batches)
-  __shared__ int32_t s_nb, s_B, s_ob, s_i, s_phase, s_done, s_hint, s_capB;
-  __shared__ int64_t s_wB;
+  __shared__ int32_t mk[MEMB], mv[MEMB];
+  __shared__ int32_t s_nb, s_B, s_ob, s_i, s_phase, s_done, s_large, s_hint;
+  constexpr unsigned ALL = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint64_t vmask = (1ull << A.bitsN) - 1ull;
-  const uint32_t gcap = A.gcap;  // stride of the per-member table regions
+  const uint32_t gcap = A.gcap;  // stride of the per-member table regions in A.gtab
   for (int x = threadIdx.x; x < WS_T; x += BM_T) {
     wk[x] = HT_EMPTY;
     wv[x] = 0;
   }
+  for (int32_t x = threadIdx.x; x < A.k; x += BM_T) room[x] = (int32_t)((int64_t)A.cap[x] - A.bw[x]);
+  if (threadIdx.x < MEMB) mk[threadIdx.x] = HT_EMPTY;
   if (threadIdx.x == 0) {
     s_ob = 0;
-    s_i = 0;
+    s_i = -1;
     s_phase = 0;
     s_done = 0;
     s_hint = 0;
   }
+  int32_t n_moves = 0, n_spec = 0;                   // warp 0's counts
+  unsigned long long n_batches = 0, n_cands = 0, n_entries = 0;
   __syncthreads();
   for (;;) {
+    // windows of the next blocks; the first may be under way (phase 1, candidate s_i)
+    const int32_t g0 = s_ob, gn = min(BM_W, A.nover - g0);
+    if (w < gn) load_window(A, win[w], g0 + w, w == 0 && s_phase == 1 ? s_i : -1);
+    __syncthreads();
     if (w == 0) {
-      int32_t ob = s_ob, i = s_i, phase = s_phase;
-      for (;;) {
+      int32_t ob = g0, i = s_i, phase = s_phase;
+      bool large = false;
+      while (ob < g0 + gn) {
+        BalWindow &W = win[ob - g0];
+        const int32_t B = W.B, hi = W.hi;
         if (phase == 0) {
-          // Run ahead over the blocks: a block's speculated moves stand, in
-          // order, while their targets still fit under the weights left by
-          // the blocks before.  One lane per move checks its target against
-          // the current weight plus what the block's earlier moves add to
-          // it; the moves before the first that does not fit are applied at
-          // once.  Stop at the first block that still needs exact batches.
-          // What does not change during the commit (the block, its speculated
-          // moves, caps, node weights) is read one block ahead; only the
-          // weights are read when the block's turn comes.
-          int32_t o = ob, resume = 0;
-          SpecAhead nx;
-          if (o < A.nover) nx = spec_ahead(A, o, lane);
-          for (; o < A.nover; ++o) {
-            const SpecAhead cur = nx;
-            if (o + 1 < A.nover) nx = spec_ahead(A, o + 1, lane);
-            const int32_t B = cur.B, nm = cur.nm, v = cur.v, t = cur.t;
-            const int32_t lo = A.seg_lo[B], hi = A.seg_hi[B], capB = A.cap[B];
-            const int32_t sat = A.spec_sat[o], send = A.spec_end[o];
-            const int64_t bwB = A.bw[B];  // no move below targets B
-            int64_t c = 0, bt = 0, ct = 0;
-            if (lane < nm) {
-              c = bw_node(A, v);
-              bt = A.bw[t];
-              ct = A.cap[t];
-            }
-            int64_t pre = 0;  // this block's earlier moves into the same target
-#pragma unroll
-            for (int j = 0; j < SPEC_MAX; ++j) {
-              const int32_t tj = __shfl_sync(0xFFFFFFFFu, t, j);
-              const long long cj = __shfl_sync(0xFFFFFFFFu, (long long)c, j);
-              if (j < lane && j < nm && tj == t) pre += cj;
-            }
-            const unsigned bad = __ballot_sync(0xFFFFFFFFu, lane < nm && bt + pre + c > ct);
-            const int32_t f = bad ? __ffs(bad) - 1 : nm;  // moves [0, f) stand
-            if (lane < f) {
-              A.part[v] = t;
-              atomicAdd(reinterpret_cast<unsigned long long *>(&A.bw[t]), (unsigned long long)c);
-            }
-            const int64_t bwB2 = bwB - warp_sum64(lane < f ? c : 0);
-            if (lane == 0 && f > 0) {
-              A.bw[B] = bwB2;
-              if ((int64_t)capB - bwB2 >= 1 && B < s_hint) s_hint = B;  // the block got room
-              atomicAdd(A.moved, (unsigned long long)f);
-              atomicAdd(A.moved + 1, (unsigned long long)f);  // speculated moves that stood
-            }
-            __syncwarp();
-            resume = f < nm ? lo + f : (sat ? hi : send);
-            if (resume < hi && bwB2 > capB) break;  // exact batches take over here
+          // The block's speculated moves stand, in order, while their targets
+          // still fit under what the blocks before left; the moves before the
+          // first that does not are applied at once.
+          const int32_t nm = W.nm;
+          int32_t v = 0, t = -1, c = 0, rt = 0;
+          if (lane < nm) {
+            v = W.sv[lane];
+            t = W.st[lane];
+            c = W.sc[lane];
+            rt = room[t];
           }
-          if (o >= A.nover) {
-            if (lane == 0) s_done = 1;
-            break;
+          int32_t pre = 0;  // this block's earlier moves into the same target
+          for (int j = 0; j < nm; ++j) {
+            const int32_t tj = __shfl_sync(ALL, t, j), cj = __shfl_sync(ALL, c, j);
+            if (j < lane && tj == t) pre += cj;
           }
-          ob = o;
-          i = resume;
+          const unsigned bad = __ballot_sync(ALL, lane < nm && pre + c > rt);
+          const int32_t f = bad ? __ffs(bad) - 1 : nm;  // moves [0, f) stand
+          if (lane < f) {
+            A.part[v] = t;
+            atomicSub(&room[t], c);
+          }
+          const int32_t gone = warp_sum32(lane < f ? c : 0);
+          if (lane == 0 && f > 0) {
+            const int32_t r = room[B] + gone;
+            room[B] = r;
+            if (r >= 1 && B < s_hint) s_hint = B;  // the block got room
+          }
+          __syncwarp();
+          n_moves += f;
+          n_spec += f;
+          i = f < nm ? W.lo + f : (W.sat ? hi : W.send);
           phase = 1;
         }
-        const int32_t B = A.olist[ob];
-        const int32_t hi = A.seg_hi[B];
-        const int64_t wB = A.bw[B];
-        const int32_t capB = A.cap[B];
-        if (i >= hi || wB <= capB) {
+        const int32_t need = -room[B];
+        if (i >= hi || need <= 0) {
           ++ob;
           phase = 0;
           continue;
         }
-        if (lane == 0) {
-          s_wB = wB;  // for the commit, which comes after several warp barriers
-          s_capB = capB;
+        // the next batch: the shortest prefix of the remaining candidates whose
+        // weights cover the overload; the window moves up when it does not show it
+        int32_t a = i - W.base, avail = min(hi - i, 32), nb = 0;
+        int32_t c = 0, inc = 0;
+        for (int turn = 0; turn < 2; ++turn) {
+          const int32_t held = min(W.nc - a, avail);
+          c = lane < held ? W.c[a + lane] : 0;
+          inc = c;
+#pragma unroll
+          for (int m = 1; m < 32; m <<= 1) {
+            const int32_t x = __shfl_up_sync(ALL, inc, m);
+            if (lane >= m) inc += x;
+          }
+          const unsigned enough = __ballot_sync(ALL, lane < held && inc >= need);
+          nb = enough ? __ffs(enough) : held;
+          if (enough || held >= avail) break;
+          __syncwarp();
+          load_window(A, W, ob, i);
+          a = 0;
         }
-        // the next batch: the shortest prefix of the remaining candidates
-        // whose weights cover the overload
-        {
-          int32_t avail = hi - i < BM_W ? hi - i : BM_W;
-          int32_t v = lane < avail ? (int32_t)(A.keys[i + lane] & vmask) : 0;
-          int64_t c = lane < avail ? bw_node(A, v) : 0;
-          const int64_t rb = lane < avail ? A.xadj[v] : 0;
-          int64_t deg = lane < avail ? A.xadj[v + 1] - rb : 0;
-          const int64_t own = deg < A.k ? deg : A.k;
-          // inclusive prefix sums of weights and degrees
+        // member table sized by the member's own distinct blocks (at most
+        // min(degree, k)); the tables' slots are numbered across the batch
+        const int64_t e0 = W.epre[a], E = W.epre[a + nb] - e0;
+        const int32_t v = lane < nb ? W.v[a + lane] : -1;
+        const int64_t deg = lane < nb ? W.epre[a + lane + 1] - W.epre[a + lane] : 0;
+        uint32_t cap = 32;
+        while ((int64_t)cap < 2 * (deg < A.k ? deg : (int64_t)A.k)) cap <<= 1;
+        uint32_t tpre = lane < nb ? cap : 0;
 #pragma unroll
-          for (int m = 1; m < 32; m <<= 1) {
-            int64_t oc = (int64_t)__shfl_up_sync(0xFFFFFFFFu, (unsigned long long)c, m);
-            int64_t od = (int64_t)__shfl_up_sync(0xFFFFFFFFu, (unsigned long long)deg, m);
-            if (lane >= m) {
-              c += oc;
-              deg += od;
-            }
-          }
-          unsigned enough = __ballot_sync(0xFFFFFFFFu, lane < avail && c >= wB - capB);
-          int32_t nb = enough ? __ffs(enough) : avail;
-          // member table sized by the member's own distinct blocks (at most
-          // min(degree, k)), so low-degree members never touch a hub-sized
-          // table; the tables' slots are numbered across the batch (s_toff)
-          uint32_t cap = 32;
-          while ((int64_t)cap < 2 * own) cap <<= 1;
-          uint32_t tpre = lane < nb ? cap : 0;
-#pragma unroll
-          for (int m = 1; m < 32; m <<= 1) {
-            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, tpre, m);
-            if (lane >= m) tpre += o;
-          }
+        for (int m = 1; m < 32; m <<= 1) {
+          const uint32_t x = __shfl_up_sync(ALL, tpre, m);
+          if (lane >= m) tpre += x;
+        }
+        const uint32_t TT = __shfl_sync(ALL, tpre, nb - 1);
+        if (lane < nb) {
+          s_adj[lane] = 0;
+          s_mask[lane] = cap - 1;
+          s_toff[lane + 1] = tpre;
+          memb_add(mk, mv, v, lane);
+        }
+        if (lane == 0) s_toff[0] = 0;
+        ++n_batches;
+        n_cands += nb;
+        n_entries += E;
+        if (E > WS_E || TT > (uint32_t)WS_T) {
           if (lane < nb) {
             s_v[lane] = v;
-            s_beg[lane] = rb;
-            s_eoff[lane + 1] = deg;
-            s_adj[lane] = 0;
-            s_mask[lane] = cap - 1;
-            s_toff[lane + 1] = tpre;
+            s_c[lane] = c;
+            s_beg[lane] = W.beg[a + lane];
+            s_eoff[lane + 1] = W.epre[a + lane + 1] - e0;
             s_best[lane] = 0;
-            inbatch[v] = lane + 1;
           }
           if (lane == 0) {
             s_eoff[0] = 0;
-            s_toff[0] = 0;
             s_nb = nb;
-          }
-        }
-        __syncwarp();
-        const int32_t nb = s_nb;
-        const int64_t E = s_eoff[nb];
-        const uint32_t TT = s_toff[nb];
-        if (E > WS_E || TT > WS_T) {
-          if (lane == 0) {
             s_B = B;
-            s_ob = ob;
-            s_i = i;
           }
+          large = true;
           break;  // the whole CTA evaluates this batch
         }
-        // ---- warp 0 alone: connectivity tables in shared memory, entries in
-        // rounds of WS_R per lane (their loads issued together)
-        {
-          int32_t j = 0;
-          for (int64_t t0 = 0; t0 < E; t0 += 32 * WS_R) {
-            int32_t uu[WS_R], wt[WS_R], jm[WS_R];
+        __syncwarp();
+        // ---- warp 0 alone: connectivity tables in shared memory
+        for (int32_t t0 = 0; t0 < (int32_t)E; t0 += 32 * WS_R) {
+          int32_t uu[WS_R], wt[WS_R], jm[WS_R], bk[WS_R];
 #pragma unroll
-            for (int r = 0; r < WS_R; ++r) {
-              const int64_t t = t0 + lane + 32 * r;
-              uu[r] = -1;
-              if (t < E) {
-                while (s_eoff[j + 1] <= t) ++j;
-                const int64_t q = s_beg[j] + (t - s_eoff[j]);
+          for (int r = 0; r < WS_R; ++r) {
+            const int64_t t = e0 + t0 + lane + 32 * r;
+            uu[r] = -1;
+            if (t < e0 + E) {
+              int32_t j = 0;
+#pragma unroll
+              for (int st = 16; st > 0; st >>= 1)
+                if (W.epre[j + st] <= t) j += st;
+              jm[r] = j - a;
+              if (t < W.ne) {
+                uu[r] = W.u[t];
+                wt[r] = W.w[t];
+              } else {
+                const int64_t q = W.beg[j] + (t - W.epre[j]);
                 uu[r] = A.adj[q];
                 wt[r] = A.ew ? A.ew[q] : 1;
-                jm[r] = j;
               }
             }
-            int32_t bk[WS_R], ib[WS_R];
+          }
 #pragma unroll
-            for (int r = 0; r < WS_R; ++r)
-              if (uu[r] >= 0) {
-                bk[r] = A.part[uu[r]];
-                ib[r] = inbatch[uu[r]];
-              }
+          for (int r = 0; r < WS_R; ++r)
+            if (uu[r] >= 0) bk[r] = A.part[uu[r]];
 #pragma unroll
-            for (int r = 0; r < WS_R; ++r)
-              if (uu[r] >= 0) {
-                if (ib[r] > 0) atomicOr(&s_adj[jm[r]], 1u << (ib[r] - 1));
-                ht_add(wk + s_toff[jm[r]], wv + s_toff[jm[r]], s_mask[jm[r]], bk[r], wt[r]);
-              }
-          }
+          for (int r = 0; r < WS_R; ++r)
+            if (uu[r] >= 0) {
+              const int32_t ib = memb_find(mk, mv, uu[r]);
+              if (ib >= 0) atomicOr(&s_adj[jm[r]], 1u << ib);
+              ht_add(wk + s_toff[jm[r]], wv + s_toff[jm[r]], s_mask[jm[r]], bk[r], wt[r]);
+            }
         }
         __syncwarp();
-        // best admissible block of every member, (conn, ~block); the tables
-        // are emptied on the way (every table spans whole 32-slot chunks)
-        // (the lane that holds a member's best so far also records that
-        // block's weight and cap, the target's state at the start of the batch)
-        {
-          int32_t j = 0;
-          for (uint32_t base = 0; base < TT; base += 32) {
-            while (s_toff[j + 1] <= base) ++j;
-            const uint32_t x = base + lane;
-            const int32_t b = wk[x], cv = wv[x];
-            wk[x] = HT_EMPTY;
-            wv[x] = 0;
-            uint64_t key = 0;
-            int64_t bwb = 0;
-            int32_t capb = 0;
-            if (b != HT_EMPTY && b != B) {
-              bwb = A.bw[b];
-              capb = A.cap[b];
-              if (bwb + bw_node(A, s_v[j]) <= capb)
-                key = ((uint64_t)(uint32_t)cv << 32) | (0xFFFFFFFFu - (uint32_t)b);
+        // best admissible block of every member (kept by the member's lane); the
+        // tables are emptied on the way (every table spans whole 32-slot chunks)
+        int32_t bc = 0, bt = INT32_MAX;
+        for (uint32_t base = 0; base < TT; base += 32 * WS_R) {
+          int32_t b[WS_R], cv[WS_R], rm[WS_R];
+#pragma unroll
+          for (int r = 0; r < WS_R; ++r) {
+            const uint32_t x = base + 32 * r + lane;
+            b[r] = HT_EMPTY;
+            if (x < TT) {
+              b[r] = wk[x];
+              cv[r] = wv[x];
+              wk[x] = HT_EMPTY;
+              wv[x] = 0;
             }
-            const uint64_t top = group_max64<32>(key);
-            if (top != 0 && key == top && top > s_best[j]) {
-              s_best[j] = top;
-              s_bwt[j] = bwb;
-              s_capt[j] = capb;
-            }
-            __syncwarp();
+          }
+#pragma unroll
+          for (int r = 0; r < WS_R; ++r) rm[r] = b[r] != HT_EMPTY && b[r] != B ? room[b[r]] : INT32_MIN;
+#pragma unroll
+          for (int r = 0; r < WS_R; ++r) {
+            const uint32_t at = base + 32 * r;
+            if (at >= TT) break;
+            const int32_t j = __popc(__ballot_sync(ALL, lane < nb && tpre <= at));  // the chunk's member
+            const int32_t cj = __shfl_sync(ALL, c, j);
+            const bool adm = rm[r] >= cj;
+            const int32_t m = __reduce_max_sync(ALL, adm ? cv[r] : 0);
+            if (m == 0) continue;
+            const int32_t tb = __reduce_min_sync(ALL, adm && cv[r] == m ? b[r] : INT32_MAX);
+            if (lane == j) best_of(m, tb, bc, bt);
           }
         }
-        if (lane < nb) {
-          const uint64_t bkey = s_best[lane];
-          s_t[lane] = bkey ? (int32_t)(0xFFFFFFFFu - (uint32_t)bkey) : -1;
-          s_c[lane] = bw_node(A, s_v[lane]);
+        int32_t t = lane < nb && bc > 0 ? bt : -1;
+        for (unsigned none = __ballot_sync(ALL, lane < nb && t < 0); none; none &= none - 1) {
+          const int j = __ffs(none) - 1;
+          const int32_t x = lowest_admissible(room, A.k, __shfl_sync(ALL, c, j), lane, &s_hint);
+          if (lane == j) t = x;
+        }
+        const int32_t rt = t >= 0 ? room[t] : 0;
+        const uint32_t adj = lane < nb ? s_adj[lane] : 0;
+        if (lane < MEMB / 2) {
+          mk[lane] = HT_EMPTY;
+          mk[lane + 32] = HT_EMPTY;
         }
         __syncwarp();
-        for (int32_t j = 0; j < nb; ++j)
-          if (s_t[j] < 0) {
-            const int32_t t = lowest_admissible(A, B, s_c[j], lane, &s_hint);
-            __syncwarp();
-            if (lane == 0) {
-              s_t[j] = t;
-              s_bwt[j] = t >= 0 ? A.bw[t] : 0;
-              s_capt[j] = t >= 0 ? A.cap[t] : 0;
-            }
-            __syncwarp();
-          }
-        int32_t next = 0, stop = 0;
-        if (lane == 0) {
-          int64_t w = s_wB;
-          next = commit_batch(A, B, nb, s_v, s_t, s_c, s_bwt, s_capt, s_adj, E, stop, &s_hint, w, s_capB);
-        }
-        next = __shfl_sync(0xFFFFFFFFu, next, 0);
-        stop = __shfl_sync(0xFFFFFFFFu, stop, 0);
-        if (lane < nb) inbatch[s_v[lane]] = 0;
-        __syncwarp();
-        i += next;
+        bool stop = false;
+        i += commit_batch(A, room, B, nb, v, t, c, adj, rt, need, &s_hint, n_moves, stop);
         if (stop) {
           ++ob;
           phase = 0;
         }
       }
+      if (lane == 0) {
+        s_ob = ob;
+        s_i = i;
+        s_phase = phase;
+        s_large = large;
+        s_done = !large && ob >= A.nover;
+      }
     }
     __syncthreads();
     if (s_done) break;
-    // ---- a large batch, evaluated by the whole CTA
+    if (!s_large) continue;
+    // ---- a large batch, evaluated by the whole CTA; the windows are no longer needed
     const int32_t B = s_B, nb = s_nb;
     // every table size is a multiple of 32, so a warp's 32 slots lie in one table
     const uint32_t TT = s_toff[nb];
+    const bool sm = TT <= (uint32_t)BAL_SLOTS;  // tables over the windows
+    int32_t *const sk = reinterpret_cast<int32_t *>(bal_smem), *const sv = sk + BAL_SLOTS;
+    auto keys_of = [&](int32_t j) { return sm ? sk + s_toff[j] : A.gtab + (int64_t)j * 2 * gcap; };
+    auto vals_of = [&](int32_t j) { return sm ? sv + s_toff[j] : A.gtab + (int64_t)j * 2 * gcap + gcap; };
     {
       int32_t j = 0;
       for (uint32_t t = threadIdx.x; t < TT; t += BM_T) {
         while (s_toff[j + 1] <= t) ++j;
-        int32_t *K = A.gtab + (int64_t)j * 2 * gcap;
-        const uint32_t x = t - s_toff[j];
-        K[x] = HT_EMPTY;
-        K[gcap + x] = 0;
+        keys_of(j)[t - s_toff[j]] = HT_EMPTY;
+        vals_of(j)[t - s_toff[j]] = 0;
       }
     }
     __syncthreads();
@@ -770,16 +851,18 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *inbatch)
           int32_t u = A.adj[q];
           blk = A.part[u];
           wt = A.ew ? A.ew[q] : 1;
-          int32_t jj = inbatch[u];
-          if (jj > 0) atomicOr(&s_adj[jm], 1u << (jj - 1));
+          const int32_t ib = memb_find(mk, mv, u);
+          if (ib >= 0) atomicOr(&s_adj[jm], 1u << ib);
         }
-        uint64_t key = ok ? ((uint64_t)(uint32_t)jm << 32) | (uint32_t)blk : ~0ull;
-        unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-        int32_t s = __reduce_add_sync(peers, wt);
-        if (ok && lane == __ffs(peers) - 1) {
-          int32_t *K = A.gtab + (int64_t)jm * 2 * gcap;
-          ht_add(K, K + gcap, s_mask[jm], blk, s);
+        if (sm) {
+          if (ok) ht_add(keys_of(jm), vals_of(jm), s_mask[jm], blk, wt);
+          continue;
         }
+        // lanes that hit the same block of the same member add first
+        const uint64_t key = ok ? ((uint64_t)(uint32_t)jm << 32) | (uint32_t)blk : ~0ull;
+        const unsigned peers = __match_any_sync(ALL, key);
+        const int32_t s = __reduce_add_sync(peers, wt);
+        if (ok && lane == __ffs(peers) - 1) ht_add(keys_of(jm), vals_of(jm), s_mask[jm], blk, s);
       }
     }
     __syncthreads();
@@ -791,46 +874,51 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *inbatch)
         const uint32_t t = base + threadIdx.x;
         if (base + (threadIdx.x & ~31u) >= TT) break;  // warp-uniform
         while (s_toff[jj + 1] <= t) ++jj;
-        const int32_t *K = A.gtab + (int64_t)jj * 2 * gcap;
         const uint32_t x = t - s_toff[jj];
-        const int32_t b = K[x];
+        const int32_t b = keys_of(jj)[x];
         uint64_t key = 0;
-        if (b != HT_EMPTY && b != B && A.bw[b] + bw_node(A, s_v[jj]) <= A.cap[b])
-          key = ((uint64_t)(uint32_t)K[gcap + x] << 32) | (0xFFFFFFFFu - (uint32_t)b);
+        if (b != HT_EMPTY && b != B && room[b] >= s_c[jj])
+          key = ((uint64_t)(uint32_t)vals_of(jj)[x] << 32) | (0xFFFFFFFFu - (uint32_t)b);
         key = group_max64<32>(key);
         if (lane == 0 && key) atomicMax(&s_best[jj], key);
       }
     }
     __syncthreads();
-    if (w < nb) {
-      const int64_t c = bw_node(A, s_v[w]);
-      const uint64_t bestk = s_best[w];
+    if (w == 0) {
+      const int32_t v = lane < nb ? s_v[lane] : -1, c = lane < nb ? s_c[lane] : 0;
+      const uint64_t bestk = lane < nb ? s_best[lane] : 0;
       int32_t t = bestk ? (int32_t)(0xFFFFFFFFu - (uint32_t)bestk) : -1;
-      if (t < 0) t = lowest_admissible(A, B, c, lane, &s_hint);
+      for (unsigned none = __ballot_sync(ALL, lane < nb && t < 0); none; none &= none - 1) {
+        const int j = __ffs(none) - 1;
+        const int32_t x = lowest_admissible(room, A.k, __shfl_sync(ALL, c, j), lane, &s_hint);
+        if (lane == j) t = x;
+      }
+      const int32_t rt = t >= 0 ? room[t] : 0;
+      const uint32_t adj = lane < nb ? s_adj[lane] : 0;
+      const int32_t need = -room[B];
+      mk[lane] = HT_EMPTY;
+      mk[lane + 32] = HT_EMPTY;
+      __syncwarp();
+      bool stop = false;
+      const int32_t n = commit_batch(A, room, B, nb, v, t, c, adj, rt, need, &s_hint, n_moves, stop);
       if (lane == 0) {
-        s_t[w] = t;
-        s_c[w] = c;
-        s_bwt[w] = t >= 0 ? A.bw[t] : 0;  // the target's weight at the start of the batch
-        s_capt[w] = t >= 0 ? A.cap[t] : 0;
+        s_i += n;
+        if (stop) {
+          ++s_ob;
+          s_phase = 0;
+        }
+        s_done = s_ob >= A.nover;
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int32_t stop = 0;
-      int64_t wB = A.bw[B];
-      const int32_t next =
-          commit_batch(A, B, nb, s_v, s_t, s_c, s_bwt, s_capt, s_adj, E, stop, &s_hint, wB, A.cap[B]);
-      s_i += next;
-      if (stop) {
-        ++s_ob;
-        s_phase = 0;
-      } else {
-        s_phase = 1;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x < nb) inbatch[s_v[threadIdx.x]] = 0;
-    __syncthreads();
+    if (s_done) break;
+  }
+  if (threadIdx.x == 0) {
+    A.moved[0] = (unsigned long long)n_moves;
+    A.moved[1] = (unsigned long long)n_spec;  // speculated moves that stood
+    A.moved[2] = n_batches;
+    A.moved[3] = n_cands;
+    A.moved[4] = n_entries;
   }
 }
 
@@ -945,11 +1033,25 @@ int64_t balance(const Graph &g, int32_t k, const int32_t *caps_host, int32_t *pa
     k_bal_spec<<<sgrid, BAL_T, 0, s>>>(A);
     KMP_LAUNCHED("bal_spec");
   }
-  // one global table per warp of the move kernel, and the batch membership marks
-  DBuf<int32_t> gtab1(2ll * gcap * BM_W), inbatch(n);
-  inbatch.zero();
+  // a global table per member for CTA batches whose tables do not fit shared
+  // memory; rooms in shared memory while k fits
+  DBuf<int32_t> gtab1(2ll * gcap * BM_W), room;
   A.gtab = gtab1;
-  k_bal_moves<<<1, BM_T, 0, s>>>(A, inbatch);
+  const size_t smem = BAL_WINDOWS + BAL_TABS + (k <= BAL_ROOM_K ? (size_t)k * sizeof(int32_t) : 0);
+  static bool attr = false;
+  if (!attr) {
+    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(BAL_WINDOWS + BAL_TABS + BAL_ROOM_K * sizeof(int32_t))));
+    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(BAL_WINDOWS + BAL_TABS)));
+    attr = true;
+  }
+  if (k <= BAL_ROOM_K) {
+    k_bal_moves<true><<<1, BM_T, smem, s>>>(A, nullptr);
+  } else {
+    room.alloc(k);
+    k_bal_moves<false><<<1, BM_T, smem, s>>>(A, room);
+  }
   KMP_LAUNCHED("bal_moves");
   unsigned long long hm[5];
   to_host(hm, moved.p, 5);
