@@ -1768,10 +1768,17 @@ __global__ void k_block_keys(int32_t n, const int32_t *part, int bits, uint64_t 
     keys[v] = ((uint64_t)(uint32_t)part[v] << bits) | (uint64_t)v;
 }
 
-__global__ void k_block_stats(int32_t n, const int64_t *xadj, const int32_t *adj, const int32_t *vw,
-                              const int32_t *part, const uint64_t *keys, uint64_t mask, int32_t *members,
-                              int32_t *bcount, unsigned long long *bweight, int32_t *ideg,
-                              unsigned long long *becount) {
+// Rows above EXT_BIG entries are listed and taken by a CTA each (k_*_big): on one
+// warp a hub's row of 10^5 entries outlasted the rest of the kernel (both kernels
+// over all rounds of R-MAT 2^22, k = 2^12: 33.6 ms).  Shorter rows stay on a warp,
+// with the gathers of EXT_U chunks in flight.
+constexpr int64_t EXT_BIG = 2048;
+constexpr int EXT_U = 4;
+__global__ void k_block_stats(int32_t n, const int64_t *__restrict__ xadj, const int32_t *__restrict__ adj,
+                              const int32_t *__restrict__ vw, const int32_t *__restrict__ part,
+                              const uint64_t *__restrict__ keys, uint64_t mask, int32_t *members, int32_t *bcount,
+                              unsigned long long *bweight, int32_t *ideg, unsigned long long *becount, int32_t *big,
+                              int32_t *nbig) {
   // a warp takes 32 consecutive positions and walks their rows one by one
   int lane = threadIdx.x & 31;
   int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1779,17 +1786,33 @@ __global__ void k_block_stats(int32_t n, const int64_t *xadj, const int32_t *adj
   for (int64_t base = gw * 32; base < n; base += nw * 32) {
     int64_t i = base + lane;
     int32_t v = -1, b = -1;
+    int64_t rb = 0, re = 0;
     if (i < n) {
       v = (int32_t)(keys[i] & mask);
       members[i] = v;
       b = part[v];
+      rb = xadj[v];
+      re = xadj[v + 1];
+      if (re - rb > EXT_BIG) {
+        big[atomicAdd(nbig, 1)] = (int32_t)i;
+        re = rb;
+      }
     }
     int32_t myd = 0;
     int jmax = (int)(n - base < 32 ? n - base : 32);
     for (int j = 0; j < jmax; ++j) {
-      int32_t vj = __shfl_sync(0xFFFFFFFFu, v, j), bj = __shfl_sync(0xFFFFFFFFu, b, j);
+      const int32_t bj = __shfl_sync(0xFFFFFFFFu, b, j);
+      const int64_t q0 = (int64_t)__shfl_sync(0xFFFFFFFFu, (unsigned long long)rb, j);
+      const int64_t q1 = (int64_t)__shfl_sync(0xFFFFFFFFu, (unsigned long long)re, j);
       int32_t d = 0;
-      for (int64_t q = xadj[vj] + lane; q < xadj[vj + 1]; q += 32) d += (part[adj[q]] == bj);
+      for (int64_t q = q0 + lane; q < q1; q += 32 * EXT_U) {
+        int32_t u[EXT_U];
+#pragma unroll
+        for (int r = 0; r < EXT_U; ++r) u[r] = q + 32 * r < q1 ? adj[q + 32 * r] : -1;
+#pragma unroll
+        for (int r = 0; r < EXT_U; ++r)
+          if (u[r] >= 0) d += (part[u[r]] == bj);
+      }
       d = warp_sum32(d);
       if (lane == j) myd = d;
     }
@@ -1797,8 +1820,31 @@ __global__ void k_block_stats(int32_t n, const int64_t *xadj, const int32_t *adj
       atomicAdd(&bcount[b], 1);
       atomicAdd(&bweight[b], (unsigned long long)(vw ? vw[v] : 1));
       ideg[i] = myd;
-      atomicAdd(&becount[b], (unsigned long long)myd);
+      if (myd) atomicAdd(&becount[b], (unsigned long long)myd);
     }
+  }
+}
+__global__ void __launch_bounds__(256) k_block_stats_big(const int32_t *big, const int32_t *nbig, const int64_t *xadj,
+                                                         const int32_t *adj, const int32_t *part, const int32_t *members,
+                                                         int32_t *ideg, unsigned long long *becount) {
+  __shared__ int32_t s_d;
+  const int32_t nb = *nbig;
+  for (int32_t x = blockIdx.x; x < nb; x += gridDim.x) {
+    const int32_t i = big[x], v = members[i], b = part[v];
+    if (threadIdx.x == 0) s_d = 0;
+    __syncthreads();
+    int32_t d = 0;
+    const int64_t e = xadj[v + 1];
+#pragma unroll 4
+    for (int64_t q = xadj[v] + threadIdx.x; q < e; q += 256) d += (part[adj[q]] == b);
+    d = warp_sum32(d);
+    if ((threadIdx.x & 31) == 0 && d) atomicAdd(&s_d, d);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      ideg[i] = s_d;
+      atomicAdd(&becount[b], (unsigned long long)s_d);
+    }
+    __syncthreads();
   }
 }
 
@@ -1811,10 +1857,11 @@ __global__ void k_local_ids(int32_t n, const int32_t *members, const int32_t *pa
   }
 }
 
-__global__ void k_fill_sub(int32_t n, const int64_t *xadj, const int32_t *adj, const int32_t *vw,
-                           const int32_t *ew, const int32_t *part, const int32_t *members,
-                           const int32_t *loc, const int64_t *gx, uint16_t *sadj, int32_t *sew,
-                           int32_t *svw) {
+__global__ void k_fill_sub(int32_t n, const int64_t *__restrict__ xadj, const int32_t *__restrict__ adj,
+                           const int32_t *__restrict__ vw, const int32_t *__restrict__ ew,
+                           const int32_t *__restrict__ part, const int32_t *__restrict__ members,
+                           const int32_t *__restrict__ loc, const int64_t *__restrict__ gx,
+                           uint16_t *__restrict__ sadj, int32_t *__restrict__ sew, int32_t *__restrict__ svw) {
   // a warp per row, order-preserving compaction of the entries inside the block
   int lane = threadIdx.x & 31;
   int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1824,21 +1871,70 @@ __global__ void k_fill_sub(int32_t n, const int64_t *xadj, const int32_t *adj, c
     int32_t b = part[v];
     if (lane == 0) svw[i] = vw ? vw[v] : 1;
     int64_t o = gx[i];
-    for (int64_t q0 = xadj[v]; q0 < xadj[v + 1]; q0 += 32) {
-      int64_t q = q0 + lane;
-      bool keep = false;
-      int32_t u = 0;
-      if (q < xadj[v + 1]) {
-        u = adj[q];
-        keep = part[u] == b;
+    const int64_t rb = xadj[v], re = xadj[v + 1];
+    if (re - rb > EXT_BIG) continue;  // k_fill_sub_big
+    for (int64_t q0 = rb; q0 < re; q0 += 32 * EXT_U) {
+      int32_t u[EXT_U], pu[EXT_U];
+#pragma unroll
+      for (int r = 0; r < EXT_U; ++r) u[r] = q0 + 32 * r + lane < re ? adj[q0 + 32 * r + lane] : -1;
+#pragma unroll
+      for (int r = 0; r < EXT_U; ++r) pu[r] = u[r] >= 0 ? part[u[r]] : -1;
+#pragma unroll
+      for (int r = 0; r < EXT_U; ++r) {
+        const bool keep = pu[r] == b;
+        const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
+        if (keep) {
+          const int64_t p = o + __popc(bal & ((1u << lane) - 1u));
+          sadj[p] = (uint16_t)loc[u[r]];
+          if (ew) sew[p] = ew[q0 + 32 * r + lane];
+        }
+        o += __popc(bal);
       }
-      unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
-      if (keep) {
-        int64_t p = o + __popc(bal & ((1u << lane) - 1u));
-        sadj[p] = (uint16_t)loc[u];
-        if (ew) sew[p] = ew[q];
+    }
+  }
+}
+__global__ void __launch_bounds__(256) k_fill_sub_big(const int32_t *big, const int32_t *nbig, const int64_t *xadj,
+                                                      const int32_t *adj, const int32_t *ew, const int32_t *part,
+                                                      const int32_t *members, const int32_t *loc, const int64_t *gx,
+                                                      uint16_t *sadj, int32_t *sew) {
+  __shared__ int32_t s_cnt[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int32_t nb = *nbig;
+  for (int32_t x = blockIdx.x; x < nb; x += gridDim.x) {
+    const int32_t i = big[x], v = members[i], b = part[v];
+    int64_t o = gx[i];
+    const int64_t re = xadj[v + 1];
+    for (int64_t t0 = xadj[v]; t0 < re; t0 += 256 * EXT_U) {  // a tile: EXT_U chunks of 32 a warp, in order
+      const int64_t q0 = t0 + 32 * EXT_U * w;
+      int32_t u[EXT_U];
+      unsigned bal[EXT_U];
+      int32_t cnt = 0;
+#pragma unroll
+      for (int r = 0; r < EXT_U; ++r) u[r] = q0 + 32 * r + lane < re ? adj[q0 + 32 * r + lane] : -1;
+#pragma unroll
+      for (int r = 0; r < EXT_U; ++r) {
+        bal[r] = __ballot_sync(0xFFFFFFFFu, u[r] >= 0 && part[u[r]] == b);
+        cnt += __popc(bal[r]);
       }
-      o += __popc(bal);
+      if (lane == 0) s_cnt[w] = cnt;
+      __syncthreads();
+      int64_t p = o;
+      int32_t tot = 0;
+      for (int y = 0; y < 8; ++y) {
+        if (y < w) p += s_cnt[y];
+        tot += s_cnt[y];
+      }
+#pragma unroll
+      for (int r = 0; r < EXT_U; ++r) {
+        if ((bal[r] >> lane) & 1u) {
+          const int64_t at = p + __popc(bal[r] & ((1u << lane) - 1u));
+          sadj[at] = (uint16_t)loc[u[r]];
+          if (ew) sew[at] = ew[q0 + 32 * r + lane];
+        }
+        p += __popc(bal[r]);
+      }
+      o += tot;
+      __syncthreads();  // the next tile rewrites the counts
     }
   }
 }
@@ -1902,9 +1998,17 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
   bcount.zero();
   bweight.zero();
   becount.zero();
+  DBuf<int32_t> big, nbig(1);
+  big.alloc(g.m / (EXT_BIG + 1) + 1);  // at most so many rows above EXT_BIG entries
+  nbig.zero();
+  const int grid_big = C.sms * 8;
   k_block_stats<<<grid, 256, 0, s>>>(n, g.xadj, g.adj, g.vw, part, keys, (1ull << bitsN) - 1ull, members,
-                                     bcount, bweight, ideg, becount);
+                                     bcount, bweight, ideg, becount, big, nbig);
   KMP_LAUNCHED("block_stats");
+  if (g.maxdeg > EXT_BIG) {
+    k_block_stats_big<<<grid_big, 256, 0, s>>>(big, nbig, g.xadj, g.adj, part, members, ideg, becount);
+    KMP_LAUNCHED("block_stats_big");
+  }
   scan_excl_i32(bcount, boff, nblocks + 1, nullptr);
   k_local_ids<<<grid, 256, 0, s>>>(n, members, part, boff, loc);
   KMP_LAUNCHED("local_ids");
@@ -1918,6 +2022,10 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
   if (g.ew) sew.alloc(E);
   k_fill_sub<<<grid, 256, 0, s>>>(n, g.xadj, g.adj, g.vw, g.ew, part, members, loc, gx, sadj, sew.p, svw);
   KMP_LAUNCHED("fill_sub");
+  if (g.maxdeg > EXT_BIG) {
+    k_fill_sub_big<<<grid_big, 256, 0, s>>>(big, nbig, g.xadj, g.adj, g.ew, part, members, loc, gx, sadj, sew.p);
+    KMP_LAUNCHED("fill_sub_big");
+  }
   std::vector<int32_t> hcount(nblocks + 1), hoff(nblocks + 1);
   std::vector<unsigned long long> hw(nblocks), he(nblocks);
   to_host(hcount.data(), bcount.p, nblocks);
