@@ -596,13 +596,12 @@ int kmp_cut(const kmp_graph *g, const kmp_vid *part, int32_t k, int64_t *cut_out
   return guarded([&] {
     if (!g || !part) fail(KMP_ERR_ARG, "NULL argument");
     if (k < 1) fail(KMP_ERR_ARG, "k < 1");
-    check_range(g->g.n, part, 0, k, "part");
-    DBuf<int64_t> bw(k), cut(1);
-    cut_and_weights(g->g, part, k, bw, cut);
-    if (bw_out) to_host(bw_out, bw.p, k);
-    int64_t c = read1(cut.p);
-    sync_and_check("cut");
-    if (cut_out) *cut_out = c;
+    std::vector<int64_t> r;
+    cut_to_host(g->g, part, k, r);
+    if (r[k + 2]) sync_and_check("cut");  // clears the word and reports it
+    if (r[k + 1]) fail(KMP_ERR_ARG, "part: value out of range");
+    if (bw_out) memcpy(bw_out, r.data(), (size_t)k * sizeof(int64_t));
+    if (cut_out) *cut_out = r[k];
   });
 }
 
