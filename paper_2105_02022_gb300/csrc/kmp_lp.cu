@@ -92,6 +92,7 @@ struct LPArgs {
   // are hashed by label into buckets of about hub_bucket entries, scattered
   // into bucket order and aggregated one bucket per warp in shared memory
   const int32_t *hubs;         // hub node ids, ascending
+  const int32_t *hpos;         // per node, its index among them (when it is one)
   int32_t nhubs;
   unsigned long long *hkc;     // best admissible key per hub
   unsigned long long *hku;     // best key per hub
@@ -535,8 +536,6 @@ __device__ void rate_cta(const LPArgs &A, int32_t u, int32_t pos, int32_t *keys,
   __syncthreads();
 }
 
-__device__ __forceinline__ int32_t hub_index(const LPArgs &A, int32_t u);
-
 __global__ void __launch_bounds__(RATE_T, 6) k_rate(LPArgs A, int s) {
   __shared__ int32_t tkeys[CTA_TAB];
   __shared__ int32_t tvals[CTA_TAB];
@@ -611,16 +610,6 @@ __device__ __forceinline__ void stamp_stage_end(const LPArgs &A, int s) {
 
 // ---- hubs (bin 6) with many labels: insert / reduce / emit
 
-__device__ __forceinline__ int32_t hub_index(const LPArgs &A, int32_t u) {
-  int32_t lo = 0, hi = A.nhubs - 1;
-  while (lo < hi) {
-    int32_t mid = (lo + hi) >> 1;
-    if (A.hubs[mid] < u) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
-
 __device__ __forceinline__ int32_t find_seg(const int64_t *off, int32_t cnt, int64_t x) {
   int32_t lo = 0, hi = cnt - 1;  // last index with off[idx] <= x
   while (lo < hi) {
@@ -656,7 +645,7 @@ __global__ void __launch_bounds__(1024) k_hub_plan(LPArgs A, int s) {
     int32_t h = 0;
     if (i < cnt) {
       int32_t u = A.vlist[lo + i];
-      h = A.hubs ? hub_index(A, u) : i;
+      h = A.hubs ? A.hpos[u] : i;
       int64_t deg = A.xadj[u + 1] - A.xadj[u];
       ne = ceil_div(deg, A.hub_chunk);
       nx = deg;
@@ -1033,7 +1022,7 @@ __global__ void __launch_bounds__(256) k_hub_emit(LPArgs A, int s) {
   for (int64_t p = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < hi;
        p += (int64_t)gridDim.x * blockDim.x) {
     int32_t u = A.vlist[p];
-    int32_t h = hub_index(A, u);
+    int32_t h = A.hpos[u];
     uint64_t kc = A.hkc[h], ku = A.hku[h];
     int32_t rown = A.hrown[h];
     emit(A, u, (int32_t)p, rown, kc, kc ? label_of_key(rkh(A), kc) : -1, ku,
@@ -1167,10 +1156,8 @@ __global__ void k_hub_list(int32_t n, const int64_t *xadj, const uint8_t *flag, 
 }
 
 // ------------------------------------------------------------------- commit
-__global__ void __launch_bounds__(256) k_classify(LPArgs A, int s) {
-  int32_t lo = A.boff[s * NB], hi = A.boff[(s + 1) * NB];
-  for (int64_t pos = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pos < hi;
-       pos += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void classify_range(const LPArgs &A, int64_t first, int64_t hi, int64_t step) {
+  for (int64_t pos = first; pos < hi; pos += step) {
     int32_t T = A.prop_t[pos];
     if (T < 0) continue;
     const unsigned long long sc = A.tgt[T].sumcnt;
@@ -1190,11 +1177,8 @@ __global__ void __launch_bounds__(256) k_classify(LPArgs A, int s) {
   }
 }
 
-__global__ void __launch_bounds__(256) k_bucket(LPArgs A, int s) {
-  if (A.ctr[0] == 0) return;
-  int32_t lo = A.boff[s * NB], hi = A.boff[(s + 1) * NB];
-  for (int64_t pos = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pos < hi;
-       pos += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void bucket_range(const LPArgs &A, int64_t first, int64_t hi, int64_t step) {
+  for (int64_t pos = first; pos < hi; pos += step) {
     int32_t T = A.prop_t[pos];
     if (T < 0 || A.acc[pos]) continue;
     int32_t sl = A.tgt[T].slot;
@@ -1202,16 +1186,26 @@ __global__ void __launch_bounds__(256) k_bucket(LPArgs A, int s) {
   }
 }
 
+__global__ void __launch_bounds__(256) k_classify(LPArgs A, int s) {
+  classify_range(A, A.boff[s * NB] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x, A.boff[(s + 1) * NB],
+                 (int64_t)gridDim.x * blockDim.x);
+}
+
+__global__ void __launch_bounds__(256) k_bucket(LPArgs A, int s) {
+  if (A.ctr[0] == 0) return;
+  bucket_range(A, A.boff[s * NB] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x, A.boff[(s + 1) * NB],
+               (int64_t)gridDim.x * blockDim.x);
+}
+
 __device__ __forceinline__ uint64_t commit_key(const LPArgs &A, int32_t pos) {
   return ((uint64_t)(uint32_t)(0x7FFFFFFF - A.prop_g[pos]) << 32) | (uint32_t)A.vlist[pos];
 }
 
-__global__ void __launch_bounds__(256) k_resolve(LPArgs A) {
-  int32_t nslots = A.ctr[0];
-  if (nslots == 0) return;
+// by block `block` of `blocks` (all its threads)
+__device__ void resolve_slots(const LPArgs &A, int32_t nslots, int32_t block, int32_t blocks) {
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t gw = (int64_t)blockIdx.x * (blockDim.x / 32) + w;
-  int64_t nw = (int64_t)gridDim.x * (blockDim.x / 32);
+  int64_t gw = (int64_t)block * (blockDim.x / 32) + w;
+  int64_t nw = (int64_t)blocks * (blockDim.x / 32);
   // small contested targets: one warp each
   for (int64_t sl = gw; sl < nslots; sl += nw) {
     int32_t T = A.slot_t[sl];
@@ -1238,7 +1232,7 @@ __global__ void __launch_bounds__(256) k_resolve(LPArgs A) {
   __shared__ unsigned long long hist[256];
   __shared__ uint64_t prefix;
   __shared__ long long accw;
-  for (int64_t sl = blockIdx.x; sl < nslots; sl += gridDim.x) {
+  for (int64_t sl = block; sl < nslots; sl += blocks) {
     int32_t T = A.slot_t[sl];
     int32_t cnt = (int32_t)(A.tgt[T].sumcnt >> 32);
     if (cnt <= 32) continue;
@@ -1325,6 +1319,11 @@ __global__ void __launch_bounds__(256) k_resolve(LPArgs A) {
   }
 }
 
+__global__ void __launch_bounds__(256) k_resolve(LPArgs A) {
+  const int32_t nslots = A.ctr[0];
+  if (nslots > 0) resolve_slots(A, nslots, blockIdx.x, gridDim.x);
+}
+
 // A warp takes 32 list entries.  The rows of its moved nodes (up to APPLY_ROW
 // entries each) are walked together, an entry per lane: the entry's owner comes
 // from a prefix sum of the row lengths, so consecutive lanes read consecutive
@@ -1333,14 +1332,13 @@ __global__ void __launch_bounds__(256) k_resolve(LPArgs A) {
 // weights.  Partition of a 2^24-node mesh, degree 16, k = 2^14, all k_apply
 // launches: 16.6 -> 13.3 ms.
 constexpr int APPLY_ROW = 256;
-__global__ void __launch_bounds__(256) k_apply(LPArgs A, int s) {
-  const int32_t lo = A.boff[s * NB], hi = A.boff[(s + 1) * NB];
+// first: the list entry of the warp's lane 0
+__device__ __forceinline__ void apply_range(const LPArgs &A, int64_t first, int64_t hi, int64_t stride) {
   uint8_t *__restrict__ nxt = act_nxt(A);
   const int32_t *__restrict__ adj = A.adj;
   const int lane = threadIdx.x & 31;
   unsigned moved = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t p0 = lo + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); p0 < hi; p0 += stride) {
+  for (int64_t p0 = first; p0 < hi; p0 += stride) {
     const int64_t pos = p0 + lane;
     const int32_t T = pos < hi ? A.prop_t[pos] : -1;
     int32_t deg = 0;
@@ -1386,6 +1384,11 @@ __global__ void __launch_bounds__(256) k_apply(LPArgs A, int s) {
   if (lane == 0 && moved) atomicAdd(&ctr_cur(A)[1], (unsigned long long)moved);
 }
 
+__global__ void __launch_bounds__(256) k_apply(LPArgs A, int s) {
+  apply_range(A, A.boff[s * NB] + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31), A.boff[(s + 1) * NB],
+              (int64_t)gridDim.x * blockDim.x);
+}
+
 // neighbours of high-degree nodes that moved become active: one block per
 // node, four entries a thread in flight
 __global__ void __launch_bounds__(256) k_scatter_big(LPArgs A) {
@@ -1410,6 +1413,104 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     p[i] = v;
+}
+
+// A whole LP run of a small graph by one CTA: every round and sub-round, a barrier
+// between the steps that are kernels otherwise.  On a graph of a few thousand
+// nodes a sub-round's five launches take 18 us whatever they do, and each run
+// captures and instantiates its graph of launches first.  Rows have at most 256
+// entries (a warp's table each), and n at most SMALL_N: four nodes a thread, a few
+// dependent reads a sub-round on one SM.  Partition of a 32,768-node mesh, whose
+// four coarse levels run here: 9.6 -> 6.9 ms.  The order of the node list inside a
+// (sub-round, bin) is arbitrary here; nothing depends on it.
+constexpr int32_t SMALL_N = 4096;
+constexpr int64_t SMALL_DEG = 256;
+constexpr int SMALL_T = 1024;
+constexpr size_t SMALL_SMEM = (size_t)(SMALL_T / 32) * (2 * WARP_TAB * sizeof(int32_t) + WARP_TAB / 2 * sizeof(uint16_t));
+__global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *rounds, int32_t nrounds) {
+  extern __shared__ __align__(16) unsigned char lps_smem[];
+  constexpr int W = SMALL_T / 32;
+  __shared__ int32_t cnt[8 * NB + 1], fill[8 * NB];
+  __shared__ unsigned long long s_scan;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int32_t *keys = reinterpret_cast<int32_t *>(lps_smem) + w * WARP_TAB;
+  int32_t *vals = reinterpret_cast<int32_t *>(lps_smem) + (W + w) * WARP_TAB;
+  uint16_t *list = reinterpret_cast<uint16_t *>(lps_smem + (size_t)W * 2 * WARP_TAB * sizeof(int32_t)) + w * (WARP_TAB / 2);
+  for (int x = lane; x < WARP_TAB; x += 32) {
+    keys[x] = HT_EMPTY;
+    vals[x] = 0;
+  }
+  const int nk = A.S * NB;
+  for (int32_t r = 0; r < nrounds; ++r) {
+    A.R = rounds + r;  // written before the launch: its values may be read through the read-only path
+    const uint64_t rk = rkey(A);
+    uint8_t *act = act_cur(A);
+    volatile unsigned long long *ctr = ctr_cur(A);
+    for (int i = threadIdx.x; i < nk; i += SMALL_T) fill[i] = 0;
+    if (threadIdx.x == 0) s_scan = 0;
+    __syncthreads();
+    // binning: counts, offsets, list; consumes act
+    for (int pass = 0; pass < 2; ++pass) {
+      unsigned long long my = 0;
+      for (int32_t v = threadIdx.x; v < A.n; v += SMALL_T) {
+        if (!act[v]) continue;
+        const int64_t d = A.xadj[v + 1] - A.xadj[v];
+        if (pass == 1) act[v] = 0;
+        if (d == 0) continue;
+        const int key = (int)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1)) * NB + deg_bin(d, A.huge_deg);
+        const int32_t at = atomicAdd(&fill[key], 1);
+        if (pass == 1) A.vlist[cnt[key] + at] = v;
+        my += (unsigned long long)d;
+      }
+      if (pass == 0 && my) atomicAdd(&s_scan, my);
+      __syncthreads();
+      if (pass == 0) {
+        if (threadIdx.x == 0) {
+          int32_t run = 0;
+          for (int i = 0; i < nk; ++i) {
+            cnt[i] = run;
+            run += fill[i];
+          }
+          cnt[nk] = run;
+          ctr[0] = s_scan;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nk; i += SMALL_T) fill[i] = 0;
+        __syncthreads();
+      }
+    }
+    for (int s = 0; s < A.S; ++s) {
+      const int32_t *bo = cnt + s * NB;
+      const int32_t lo = bo[0], hi = bo[NB];
+      if (lo == hi) continue;
+      if (threadIdx.x < 3) A.ctr[threadIdx.x] = 0;
+#define KMP_GROUP_BIN(BIN, G)                                                  \
+  for (int32_t b0 = bo[BIN] + w * (32 / G); b0 < bo[BIN + 1]; b0 += W * (32 / G)) { \
+    const int32_t idx = b0 + lane / G;                                         \
+    rate_group<G>(A, idx < bo[BIN + 1] ? A.vlist[idx] : -1, idx, lane);        \
+  }
+      KMP_GROUP_BIN(0, 4)
+      KMP_GROUP_BIN(1, 8)
+      KMP_GROUP_BIN(2, 16)
+      KMP_GROUP_BIN(3, 32)
+#undef KMP_GROUP_BIN
+      for (int32_t idx = bo[4] + w; idx < bo[5]; idx += W) rate_warp(A, A.vlist[idx], idx, lane, keys, vals, list);
+      __syncthreads();
+      classify_range(A, lo + threadIdx.x, hi, SMALL_T);
+      __syncthreads();
+      const int32_t nslots = *(volatile int32_t *)&A.ctr[0];
+      if (nslots > 0) {
+        bucket_range(A, lo + threadIdx.x, hi, SMALL_T);
+        __syncthreads();
+        resolve_slots(A, nslots, 0, 1);
+        __syncthreads();
+      }
+      apply_range(A, lo + (threadIdx.x & ~31), hi, SMALL_T);
+      __syncthreads();
+    }
+    // a round that moved nothing leaves no active node: the rest would change nothing
+    if (ctr[1] == 0) break;
+  }
 }
 
 // CTAs of a kernel (no dynamic shared memory) that an SM holds at once
@@ -1473,12 +1574,14 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   const int32_t hub_bucket = C.tune.hub_bucket > 0 ? C.tune.hub_bucket : 256;
   int32_t nhubs = 0;
   int64_t nbmax = 0;
-  DBuf<int32_t> hubs, hrown, plan_h, hdense, hlab, hslab, hsw, hbcnt, hbcur, hboff, hbsum;
+  DBuf<int32_t> hubs, hpos, hrown, plan_h, hdense, hlab, hslab, hsw, hbcnt, hbcur, hboff, hbsum;
   DBuf<int64_t> plan_e, plan_x, plan_b, plan_tot;
   DBuf<unsigned long long> hkc, hku;
   if (hub_path) {
     DBuf<uint8_t> flag(n);
-    DBuf<int32_t> pos(n), cnt(1);
+    DBuf<int32_t> cnt(1);
+    hpos.alloc(n);  // an index per node: the plan and emit kernels look hubs up every sub-round
+    DBuf<int32_t> &pos = hpos;
     k_hub_flags<<<grid_for(n, 256), 256, 0, stream>>>(n, g.xadj, huge, flag);
     KMP_LAUNCHED("hub_flags");
     scan_excl_u8_to_i32(flag, pos, n, cnt);
@@ -1563,6 +1666,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   A.ctr = ctr;
   A.bigmove = bigmove;
   A.hubs = hubs.p;
+  A.hpos = hpos.p;
   A.nhubs = nhubs;
 
   A.hkc = hkc.p;
@@ -1714,7 +1818,22 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
       }
     }
   };
-  if (C.tune.lp_graphs) {
+  if (n <= SMALL_N && g.maxdeg <= SMALL_DEG && !C.profile) {
+    std::vector<LPRound> hr(rounds);
+    for (int r = 0; r < rounds; ++r) {
+      const uint64_t rk = key_step(basekey, (uint64_t)r);
+      hr[r] = LPRound{rk, (uint32_t)(rk >> 32), r, r + 1, 0};
+    }
+    DBuf<LPRound> dr(rounds);
+    to_dev(dr.p, hr.data(), (size_t)rounds);
+    static bool attr = false;
+    if (!attr) {
+      KMP_CUDA(cudaFuncSetAttribute(k_lp_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
+      attr = true;
+    }
+    k_lp_small<<<1, SMALL_T, SMALL_SMEM, stream>>>(A, dr, rounds);
+    KMP_LAUNCHED("lp_small");
+  } else if (C.tune.lp_graphs) {
     // one captured round, replayed for every round: its kernels read the
     // round's key, buffers and counters from device memory.  A round after
     // one that moved nothing has no active node and changes nothing, so all
