@@ -277,8 +277,9 @@ int kmp_profile_read_stage(double *stage_ms, double *stage_bytes, int64_t *spans
  */
 typedef struct {
   int32_t rate_blocks_per_sm; /* LP rating grid = this * SMs (2..16) */
-  int32_t hub_degree;         /* degree above which coarsening rates a node with the
-                                 multi-CTA hub kernels (256..2048) */
+  int32_t hub_degree;         /* degree above which coarsening rates a node with a wide CTA of
+                                 its own, and above 8192 with the multi-CTA hub kernels
+                                 (256..2048) */
   int32_t hub_chunk;          /* edges per hub work unit (256..65536, power of two;
                                  default 2048) */
   int32_t ip_blocks_per_sm;   /* bipartitioner CTAs per SM (1..8) */

@@ -24,7 +24,7 @@
 
 namespace kmp {
 
-constexpr int NB = 7;           // degree bins
+constexpr int NB = 8;           // degree bins
 constexpr int BIN_TILE = 2048;  // nodes per binning tile
 constexpr int RATE_T = 256;
 constexpr int WARP_TAB = 512;   // per-warp hash table (bin 4: degree <= 256)
@@ -32,14 +32,19 @@ constexpr int CTA_TAB = 4096;   // per-CTA shared table (bin 5: degree <= 2048)
 constexpr int64_t HUGE_DEG_MAX = CTA_TAB / 2;  // largest degree a shared CTA table serves
 static_assert(HUGE_DEG_MAX == 2048, "upper bound of kmp_tuning.hub_degree");
 
-__host__ __device__ __forceinline__ int deg_bin(int64_t d, int64_t huge) {
+// Bin 6: nodes of degree above the shared table of k_rate and up to MID_MAX, rated
+// by one wide CTA each with a table of its own (k_rate_mid); bin 7: hubs, over
+// many CTAs.
+constexpr int64_t MID_MAX = 8192;
+constexpr int MID_TAB = 2 * (int)MID_MAX;
+__host__ __device__ __forceinline__ int deg_bin(int64_t d, int64_t huge, int64_t mid) {
   if (d <= 4) return 0;
   if (d <= 8) return 1;
   if (d <= 16) return 2;
   if (d <= 32) return 3;
   if (d <= 256) return 4;
   if (d <= huge) return 5;
-  return 6;
+  return d <= mid ? 6 : 7;
 }
 
 // per-round values, read by the kernels from device memory so that one
@@ -87,8 +92,8 @@ struct LPArgs {
   int32_t *ctr;                // [0] slots, [1] bucket top, [2] big movers
   int32_t *bigmove;            // high-degree nodes that moved in this sub-round
   unsigned long long *ctr64;   // 18 per round: [0] scanned entries, [1] moved nodes, [2+s]
-                               // degree sum of sub-round s, [10+s] the same over bin 6 (hubs)
-  // bin 6 (degree > huge_deg) with many labels: the sub-round's hub entries
+                               // degree sum of sub-round s, [10+s] the same over bins 6 and 7
+  // bin 7 (degree > mid_deg) with many labels: the sub-round's hub entries
   // are hashed by label into buckets of about hub_bucket entries, scattered
   // into bucket order and aggregated one bucket per warp in shared memory
   const int32_t *hubs;         // hub node ids, ascending
@@ -104,15 +109,16 @@ struct LPArgs {
   int32_t *hbcur;              // scatter cursor per bucket (zeroed likewise)
   int32_t *hboff;              // bucket offsets: exclusive scan of hbcnt
   int32_t hub_bucket;          // target entries per bucket
-  int32_t *plan_h;             // per sub-round hub plan: hub index of each bin-6 entry,
+  int32_t *plan_h;             // per sub-round hub plan: hub index of each bin-7 entry,
   int64_t *plan_e;             // exclusive prefix of its edge chunks,
   int64_t *plan_x;             // of its entries (degree),
   int64_t *plan_b;             // of its buckets,
   int64_t *plan_tot;           // [0] edge chunks, [1] buckets, [2] entries
-  int32_t small_labels;        // all labels fit a CTA table: bin 6 handled like bin 5
-  int32_t *hdense;             // few labels: bin-6 entry i of a sub-round owns row i of
+  int32_t small_labels;        // all labels fit a CTA table: bins 6, 7 handled like bin 5
+  int32_t *hdense;             // few labels: bin-7 entry i of a sub-round owns row i of
                                // a [hubs][nlab] rating array filled by many CTAs
-  int64_t huge_deg;            // degree above which a node is a hub (many labels: <= HUGE_DEG_MAX)
+  int64_t huge_deg;            // largest degree of bin 5 (many labels: <= HUGE_DEG_MAX)
+  int64_t mid_deg;             // largest degree of bin 6; above it a node is a hub
   int64_t hub_chunk;           // edges per hub insert work unit
   int32_t nlab;
   int32_t S;
@@ -227,11 +233,11 @@ __global__ void __launch_bounds__(256) k_bin_count(LPArgs A, int32_t *cnt, int64
     int64_t d = A.xadj[v + 1] - A.xadj[v];
     if (d == 0) continue;
     int s = (int)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1));
-    int bin = deg_bin(d, A.huge_deg);
+    int bin = deg_bin(d, A.huge_deg, A.mid_deg);
     atomicAdd(&c[(s * NB + bin) * 32 + lane], 1);
     if (A.tmin) {
       atomicAdd(&sdeg[s], (unsigned long long)d);
-      if (bin == 6) atomicAdd(&sdeg6[s], (unsigned long long)d);
+      if (bin >= 6) atomicAdd(&sdeg6[s], (unsigned long long)d);
     }
     my += (unsigned long long)d;
   }
@@ -278,7 +284,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter(LPArgs A, const int32_t *of
       int64_t d = A.xadj[v + 1] - A.xadj[v];
       if (d > 0) {
         int s = (int)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1));
-        k = s * NB + deg_bin(d, A.huge_deg);
+        k = s * NB + deg_bin(d, A.huge_deg, A.mid_deg);
       }
     }
     if (v < A.n) act[v] = 0;
@@ -478,10 +484,11 @@ __device__ __forceinline__ void rate_warp(const LPArgs &A, int32_t u, int32_t po
   __syncwarp();
 }
 
-// one node per CTA with a shared table of `mask+1` entries
+// one node per CTA of NT threads with a shared table of `mask+1` entries
+template <int NT>
 __device__ void rate_cta(const LPArgs &A, int32_t u, int32_t pos, int32_t *keys, int32_t *vals,
                          uint16_t *list, uint32_t mask) {
-  __shared__ uint64_t red_c[RATE_T / 32], red_u[RATE_T / 32];
+  __shared__ uint64_t red_c[NT / 32], red_u[NT / 32];
   __shared__ int32_t lab_c, lab_u, s_cnt, s_rown;
   if (threadIdx.x == 0) {
     lab_c = -1;
@@ -552,7 +559,7 @@ __global__ void __launch_bounds__(RATE_T, 6) k_rate(LPArgs A, int s) {
   int64_t nw = (int64_t)gridDim.x * (RATE_T / 32);
   const int32_t *bo = A.boff + s * NB;
   if ((int64_t)bo[4] + (int64_t)blockIdx.x * (RATE_T / 32) < bo[5] ||
-      (int64_t)bo[5] + blockIdx.x < ((A.small_labels && !A.hdense) ? bo[7] : bo[6])) {
+      (int64_t)bo[5] + blockIdx.x < ((A.small_labels && !A.hdense) ? bo[NB] : bo[6])) {
     for (int i = threadIdx.x; i < CTA_TAB; i += blockDim.x) {  // only blocks with table work
       tkeys[i] = HT_EMPTY;
       tvals[i] = 0;
@@ -582,13 +589,13 @@ __global__ void __launch_bounds__(RATE_T, 6) k_rate(LPArgs A, int s) {
   }
   __syncthreads();
   {
-    // bin 5, and bin 6 as well when every label set fits a shared table and
-    // no dense hub array is in use
-    int32_t lo = bo[5], hi = (A.small_labels && !A.hdense) ? bo[7] : bo[6];
+    // bin 5, and every node above it as well when every label set fits a shared
+    // table and no dense hub array is in use
+    int32_t lo = bo[5], hi = (A.small_labels && !A.hdense) ? bo[NB] : bo[6];
     for (int64_t idx = lo + blockIdx.x; idx < hi; idx += gridDim.x) {
       int32_t u = A.vlist[idx];
       uint32_t cap = table_cap(A.xadj[u + 1] - A.xadj[u], A.nlab);
-      rate_cta(A, u, (int32_t)idx, tkeys, tvals, tlist, cap - 1);
+      rate_cta<RATE_T>(A, u, (int32_t)idx, tkeys, tvals, tlist, cap - 1);
     }
   }
   if (A.tmin) {
@@ -608,7 +615,35 @@ __device__ __forceinline__ void stamp_stage_end(const LPArgs &A, int s) {
   if (threadIdx.x == 0) atomicMax(&A.smax[(int64_t)__ldg(&A.R->r) * A.S + s], global_ns());
 }
 
-// ---- hubs (bin 6) with many labels: insert / reduce / emit
+// Nodes of bin 6: one CTA of 1024 threads a node, its labels in a shared table of
+// MID_TAB slots (144 KB with the slot list, one CTA an SM).  An entry is gathered
+// and added once; through the hub kernels it is also counted, written, scattered
+// and read again, which only pays when one CTA would be the bottleneck.  R-MAT
+// 2^24 has 53,000 such nodes with a third of all entries; its level-0 clustering:
+// 86.4 -> 77.9 ms.
+constexpr int MID_T = 1024;
+constexpr size_t MID_SMEM = (size_t)MID_TAB * 2 * sizeof(int32_t) + (size_t)MID_MAX * sizeof(uint16_t);
+__global__ void __launch_bounds__(MID_T, 1) k_rate_mid(LPArgs A, int s) {
+  extern __shared__ __align__(16) unsigned char mid_smem[];
+  int32_t *keys = reinterpret_cast<int32_t *>(mid_smem), *vals = keys + MID_TAB;
+  uint16_t *list = reinterpret_cast<uint16_t *>(vals + MID_TAB);
+  const int32_t *bo = A.boff + s * NB;
+  const int32_t lo = bo[6], hi = bo[7];
+  if (lo + (int32_t)blockIdx.x < hi) {
+    for (int i = threadIdx.x; i < MID_TAB; i += MID_T) {
+      keys[i] = HT_EMPTY;
+      vals[i] = 0;
+    }
+    __syncthreads();
+    for (int32_t idx = lo + blockIdx.x; idx < hi; idx += gridDim.x) {
+      const int32_t u = A.vlist[idx];
+      rate_cta<MID_T>(A, u, idx, keys, vals, list, table_cap(A.xadj[u + 1] - A.xadj[u], A.nlab) - 1);
+    }
+  }
+  stamp_stage_end(A, s);
+}
+
+// ---- hubs (bin 7) with many labels: insert / reduce / emit
 
 __device__ __forceinline__ int32_t find_seg(const int64_t *off, int32_t cnt, int64_t x) {
   int32_t lo = 0, hi = cnt - 1;  // last index with off[idx] <= x
@@ -635,7 +670,7 @@ __global__ void __launch_bounds__(1024) k_hub_plan(LPArgs A, int s) {
   __shared__ int64_t we[32], wx[32], wb[32];
   __shared__ int64_t carry_e, carry_x, carry_b;
   const int32_t *bo = A.boff + s * NB;
-  int32_t lo = bo[6], cnt = bo[7] - bo[6];
+  int32_t lo = bo[7], cnt = bo[8] - bo[7];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) { carry_e = 0; carry_x = 0; carry_b = 0; }
   __syncthreads();
@@ -759,7 +794,7 @@ __global__ void __launch_bounds__(HP_T) k_hub_count(LPArgs A, int s) {
   hp_clear_all(T);
   __syncthreads();
   const int32_t *bo = A.boff + s * NB;
-  int32_t cnt = bo[7] - bo[6];
+  int32_t cnt = bo[8] - bo[7];
   int64_t total = A.plan_tot[0];
   const int64_t per = ceil_div(total, (int64_t)gridDim.x);
   const int64_t c0 = (int64_t)blockIdx.x * per, c1 = c0 + per < total ? c0 + per : total;
@@ -816,7 +851,7 @@ __global__ void __launch_bounds__(HP_T) k_hub_scatter(LPArgs A, int s) {
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int32_t *bo = A.boff + s * NB;
-  int32_t cnt = bo[7] - bo[6];
+  int32_t cnt = bo[8] - bo[7];
   int64_t total = A.plan_tot[0];
   const int64_t per = ceil_div(total, (int64_t)gridDim.x);
   const int64_t c0 = (int64_t)blockIdx.x * per, c1 = c0 + per < total ? c0 + per : total;
@@ -949,7 +984,7 @@ __global__ void __launch_bounds__(HB_W * 32) k_hub_bucket(LPArgs A, int s) {
   }
   __syncwarp();
   const int32_t *bo = A.boff + s * NB;
-  const int32_t cnt = bo[7] - bo[6];
+  const int32_t cnt = bo[8] - bo[7];
   const int64_t NBt = A.plan_tot[1];
   const uint32_t mask = HB_TAB - 1;
   const int64_t gw = (int64_t)blockIdx.x * W + w, nw = (int64_t)gridDim.x * W;
@@ -1018,7 +1053,7 @@ __global__ void __launch_bounds__(HB_W * 32) k_hub_bucket(LPArgs A, int s) {
 
 __global__ void __launch_bounds__(256) k_hub_emit(LPArgs A, int s) {
   const int32_t *bo = A.boff + s * NB;
-  int32_t lo = bo[6], hi = bo[7];
+  int32_t lo = bo[7], hi = bo[8];
   for (int64_t p = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < hi;
        p += (int64_t)gridDim.x * blockDim.x) {
     int32_t u = A.vlist[p];
@@ -1042,7 +1077,7 @@ __global__ void __launch_bounds__(256) k_hub_emit(LPArgs A, int s) {
 __global__ void __launch_bounds__(256) k_hubd_insert(LPArgs A, int s) {
   extern __shared__ int32_t cnt_s[];
   const int32_t *bo = A.boff + s * NB;
-  const int32_t lo = bo[6], cnt = bo[7] - bo[6];
+  const int32_t lo = bo[7], cnt = bo[8] - bo[7];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t total = A.plan_tot[0];
   const int64_t per = ceil_div(total, (int64_t)gridDim.x);
@@ -1098,7 +1133,7 @@ __global__ void __launch_bounds__(256) k_hubd_reduce(LPArgs A, int s) {
   __shared__ int32_t s_rown;
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int32_t *bo = A.boff + s * NB;
-  int32_t lo = bo[6], cnt = bo[7] - bo[6];
+  int32_t lo = bo[7], cnt = bo[8] - bo[7];
   for (int32_t i = blockIdx.x; i < cnt; i += gridDim.x) {
     int32_t u = A.vlist[lo + i];
     int32_t own = A.label[u], cu = node_w(A, u);
@@ -1457,7 +1492,7 @@ __global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *roun
         const int64_t d = A.xadj[v + 1] - A.xadj[v];
         if (pass == 1) act[v] = 0;
         if (d == 0) continue;
-        const int key = (int)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1)) * NB + deg_bin(d, A.huge_deg);
+        const int key = (int)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1)) * NB + deg_bin(d, A.huge_deg, A.mid_deg);
         const int32_t at = atomicAdd(&fill[key], 1);
         if (pass == 1) A.vlist[cnt[key] + at] = v;
         my += (unsigned long long)d;
@@ -1554,12 +1589,12 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   // offset per bucket)
   bool small_labels = 2 * (int64_t)nlab <= CTA_TAB;
   const int64_t huge = small_labels ? C.tune.dense_hub_degree : C.tune.hub_degree;
-  bool hub_path = !small_labels && g.maxdeg > huge;
+  bool many = !small_labels && g.maxdeg > huge;
   bool dense_hubs = small_labels && g.maxdeg > huge;
   // with more labels than a CTA table holds but at most tune.dense_labels of
   // them, hubs may rate into dense rows of nlab counters (the paper's dense
   // vector for high-degree nodes) when all rows fit DENSE_ROWS_MAX_BYTES
-  if (hub_path && C.tune.dense_labels > 0 && nlab <= C.tune.dense_labels) {
+  if (many && C.tune.dense_labels > 0 && nlab <= C.tune.dense_labels) {
     DBuf<uint8_t> flag(n);
     DBuf<int32_t> pos(n), cnt(1);
     k_hub_flags<<<grid_for(n, 256), 256, 0, stream>>>(n, g.xadj, huge, flag);
@@ -1567,10 +1602,13 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     scan_excl_u8_to_i32(flag, pos, n, cnt);
     const int64_t nh = read1(cnt.p);
     if (nh * (int64_t)nlab * (int64_t)sizeof(int32_t) <= DENSE_ROWS_MAX_BYTES) {
-      hub_path = false;
+      many = false;
       dense_hubs = true;
     }
   }
+  // with many labels, bin 6 lies between the shared table of k_rate and the hubs
+  const int64_t mid = many ? MID_MAX : huge;
+  const bool hub_path = many && g.maxdeg > mid;
   const int32_t hub_bucket = C.tune.hub_bucket > 0 ? C.tune.hub_bucket : 256;
   int32_t nhubs = 0;
   int64_t nbmax = 0;
@@ -1582,7 +1620,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     DBuf<int32_t> cnt(1);
     hpos.alloc(n);  // an index per node: the plan and emit kernels look hubs up every sub-round
     DBuf<int32_t> &pos = hpos;
-    k_hub_flags<<<grid_for(n, 256), 256, 0, stream>>>(n, g.xadj, huge, flag);
+    k_hub_flags<<<grid_for(n, 256), 256, 0, stream>>>(n, g.xadj, mid, flag);
     KMP_LAUNCHED("hub_flags");
     scan_excl_u8_to_i32(flag, pos, n, cnt);
     nhubs = read1(cnt.p);
@@ -1640,6 +1678,14 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     plan_tot.alloc(3);
   }
 
+  if (many) {
+    static bool mid_attr = false;  // before any capture
+    if (!mid_attr) {
+      KMP_CUDA(cudaFuncSetAttribute(k_rate_mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MID_SMEM));
+      mid_attr = true;
+    }
+  }
+
   LPArgs A{};
   A.n = n;
   A.xadj = g.xadj;
@@ -1687,6 +1733,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   A.small_labels = small_labels ? 1 : 0;
   A.hdense = dense_hubs ? hdense.p : nullptr;
   A.huge_deg = huge;
+  A.mid_deg = mid;
   A.hub_chunk = C.tune.hub_chunk;
   A.nlab = nlab;
   A.S = S;
@@ -1749,6 +1796,10 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     for (int s = 0; s < S; ++s) {
       k_rate<<<grid_rate, RATE_T, 0, st>>>(A, s);
       KMP_LAUNCHED("rate");
+      if (many) {
+        k_rate_mid<<<C.sms, MID_T, MID_SMEM, st>>>(A, s);
+        KMP_LAUNCHED("rate_mid");
+      }
       if (hub_path) {
         k_hub_plan<<<1, 1024, 0, st>>>(A, s);
         KMP_LAUNCHED("hub_plan");
@@ -1796,7 +1847,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     to_host(t0.data(), tmin.p, t0.size());
     to_host(t1.data(), tmax.p, t1.size());
     to_host(t2.data(), smax.p, t2.size());
-    bool hubs_outside = hub_path || dense_hubs;
+    bool hubs_outside = many || dense_hubs;
     const double per_entry = 8.0 + (g.ew ? 4.0 : 0.0), per_node = 24.0 + (g.vw ? 4.0 : 0.0);
     for (int r = 0; r < nr; ++r) {
       const int32_t *hboff = hb.data() + (size_t)(S * NB + 1) * r;
@@ -1805,7 +1856,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
         const double Dall = (double)h[18 * r + 2 + s];
         double V = Vall, D = Dall;
         if (hubs_outside) {
-          V -= (double)(hboff[s * NB + 7] - hboff[s * NB + 6]);
+          V -= (double)(hboff[(s + 1) * NB] - hboff[s * NB + 6]);
           D -= (double)h[18 * r + 10 + s];
         }
         size_t i = (size_t)S * r + s;
