@@ -287,18 +287,19 @@ __global__ void __launch_bounds__(BAL_T) k_bal_sort(BalArgs A) {
 
 // Moves in candidate order, evaluated in batches of up to 32.  A batch holds
 // the shortest prefix of the remaining candidates whose weights cover the
-// overload (it may need more moves, never fewer).  The batch's adjacency
-// rows are walked at once (by warp 0 alone for a small batch, else by the
-// whole CTA), building one connectivity table per member and marking which
-// members are neighbours of each other; each member's target is picked from
-// the state at the start of the batch, and one thread commits in order.
-// While a block is emptied, every other block only gains
-// weight, so a target that is still admissible is still the best (or still
-// the lowest-id admissible one), and "no admissible target" stays true; only
-// a move of a neighbour changes connectivity.  A member passes iff its target
-// still fits and no earlier move of the batch was its neighbour; at the first
-// one that does not, the next batch starts there (its first member always
-// passes).  The result equals one move at a time.
+// overload (it may need more moves, never fewer).  The batch's adjacency rows
+// are walked at once, building one connectivity table per member and marking
+// which members are neighbours of each other.  A small batch (warp 0 alone) then
+// decides its members in order, each from its table and the current rooms; a
+// move adds its edge weights to the tables of the later members next to it.  A
+// large batch (the whole CTA) picks every member's target from the state at its
+// start and commits in order: while a block is emptied, every other block only
+// gains weight, so a target that is still admissible is still the best (or
+// still the lowest-id admissible one), and "no admissible target" stays true;
+// only a move of a neighbour changes connectivity.  There a member passes iff
+// its target still fits and no earlier move of the batch was its neighbour; at
+// the first one that does not, the next batch starts (its first member always
+// passes).  Either way the result equals one move at a time.
 constexpr int BM_T = 1024;
 constexpr int BM_W = BM_T / 32;
 
@@ -394,7 +395,9 @@ __global__ void __launch_bounds__(BAL_T) k_bal_spec(BalArgs A) {
 // slots is evaluated by warp 0 alone, in shared-memory tables; a larger one by
 // the CTA, in shared memory too (over the windows, which are read again after it)
 // while its tables fit.  Mesh of 2^20 nodes, 8192 blocks of 128 nodes brought from
-// 10% to 3% imbalance, the whole call: 97.0 -> 58.4 ms.
+// 10% to 3% imbalance, the whole call: 97.0 -> 58.4 ms with the windows and rooms,
+// 30.8 ms with small batches decided to their end (a batch used to stop at the
+// first member next to an earlier move, and its tables were built again).
 constexpr int WS_E = 256;
 constexpr int WS_T = 2048;
 constexpr int WS_R = 4;   // entries per lane whose gathers are issued together
@@ -590,6 +593,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
   __shared__ uint32_t s_adj[BM_W], s_mask[BM_W], s_toff[BM_W + 1];
   __shared__ unsigned long long s_best[BM_W];
   __shared__ int32_t mk[MEMB], mv[MEMB];
+  __shared__ int32_t adjw[32][33];  // edge weights between the members of a small batch, where s_adj has the bit
   __shared__ int32_t s_nb, s_B, s_ob, s_i, s_phase, s_done, s_large, s_hint;
   constexpr unsigned ALL = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -753,61 +757,55 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
           for (int r = 0; r < WS_R; ++r)
             if (uu[r] >= 0) {
               const int32_t ib = memb_find(mk, mv, uu[r]);
-              if (ib >= 0) atomicOr(&s_adj[jm[r]], 1u << ib);
+              if (ib >= 0) {
+                atomicOr(&s_adj[jm[r]], 1u << ib);
+                adjw[jm[r]][ib] = wt[r];
+              }
               ht_add(wk + s_toff[jm[r]], wv + s_toff[jm[r]], s_mask[jm[r]], bk[r], wt[r]);
             }
         }
         __syncwarp();
-        // best admissible block of every member (kept by the member's lane); the
-        // tables are emptied on the way (every table spans whole 32-slot chunks)
-        int32_t bc = 0, bt = INT32_MAX;
-        for (uint32_t base = 0; base < TT; base += 32 * WS_R) {
-          int32_t b[WS_R], cv[WS_R], rm[WS_R];
-#pragma unroll
-          for (int r = 0; r < WS_R; ++r) {
-            const uint32_t x = base + 32 * r + lane;
-            b[r] = HT_EMPTY;
-            if (x < TT) {
-              b[r] = wk[x];
-              cv[r] = wv[x];
-              wk[x] = HT_EMPTY;
-              wv[x] = 0;
+        // In order, each member from its own table and the rooms as the members
+        // before it left them; a move adds its weight to the tables of the later
+        // members it neighbours (bits of s_adj, weights in adjw), so every member
+        // is decided here, whatever the earlier ones did.
+        const uint32_t madj = lane < nb ? s_adj[lane] : 0;
+        int32_t left = need, j = 0;
+        for (; j < nb && left > 0; ++j) {
+          const uint32_t t0 = s_toff[j], t1 = s_toff[j + 1];
+          const int32_t cj = __shfl_sync(ALL, c, j);
+          int32_t bc = 0, bt = INT32_MAX;
+          for (uint32_t x = t0 + lane; x < t1; x += 32) {
+            const int32_t b = wk[x];
+            if (b != HT_EMPTY && b != B && room[b] >= cj) best_of(wv[x], b, bc, bt);
+          }
+          const int32_t m = __reduce_max_sync(ALL, bc);
+          int32_t t;
+          if (m > 0) t = __reduce_min_sync(ALL, bc == m ? bt : INT32_MAX);
+          else t = lowest_admissible(room, A.k, cj, lane, &s_hint);
+          if (t >= 0) {
+            if (lane == j) {
+              A.part[v] = t;
+              room[t] -= cj;
             }
+            if (lane > j && ((madj >> j) & 1u)) ht_add(wk + (tpre - cap), wv + (tpre - cap), cap - 1, t, adjw[lane][j]);
+            left -= cj;
+            ++n_moves;
           }
-#pragma unroll
-          for (int r = 0; r < WS_R; ++r) rm[r] = b[r] != HT_EMPTY && b[r] != B ? room[b[r]] : INT32_MIN;
-#pragma unroll
-          for (int r = 0; r < WS_R; ++r) {
-            const uint32_t at = base + 32 * r;
-            if (at >= TT) break;
-            const int32_t j = __popc(__ballot_sync(ALL, lane < nb && tpre <= at));  // the chunk's member
-            const int32_t cj = __shfl_sync(ALL, c, j);
-            const bool adm = rm[r] >= cj;
-            const int32_t m = __reduce_max_sync(ALL, adm ? cv[r] : 0);
-            if (m == 0) continue;
-            const int32_t tb = __reduce_min_sync(ALL, adm && cv[r] == m ? b[r] : INT32_MAX);
-            if (lane == j) best_of(m, tb, bc, bt);
-          }
+          __syncwarp();
         }
-        int32_t t = lane < nb && bc > 0 ? bt : -1;
-        for (unsigned none = __ballot_sync(ALL, lane < nb && t < 0); none; none &= none - 1) {
-          const int j = __ffs(none) - 1;
-          const int32_t x = lowest_admissible(room, A.k, __shfl_sync(ALL, c, j), lane, &s_hint);
-          if (lane == j) t = x;
+        for (uint32_t x = lane; x < TT; x += 32) {
+          wk[x] = HT_EMPTY;
+          wv[x] = 0;
         }
-        const int32_t rt = t >= 0 ? room[t] : 0;
-        const uint32_t adj = lane < nb ? s_adj[lane] : 0;
-        if (lane < MEMB / 2) {
-          mk[lane] = HT_EMPTY;
-          mk[lane + 32] = HT_EMPTY;
+        mk[lane] = HT_EMPTY;
+        mk[lane + 32] = HT_EMPTY;
+        if (lane == 0 && left != need) {
+          room[B] = -left;
+          if (left < 0 && B < s_hint) s_hint = B;  // the block got room
         }
         __syncwarp();
-        bool stop = false;
-        i += commit_batch(A, room, B, nb, v, t, c, adj, rt, need, &s_hint, n_moves, stop);
-        if (stop) {
-          ++ob;
-          phase = 0;
-        }
+        i += j;
       }
       if (lane == 0) {
         s_ob = ob;
