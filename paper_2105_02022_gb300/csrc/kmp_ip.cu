@@ -32,20 +32,19 @@ constexpr int IPW = IPT / 32;
 constexpr int IP_MAXL = 63;
 constexpr int32_t IP_MAX_N = 65535;
 constexpr uint16_t IP_NONE = 0xFFFF;  // no node: ids are below IP_MAX_N
-// Dynamic shared memory of a bipartitioner CTA: a hash table per warp (wtab slots
-// of key and weight: rows up to wtab / 2 entries) and behind them the working
-// state of the item's phases (dyn_words).  An item's time is latency, so what
-// counts is how many an SM works on.  A round with more items than SMs: 256
-// slots and 12,800 words, 67 KB in all, three CTAs an SM (with 80 registers a
-// thread).  That holds items of up to 2300 nodes; larger ones work in their
-// scratch, which is still faster than two CTAs an SM that hold 3350 nodes (4096
-// items of 200..4000 nodes: 32.4 against 38.2 ms).  Otherwise the items are on
-// the critical path: one CTA an SM with what it offers.
-struct IPShape {
-  int32_t wtab, dyn_words;
-};
-constexpr IPShape IP_SHAPE3{256, 12800}, IP_SHAPE1{512, 45000};
-constexpr size_t ip_smem(IPShape s) { return 4 * (size_t)(2 * IPW * s.wtab + s.dyn_words); }
+// Dynamic shared memory of a bipartitioner CTA: the working state of the item's
+// phases (dyn_words) and behind it a hash table per warp (wtab slots of key and
+// weight: rows up to wtab / 2 entries).  An item's time is latency, so what counts
+// is how many an SM works on.  A round with more items than SMs: 67 KB in all,
+// three CTAs an SM (with 80 registers a thread).  That holds items of up to 2300
+// nodes; larger ones work in their scratch, which is still faster than two CTAs an
+// SM that hold 3350 nodes (4096 items of 200..4000 nodes: 32.4 against 38.2 ms).
+// Otherwise the items are on the critical path: one CTA an SM with what it offers.
+// The tables take what the largest item's state leaves, from 256 to 2048 slots:
+// coarse R-MAT items of 300 nodes have rows of 300 entries, and a row beyond its
+// warp's table is aggregated in the item's scratch (partition of R-MAT 2^22, k = 4096:
+// 372.0 -> 368.4 ms).
+constexpr int32_t IP_WORDS3 = 16896, IP_WORDS1 = 53192, IP_WTAB_MIN = 256, IP_WTAB_MAX = 2048;
 
 struct ItemDesc {
   int64_t vbase;  // first member position
@@ -2124,16 +2123,18 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
       // working state: the LP arrays (5.5 words a node and the sort space of a
       // sub-round's contested proposals), then FM's (3.6 words a node, the entries
       // where they fit) of the largest item, at least 16 KB (the portfolio of small
-      // coarsest graphs); see IPShape
+      // coarsest graphs); see IP_WORDS*
       const int64_t want = std::max<int64_t>(6 * maxn + maxn / 8 + 256, 4096);
-      const IPShape shape = (int64_t)items.size() <= C.sms ? IP_SHAPE1 : IP_SHAPE3;
-      A.wtab = shape.wtab;
-      A.dyn_words = (int32_t)std::min<int64_t>((want + 3) & ~3ll, shape.dyn_words);
-      const size_t dyn_bytes = ip_smem(IPShape{A.wtab, A.dyn_words});
+      const int64_t words = (int64_t)items.size() <= C.sms ? IP_WORDS1 : IP_WORDS3;
+      int32_t wtab = IP_WTAB_MIN;
+      while (wtab < IP_WTAB_MAX && 2 * IPW * (2 * wtab) + want <= words) wtab *= 2;
+      A.wtab = wtab;
+      A.dyn_words = (int32_t)std::min<int64_t>((want + 3) & ~3ll, words - 2 * IPW * wtab);
+      const size_t dyn_bytes = 4 * (size_t)(2 * IPW * A.wtab + A.dyn_words);
       static bool attr_set = false;
       if (!attr_set) {
         KMP_CUDA(cudaFuncSetAttribute(k_ip_items, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)ip_smem(IP_SHAPE1)));
+                                      4 * IP_WORDS1));
         attr_set = true;
       }
       k_ip_items<<<gridip, IPT, dyn_bytes, s>>>(A);
