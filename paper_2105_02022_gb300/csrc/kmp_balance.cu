@@ -393,8 +393,7 @@ __global__ void __launch_bounds__(BAL_T) k_bal_spec(BalArgs A) {
 // memory while k fits, and the blocks of the neighbours, the one gather from
 // global memory left per batch.  A batch with at most WS_E entries and WS_T table
 // slots is evaluated by warp 0 alone, in shared-memory tables; a larger one by
-// the CTA, in shared memory too (over the windows, which are read again after it)
-// while its tables fit.  Mesh of 2^20 nodes, 8192 blocks of 128 nodes brought from
+// the CTA, in shared memory too while its tables fit beside the windows or over them.  Mesh of 2^20 nodes, 8192 blocks of 128 nodes brought from
 // 10% to 3% imbalance, the whole call: 97.0 -> 58.4 ms with the windows and rooms,
 // 30.8 ms with small batches decided to their end (a batch used to stop at the
 // first member next to an earlier move, and its tables were built again).
@@ -582,8 +581,15 @@ constexpr int32_t BAL_SLOTS = (int32_t)(BAL_WINDOWS / (2 * sizeof(int32_t))) & ~
 constexpr size_t BAL_TABS = 2 * WS_T * sizeof(int32_t);
 constexpr int32_t BAL_ROOM_K = 26000;  // rooms in shared memory: 104 KB beside 94 KB of windows and 16 KB of tables
 
+// dynamic shared memory of the commit: windows, warp 0's tables, rooms, and the
+// tables of large batches in what is left (`slots` of them; a batch that needs
+// more lies over the windows, which are then read again, or in global memory).
+// With all large batches over the windows, 32 windows were read again for each:
+// partition of R-MAT 2^22, k = 4096, 368.4 ms, and 353.1 like this.
+constexpr size_t BAL_SMEM_MAX = 224000;
+
 template <bool SROOM>
-__global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
+__global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, int32_t slots) {
   extern __shared__ __align__(16) unsigned char bal_smem[];
   BalWindow *const win = reinterpret_cast<BalWindow *>(bal_smem);
   int32_t *const wk = reinterpret_cast<int32_t *>(bal_smem + BAL_WINDOWS), *const wv = wk + WS_T;  // empty between batches
@@ -614,13 +620,18 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
   int32_t n_moves = 0, n_spec = 0;                   // warp 0's counts
   unsigned long long n_batches = 0, n_cands = 0, n_entries = 0;
   __syncthreads();
+  int32_t g0 = 0, gn = 0;  // blocks whose windows are held
+  bool reload = true;
   for (;;) {
-    // windows of the next blocks; the first may be under way (phase 1, candidate s_i)
-    const int32_t g0 = s_ob, gn = min(BM_W, A.nover - g0);
-    if (w < gn) load_window(A, win[w], g0 + w, w == 0 && s_phase == 1 ? s_i : -1);
-    __syncthreads();
+    if (reload) {
+      // windows of the next blocks; the first may be under way (phase 1, candidate s_i)
+      g0 = s_ob;
+      gn = min(BM_W, A.nover - g0);
+      if (w < gn) load_window(A, win[w], g0 + w, w == 0 && s_phase == 1 ? s_i : -1);
+      __syncthreads();
+    }
     if (w == 0) {
-      int32_t ob = g0, i = s_i, phase = s_phase;
+      int32_t ob = s_ob, i = s_i, phase = s_phase;
       bool large = false;
       while (ob < g0 + gn) {
         BalWindow &W = win[ob - g0];
@@ -817,13 +828,16 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
     }
     __syncthreads();
     if (s_done) break;
+    reload = true;
     if (!s_large) continue;
-    // ---- a large batch, evaluated by the whole CTA; the windows are no longer needed
+    // ---- a large batch, evaluated by the whole CTA
     const int32_t B = s_B, nb = s_nb;
     // every table size is a multiple of 32, so a warp's 32 slots lie in one table
     const uint32_t TT = s_toff[nb];
-    const bool sm = TT <= (uint32_t)BAL_SLOTS;  // tables over the windows
-    int32_t *const sk = reinterpret_cast<int32_t *>(bal_smem), *const sv = sk + BAL_SLOTS;
+    const bool beside = TT <= (uint32_t)slots, over = !beside && TT <= (uint32_t)BAL_SLOTS, sm = beside || over;
+    reload = over;
+    int32_t *const sk = over ? reinterpret_cast<int32_t *>(bal_smem) : wv + WS_T + (SROOM ? A.k : 0);
+    int32_t *const sv = sk + (over ? BAL_SLOTS : slots);
     auto keys_of = [&](int32_t j) { return sm ? sk + s_toff[j] : A.gtab + (int64_t)j * 2 * gcap; };
     auto vals_of = [&](int32_t j) { return sm ? sv + s_toff[j] : A.gtab + (int64_t)j * 2 * gcap + gcap; };
     {
@@ -909,7 +923,9 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom) {
       }
     }
     __syncthreads();
-    if (s_done) break;
+    const bool done = s_done;
+    __syncthreads();  // warp 0 may go straight on to the next blocks and write it again
+    if (done) break;
   }
   if (threadIdx.x == 0) {
     A.moved[0] = (unsigned long long)n_moves;
@@ -1035,20 +1051,19 @@ int64_t balance(const Graph &g, int32_t k, const int32_t *caps_host, int32_t *pa
   // memory; rooms in shared memory while k fits
   DBuf<int32_t> gtab1(2ll * gcap * BM_W), room;
   A.gtab = gtab1;
-  const size_t smem = BAL_WINDOWS + BAL_TABS + (k <= BAL_ROOM_K ? (size_t)k * sizeof(int32_t) : 0);
+  const size_t fixed = BAL_WINDOWS + BAL_TABS + (k <= BAL_ROOM_K ? (size_t)k * sizeof(int32_t) : 0);
+  const int32_t slots = (int32_t)((BAL_SMEM_MAX - fixed) / (2 * sizeof(int32_t))) & ~31;
   static bool attr = false;
   if (!attr) {
-    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(BAL_WINDOWS + BAL_TABS + BAL_ROOM_K * sizeof(int32_t))));
-    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(BAL_WINDOWS + BAL_TABS)));
+    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAL_SMEM_MAX));
+    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAL_SMEM_MAX));
     attr = true;
   }
   if (k <= BAL_ROOM_K) {
-    k_bal_moves<true><<<1, BM_T, smem, s>>>(A, nullptr);
+    k_bal_moves<true><<<1, BM_T, BAL_SMEM_MAX, s>>>(A, nullptr, slots);
   } else {
     room.alloc(k);
-    k_bal_moves<false><<<1, BM_T, smem, s>>>(A, room);
+    k_bal_moves<false><<<1, BM_T, BAL_SMEM_MAX, s>>>(A, room, slots);
   }
   KMP_LAUNCHED("bal_moves");
   unsigned long long hm[5];
