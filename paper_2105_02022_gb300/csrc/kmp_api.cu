@@ -540,7 +540,6 @@ int kmp_contract(const kmp_graph *g, const kmp_vid *label, kmp_graph **coarse_ou
   return guarded([&] {
     if (!g || !label || !coarse_out || !map_out) fail(KMP_ERR_ARG, "NULL argument");
     *coarse_out = nullptr;
-    check_range(g->g.n, label, 0, g->g.n, "label");
     Graph c = contract_graph(g->g, label, map_out);
     sync_and_check("contract");
     kmp_graph *h = new kmp_graph;

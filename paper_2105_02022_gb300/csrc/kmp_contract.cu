@@ -43,10 +43,14 @@ __host__ __device__ __forceinline__ int row_class(unsigned long long ub) {
                          : CLS_GLOBAL;
 }
 
-__global__ void k_map_used(int32_t n, const int32_t *label, uint8_t *used) {
+// labels outside [0, n) set *bad and mark nothing
+__global__ void k_map_used(int32_t n, const int32_t *label, uint8_t *used, int32_t *bad) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-       v += (int64_t)gridDim.x * blockDim.x)
-    used[label[v]] = 1;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t l = label[v];
+    if (l < 0 || l >= n) *bad = 1;
+    else used[l] = 1;
+  }
 }
 
 __global__ void k_map(int32_t n, const int32_t *label, const int32_t *cid, int32_t *map) {
@@ -920,17 +924,22 @@ __global__ void k_graph_facts(int32_t n, const int64_t *xadj, const int32_t *vw,
   }
 }
 
-void compute_facts(Graph &g) {
-  DBuf<unsigned long long> f(4);
-  f.zero();
-  k_graph_facts<<<grid_for(g.n, 256), 256, 0, ctx().stream>>>(g.n, g.xadj, g.vw, f);
-  KMP_LAUNCHED("graph_facts");
-  unsigned long long h[4];
-  to_host(h, f.p, 4);
-  g.maxdeg = (int64_t)h[0];
-  g.n_isolated = (int64_t)h[1];
+static void set_facts(Graph &g, const int64_t *h) {
+  g.maxdeg = h[0];
+  g.n_isolated = h[1];
   g.max_vw = (int32_t)h[2];
-  g.total_vw = (int64_t)h[3];
+  g.total_vw = h[3];
+}
+
+void compute_facts(Graph &g) {
+  DBuf<int64_t> f(4);
+  f.zero();
+  k_graph_facts<<<grid_for(g.n, 256), 256, 0, ctx().stream>>>(g.n, g.xadj, g.vw,
+                                                             reinterpret_cast<unsigned long long *>(f.p));
+  KMP_LAUNCHED("graph_facts");
+  int64_t h[4];
+  to_host(h, f.p, 4);
+  set_facts(g, h);
 }
 
 void free_graph(Graph &g) {
@@ -950,13 +959,17 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
   int grid = grid_for(n, 256);
   DBuf<uint8_t> used(n);
   used.zero();
-  DBuf<int32_t> cid(n), ncd(1);
-  k_map_used<<<grid, 256, 0, s>>>(n, label, used);
+  DBuf<int32_t> cid(n), ncd(2);  // coarse nodes, bad labels
+  ncd.zero();
+  k_map_used<<<grid, 256, 0, s>>>(n, label, used, ncd.p + 1);
   KMP_LAUNCHED("map_used");
   scan_excl_u8_to_i32(used, cid, n, ncd);
+  int32_t hn[2];
+  to_host(hn, ncd.p, 2);
+  if (hn[1]) fail(KMP_ERR_ARG, "label: value out of range");
+  const int32_t nc = hn[0];
   k_map<<<grid, 256, 0, s>>>(n, label, cid, map);
   KMP_LAUNCHED("map");
-  int32_t nc = read1(ncd.p);
 
   Graph out;
   out.n = nc;
@@ -973,13 +986,12 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
   k_members<<<grid, 256, 0, s>>>(n, map, moff, mcur, members);
   KMP_LAUNCHED("members");
   // temporary rows at upper-bound offsets
-  DBuf<int64_t> ub64(nc + 1), toff(nc + 1), ttot(1);
+  DBuf<int64_t> ub64(nc + 1), toff(nc + 1);
   int gridc = grid_for(nc, 256);
   k_ub_to_i64<<<gridc, 256, 0, s>>>(nc, cub, ub64);
   KMP_LAUNCHED("ub_copy");
-  scan_excl_i64(ub64, toff, nc, ttot);
-  int64_t tot = read1(ttot.p);
-  DBuf<int32_t> tadj(tot), tw(tot), cdeg(nc + 1);
+  scan_excl_i64(ub64, toff, nc, nullptr);
+  DBuf<int32_t> tadj(g.m), tw(g.m), cdeg(nc + 1);  // every entry belongs to one coarse row
   cdeg.zero();
   DBuf<int32_t> lists((int64_t)NCLASS * nc), counts(NCLASS);
   counts.zero();
@@ -1078,12 +1090,19 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
       }
     }
   }
-  DBuf<int64_t> mtot(1);
+  // entries and facts of the coarse graph in one read
+  DBuf<int64_t> sizes(5);
+  sizes.zero();
   out.xadj = static_cast<int64_t *>(dmalloc((nc + 1) * sizeof(int64_t)));
-  scan_excl_i32_to_i64(cdeg, out.xadj, nc, mtot);
-  k_set_last_i64<<<1, 1, 0, s>>>(out.xadj, nc, mtot);
+  scan_excl_i32_to_i64(cdeg, out.xadj, nc, sizes.p + 4);
+  k_set_last_i64<<<1, 1, 0, s>>>(out.xadj, nc, sizes.p + 4);
   KMP_LAUNCHED("set_last");
-  out.m = read1(mtot.p);
+  k_graph_facts<<<gridc, 256, 0, s>>>(nc, out.xadj, cvw, reinterpret_cast<unsigned long long *>(sizes.p));
+  KMP_LAUNCHED("graph_facts");
+  int64_t hs[5];
+  to_host(hs, sizes.p, 5);
+  set_facts(out, hs);
+  out.m = hs[4];
   out.adj = static_cast<int32_t *>(dmalloc((out.m > 0 ? out.m : 1) * sizeof(int32_t)));
   out.ew = static_cast<int32_t *>(dmalloc((out.m > 0 ? out.m : 1) * sizeof(int32_t)));
   if (nc > 0) {
@@ -1092,7 +1111,6 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
     KMP_LAUNCHED("copy_rows");
   }
   out.vw = cvw.release();
-  compute_facts(out);
   return out;
 }
 
@@ -1122,11 +1140,12 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
                                                 const int32_t *__restrict__ adj, const int32_t *__restrict__ vw,
                                                 const int32_t *__restrict__ ew, const int32_t *__restrict__ part,
                                                 unsigned long long *bw, unsigned long long *cut,
-                                                unsigned long long *bad) {
+                                                unsigned long long *bad, const int *status) {
   __shared__ unsigned long long sbw[CUT_SBW];
   const bool local = k <= CUT_SBW;
   if (local)
     for (int i = threadIdx.x; i < k; i += blockDim.x) sbw[i] = 0;
+  if (status && blockIdx.x == 0 && threadIdx.x == 0) bad[1] = (unsigned long long)(long long)*status;
   __syncthreads();
   bool off = false;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
@@ -1194,11 +1213,7 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
       if (sbw[i]) atomicAdd(&bw[i], sbw[i]);
 }
 
-// every edge was counted from both ends; status (nullable): the device status word behind the cut's
-__global__ void k_cut_finish(int64_t *c, const int *status, int64_t *status_out) {
-  *c /= 2;
-  if (status) *status_out = *status;
-}
+__global__ void k_half(int64_t *c) { *c /= 2; }  // every edge was counted from both ends
 
 // block weights only (no edge traffic)
 __global__ void __launch_bounds__(256) k_bw_only(int32_t n, int32_t k, const int32_t *vw,
@@ -1229,11 +1244,13 @@ void block_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw_d
   KMP_LAUNCHED("bw_only");
 }
 
-static void launch_cut(const Graph &g, const int32_t *part, int32_t k, int64_t *bw, int64_t *cut, int64_t *bad) {
+// bad, status (nullable): as in k_cut_bw; the status word goes behind bad
+static void launch_cut(const Graph &g, const int32_t *part, int32_t k, int64_t *bw, int64_t *cut, int64_t *bad,
+                       const int *status) {
   const int64_t work = std::max<int64_t>(g.n, ceil_div(g.m, CUT_TILE) * 32);
   k_cut_bw<<<grid_for(work, 256, 8), 256, 0, ctx().stream>>>(
       g.n, g.m, k, g.xadj, g.adj, g.vw, g.ew, part, reinterpret_cast<unsigned long long *>(bw),
-      reinterpret_cast<unsigned long long *>(cut), reinterpret_cast<unsigned long long *>(bad));
+      reinterpret_cast<unsigned long long *>(cut), reinterpret_cast<unsigned long long *>(bad), status);
   KMP_LAUNCHED("cut_bw");
 }
 
@@ -1242,22 +1259,21 @@ void cut_and_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw
   cudaStream_t s = ctx().stream;
   KMP_CUDA(cudaMemsetAsync(bw_dev, 0, (size_t)k * sizeof(int64_t), s));
   KMP_CUDA(cudaMemsetAsync(cut_dev, 0, sizeof(int64_t), s));
-  launch_cut(g, part, k, bw_dev, cut_dev, nullptr);
-  k_cut_finish<<<1, 1, 0, s>>>(cut_dev, nullptr, nullptr);
-  KMP_LAUNCHED("cut_finish");
+  launch_cut(g, part, k, bw_dev, cut_dev, nullptr, nullptr);
+  k_half<<<1, 1, 0, s>>>(cut_dev);
+  KMP_LAUNCHED("half");
 }
 
 // Block weights, cut, the range check of the block ids and the status word in
-// one buffer: one clear, two kernels, one copy and one wait.
+// one buffer: one clear, one kernel, one copy and one wait.
 void cut_to_host(const Graph &g, const int32_t *part, int32_t k, std::vector<int64_t> &out) {
   Context &C = ctx();
   DBuf<int64_t> d((size_t)k + 3);
   d.zero();
-  launch_cut(g, part, k, d.p, d.p + k, d.p + k + 1);
-  k_cut_finish<<<1, 1, 0, C.stream>>>(d.p + k, C.d_status, d.p + k + 2);
-  KMP_LAUNCHED("cut_finish");
+  launch_cut(g, part, k, d.p, d.p + k, d.p + k + 1, C.d_status);
   out.resize((size_t)k + 3);
   to_host(out.data(), d.p, out.size());
+  out[k] /= 2;
 }
 
 }  // namespace kmp
