@@ -282,7 +282,7 @@ typedef struct {
                                  (256..2048) */
   int32_t hub_chunk;          /* edges per hub work unit (256..65536, power of two;
                                  default 2048) */
-  int32_t ip_blocks_per_sm;   /* bipartitioner CTAs per SM (1..8) */
+  int32_t ip_blocks_per_sm;   /* bipartitioner CTAs per SM (1..8; 3 are resident at most) */
   int32_t dense_hub_degree;   /* with few labels (refinement: labels are block ids), degree
                                  above which a node's rating is split over many CTAs into a
                                  dense per-label row instead of one CTA (512..2^30) */

@@ -505,8 +505,13 @@ __device__ int32_t lowest_admissible(const int32_t *room, int32_t k, int32_t c, 
 // the batch's members by node id (shared memory): -1 or the member
 __device__ __forceinline__ void memb_add(int32_t *mk, int32_t *mv, int32_t v, int32_t j) {
   uint32_t h = fmix32((uint32_t)v) & (MEMB - 1);
-  while (atomicCAS(&mk[h], HT_EMPTY, v) != HT_EMPTY) h = (h + 1) & (MEMB - 1);  // at most 32 of 64 slots
-  mv[h] = j;
+  for (int probe = 0; probe < MEMB; ++probe) {  // at most 32 of 64 slots are taken
+    if (atomicCAS(&mk[h], HT_EMPTY, v) == HT_EMPTY) {
+      mv[h] = j;
+      return;
+    }
+    h = (h + 1) & (MEMB - 1);
+  }
 }
 __device__ __forceinline__ int32_t memb_find(const int32_t *mk, const int32_t *mv, int32_t v) {
   uint32_t h = fmix32((uint32_t)v) & (MEMB - 1);

@@ -15,9 +15,9 @@
 //      far is infeasible;
 //   3. projects the best bipartition up the item's hierarchy and runs 2-way FM
 //      (one warp) on every level.
-// Scratch comes from a per-item region through a bump allocator; if a region
-// is too small the launch reports it and the host repeats the round with
-// larger regions, so results never depend on scratch sizes.
+// Scratch comes from a region per CTA through a bump allocator, reset for every
+// item; if a region is too small the launch reports it and the host repeats the
+// round with larger regions, so results never depend on scratch sizes.
 #include <algorithm>
 #include <cmath>
 #include <numeric>

@@ -6,8 +6,8 @@
 //   rate     : every node of the sub-round sums the edge weight to each
 //              neighbouring cluster (degree-binned: 4..32-lane groups with
 //              shuffles, a warp with a shared-memory hash table, a CTA with a
-//              shared-memory table, a CTA with a global table for very high
-//              degrees), picks the best admissible cluster K with
+//              shared-memory table, a wide CTA up to 8192 neighbours, many CTAs
+//              for hubs), picks the best admissible cluster K with
 //              w(K) + c(u) <= cap(K) by (rating desc, perm32 asc) and proposes
 //              it when it beats the own cluster.
 //   classify : a target whose total proposed weight fits is accepted whole;
