@@ -1131,7 +1131,8 @@ void project(int32_t n_fine, const int32_t *map, const int32_t *part_c, int32_t 
 // of those that end at or before it.  So a hub's row is shared by many warps and
 // a short row costs no round trip of its own (rows one after the other on the
 // warp that held their 32 nodes: R-MAT 2^22 1.48 ms, mesh of 2^24 nodes 1.41 ms;
-// for the cut alone).  Weights are summed in shared memory when k is small.  bad (nullable)
+// for the cut alone).  Tiles start at xadj[0]: entries before it belong to no row and
+// are not read.  Weights are summed in shared memory when k is small.  bad (nullable)
 // is set when a block id lies outside [0, k); such ids index nothing.
 constexpr int CUT_SBW = 2048;
 constexpr int CUT_TILE = 2048;
@@ -1160,8 +1161,9 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   unsigned long long c = 0;
-  for (int64_t tile = gw; tile * CUT_TILE < m; tile += nw) {
-    int64_t e = tile * CUT_TILE;
+  const int64_t m0 = xadj[0];
+  for (int64_t tile = gw; m0 + tile * CUT_TILE < m; tile += nw) {
+    int64_t e = m0 + tile * CUT_TILE;
     const int64_t e1 = e + CUT_TILE < m ? e + CUT_TILE : m;
     int64_t v0 = 0, hi = n - 1;  // the last row that starts at or before e
     while (v0 < hi) {
