@@ -53,7 +53,8 @@ def build_kmp(verbose: bool = False, extra=()) -> str:
     """Compile every csrc/*.cu for sm_103a (in parallel) and link libkmp.so."""
     os.makedirs(BUILD, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    hdrs = sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h")))
+    hdrs = sorted(h for pat in (os.path.join(CSRC, "*.cuh"), os.path.join(CSRC, "*.h"), os.path.join(INCLUDE, "*.h"))
+                  for h in glob.glob(pat))
     out = lib_path()
     nvcc = _nvcc()
     objs = []

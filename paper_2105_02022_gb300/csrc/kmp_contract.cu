@@ -22,6 +22,7 @@
 #include <climits>
 
 #include "kmp_internal.cuh"
+#include "kmp_plan.h"
 
 namespace kmp {
 
@@ -758,7 +759,9 @@ void launch_large_sort_smem(int32_t nc, const int32_t *rows, int32_t nrows, cons
 // The longest rows (rank r, entries [boff[r], boff[r + 1]) of all of them) are
 // ordered by a counting sort on (r, neighbour >> SEG_LO): such a segment holds
 // distinct neighbours within 2^SEG_LO ids, so a bitmap of the segment and its
-// popcount prefix give every entry's place.  Entries are taken one a thread,
+// popcount prefix give every entry's place.  The kernels take a batch of rows
+// (seg_batches; nearly always all of them), N entries from boff[0] on, and index
+// what they sort from there.  Entries are taken one a thread,
 // whatever the rows' lengths (a warp a row took 8.5 of the 73 ms that
 // contracting R-MAT 2^24 takes), read from the temporary rows, scattered once,
 // and written back in place.
@@ -774,7 +777,8 @@ __device__ __forceinline__ int32_t row_of(const int64_t *boff, int32_t nrows, in
 }
 __global__ void k_seg_hist(int64_t N, const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
                            const int32_t *tadj, int hb, int32_t *hist) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t e0 = boff[0];
+  for (int64_t i = e0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e0 + N; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t r = row_of(boff, nrows, i);
     atomicAdd(&hist[((int64_t)r << hb) | (tadj[toff[rows[r]] + (i - boff[r])] >> SEG_LO)], 1);
   }
@@ -782,7 +786,8 @@ __global__ void k_seg_hist(int64_t N, const int32_t *rows, int32_t nrows, const 
 __global__ void k_seg_scatter(int64_t N, const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
                               const int32_t *tadj, const int32_t *tw, int hb, const int32_t *off, int32_t *cur,
                               int32_t *ek, int32_t *ev) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t e0 = boff[0];
+  for (int64_t i = e0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < e0 + N; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t r = row_of(boff, nrows, i);
     const int64_t q = toff[rows[r]] + (i - boff[r]);
     const int32_t y = tadj[q];
@@ -807,7 +812,7 @@ __global__ void __launch_bounds__(256) k_seg_place(int64_t X, const int32_t *his
     if (d == 0) continue;
     const int64_t o = off[x];
     const int32_t r = (int32_t)(x >> hb);
-    const int64_t to = toff[rows[r]] + (o - boff[r]);
+    const int64_t to = toff[rows[r]] + (boff[0] + o - boff[r]);
 #pragma unroll
     for (int u = 0; u < PER; ++u) bm[tid * PER + u] = 0;
     __syncthreads();
@@ -833,28 +838,6 @@ __global__ void __launch_bounds__(256) k_seg_place(int64_t X, const int32_t *his
       tw[p] = ev[o + j];
     }
     __syncthreads();  // the next segment reuses the bitmap
-  }
-}
-// entries as (rank << bits | neighbour, weight) and back, for the radix sort
-// that serves coarse graphs whose segment counters would not fit int32
-__global__ void k_large_gather(int64_t N, const int32_t *rows, int32_t nrows, const int64_t *boff, const int64_t *toff,
-                               const int32_t *tadj, const int32_t *tw, int bits, uint64_t *ek, int32_t *ev) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t r = row_of(boff, nrows, i);
-    const int64_t q = toff[rows[r]] + (i - boff[r]);
-    ek[i] = ((uint64_t)r << bits) | (uint64_t)(uint32_t)tadj[q];
-    ev[i] = tw[q];
-  }
-}
-__global__ void k_large_place(int64_t N, const uint64_t *ek, const int32_t *ev, int bits, const int32_t *rows,
-                              const int64_t *boff, const int64_t *toff, int32_t *tadj, int32_t *tw) {
-  const uint64_t mask = (1ull << bits) - 1ull;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = (int64_t)(ek[i] >> bits);
-    const int64_t p = toff[rows[r]] + (i - boff[r]);
-    tadj[p] = (int32_t)(ek[i] & mask);
-    tw[p] = ev[i];
   }
 }
 
@@ -1054,38 +1037,29 @@ Graph contract_graph(const Graph &g, const int32_t *label, int32_t *map) {
     if (sc[2] > 0) {
       const int32_t nbig = sc[2];
       const int32_t *brows = slists.p + 2ll * nlarge;
-      DBuf<int64_t> bdeg(nbig), boff(nbig), btot(1);
+      DBuf<int64_t> bdeg(nbig), boff(nbig + 1);
       k_gather_deg<<<grid_for(nbig, 256), 256, 0, s>>>(brows, nbig, cdeg, bdeg);
       KMP_LAUNCHED("gather_deg");
-      scan_excl_i64(bdeg, boff, nbig, btot);
-      const int64_t NE = read1(btot.p);
+      scan_excl_i64(bdeg, boff, nbig, boff.p + nbig);
+      std::vector<int64_t> hoff((size_t)nbig + 1);
+      to_host(hoff.data(), boff.p, hoff.size());
       // (a row above SORT_L entries has more than 2^SEG_LO distinct neighbours, so
       // bits > SEG_LO here)
       const int hb = bits - SEG_LO;
-      const int64_t X = (int64_t)nbig << hb;
-      const int gridN = grid_for(NE, 256);
-      if (X > (int64_t)INT32_MAX / 2) {
-        // counters beyond int32 indexing (coarse graphs near 2^31 nodes): one
-        // key-value radix sort of (rank, neighbour) instead
-        DBuf<uint64_t> ek(NE), ektmp(NE);
-        DBuf<int32_t> ev(NE), evtmp(NE);
-        int rbits = 1;
-        while ((1ll << rbits) < (int64_t)nbig) ++rbits;
-        k_large_gather<<<gridN, 256, 0, s>>>(NE, brows, nbig, boff, toff, tadj, tw, bits, ek, ev);
-        KMP_LAUNCHED("large_gather");
-        radix_sort_kv(ek, ev, ektmp, evtmp, NE, rbits + bits);
-        k_large_place<<<gridN, 256, 0, s>>>(NE, ek, ev, bits, brows, boff, toff, tadj, tw);
-        KMP_LAUNCHED("large_place");
-      } else {
-        DBuf<int32_t> ek(NE), ev(NE), hist(X), off(X), cur(X), htot(1);
+      for (const auto &[r0, r1] : seg_batches(hoff.data(), nbig, hb, SEG_MAX_ENTRIES, SEG_MAX_COUNTERS)) {
+        const int32_t *rows = brows + r0;
+        const int64_t *off0 = boff.p + r0;
+        const int64_t NE = hoff[r1] - hoff[r0], X = (int64_t)(r1 - r0) << hb;
+        const int gridN = grid_for(NE, 256);
+        DBuf<int32_t> ek(NE), ev(NE), hist(X), off(X), cur(X);
         hist.zero();
         cur.zero();
-        k_seg_hist<<<gridN, 256, 0, s>>>(NE, brows, nbig, boff, toff, tadj, hb, hist);
+        k_seg_hist<<<gridN, 256, 0, s>>>(NE, rows, r1 - r0, off0, toff, tadj, hb, hist);
         KMP_LAUNCHED("seg_hist");
-        scan_excl_i32(hist, off, X, htot);
-        k_seg_scatter<<<gridN, 256, 0, s>>>(NE, brows, nbig, boff, toff, tadj, tw, hb, off, cur, ek, ev);
+        scan_excl_i32(hist, off, X, nullptr);
+        k_seg_scatter<<<gridN, 256, 0, s>>>(NE, rows, r1 - r0, off0, toff, tadj, tw, hb, off, cur, ek, ev);
         KMP_LAUNCHED("seg_scatter");
-        k_seg_place<<<grid_for(X, 1), 256, 0, s>>>(X, hist, off, hb, ek, ev, brows, boff, toff, tadj, tw);
+        k_seg_place<<<grid_for(X, 1), 256, 0, s>>>(X, hist, off, hb, ek, ev, rows, off0, toff, tadj, tw);
         KMP_LAUNCHED("seg_place");
       }
     }
