@@ -604,7 +604,9 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
   __shared__ uint32_t s_adj[BM_W], s_mask[BM_W], s_toff[BM_W + 1];
   __shared__ unsigned long long s_best[BM_W];
   __shared__ int32_t mk[MEMB], mv[MEMB];
-  __shared__ int32_t adjw[32][33];  // edge weights between the members of a small batch, where s_adj has the bit
+  // weight from member to member of a small batch, summed over the entries that join them
+  // (parallel ones count together), where s_adj has the bit; zero between batches
+  __shared__ int32_t adjw[32][33];
   __shared__ int32_t s_nb, s_B, s_ob, s_i, s_phase, s_done, s_large, s_hint;
   constexpr unsigned ALL = 0xFFFFFFFFu;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -615,6 +617,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
   }
   for (int32_t x = threadIdx.x; x < A.k; x += BM_T) room[x] = (int32_t)((int64_t)A.cap[x] - A.bw[x]);
   if (threadIdx.x < MEMB) mk[threadIdx.x] = HT_EMPTY;
+  for (int x = threadIdx.x; x < 32 * 33; x += BM_T) (&adjw[0][0])[x] = 0;
   if (threadIdx.x == 0) {
     s_ob = 0;
     s_i = -1;
@@ -775,7 +778,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
               const int32_t ib = memb_find(mk, mv, uu[r]);
               if (ib >= 0) {
                 atomicOr(&s_adj[jm[r]], 1u << ib);
-                adjw[jm[r]][ib] = wt[r];
+                atomicAdd(&adjw[jm[r]][ib], wt[r]);
               }
               ht_add(wk + s_toff[jm[r]], wv + s_toff[jm[r]], s_mask[jm[r]], bk[r], wt[r]);
             }
@@ -814,6 +817,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
           wk[x] = HT_EMPTY;
           wv[x] = 0;
         }
+        for (uint32_t x = madj; x; x &= x - 1) adjw[lane][__ffs(x) - 1] = 0;
         mk[lane] = HT_EMPTY;
         mk[lane + 32] = HT_EMPTY;
         if (lane == 0 && left != need) {
