@@ -37,10 +37,13 @@ static int guarded(F &&f) {
 }
 
 // ---------------------------------------------------------- validation
+// bad: error bits, and BAD_ORDER (no error) when a row's ids do not strictly increase
+constexpr unsigned long long BAD_ORDER = 32;
 __global__ void k_validate(int32_t n, const int64_t *xadj, const int32_t *adj, const int32_t *vw,
                            const int32_t *ew, int64_t m, unsigned long long *bad,
                            unsigned long long *ewsum) {
   unsigned long long s = 0;
+  bool rises = true;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     int64_t b = xadj[v], e = xadj[v + 1];
@@ -49,8 +52,11 @@ __global__ void k_validate(int32_t n, const int64_t *xadj, const int32_t *adj, c
       continue;
     }
     if (vw && vw[v] <= 0) atomicOr(bad, 2ull);
+    int32_t prev = -1;
     for (int64_t q = b; q < e; ++q) {
       int32_t u = adj[q];
+      if (u <= prev) rises = false;
+      prev = u;
       if (u < 0 || u >= n) atomicOr(bad, 4ull);
       else if (u == v) atomicOr(bad, 8ull);
       int32_t w = ew ? ew[q] : 1;
@@ -60,7 +66,9 @@ __global__ void k_validate(int32_t n, const int64_t *xadj, const int32_t *adj, c
   }
 #pragma unroll
   for (int mm = 16; mm > 0; mm >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, mm);
+  rises = __all_sync(0xFFFFFFFFu, rises);
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(ewsum, s);
+  if ((threadIdx.x & 31) == 0 && !rises) atomicOr(bad, BAD_ORDER);
 }
 
 __global__ void k_check_range(int64_t n, const int32_t *a, int32_t lo, int32_t hi,
@@ -118,7 +126,8 @@ static Graph make_graph(int32_t n, const int64_t *xadj, const int32_t *adj, cons
   }
   unsigned long long h[2];
   to_host(h, chk.p, 2);
-  if (h[0] || (h[1] / 2) >= (1ull << 31)) {
+  g.multi = (h[0] & BAD_ORDER) != 0;
+  if ((h[0] & ~BAD_ORDER) || (h[1] / 2) >= (1ull << 31)) {
     Graph t = g;
     free_graph(t);
     if (h[0] & 1) fail(KMP_ERR_ARG, "xadj is not a valid offset array");

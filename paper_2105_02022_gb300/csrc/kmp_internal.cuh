@@ -121,6 +121,7 @@ struct Graph {
   int32_t max_vw = 1;
   int64_t maxdeg = 0;
   int64_t n_isolated = 0;
+  bool multi = false;       // some row's ids do not strictly increase: it may hold parallel entries
   bool owned = true;
 };
 
