@@ -20,10 +20,10 @@
 // round with larger regions, so results never depend on scratch sizes.
 #include <algorithm>
 #include <cmath>
-#include <numeric>
 
 #include "kmp_internal.cuh"
 #include "kmp_mpnn.cuh"
+#include "kmp_plan.h"
 
 namespace kmp {
 
@@ -59,15 +59,15 @@ struct IPArgs {
   const ItemDesc *items;
   const int32_t *order;   // item processing order
   int32_t nitems;
-  int32_t *queue;         // work counter
+  int32_t *queue;         // items taken beyond the CTAs' first ones
   int32_t *oom;           // set when a scratch region was too small
   const int64_t *gx;      // induced CSR offsets over all members (n+1)
   const uint16_t *sadj;   // local neighbour ids (an item has at most IP_MAX_N nodes)
   const int32_t *sew;     // null: unit weights
   const int32_t *svw;
   int32_t *side_out;      // per member position
-  int32_t *scratch;       // a region of slot words per CTA, reused by its items
-  int64_t slot;
+  int32_t *scratch;       // CTA b's region, reused by its items: [region[b], region[b + 1])
+  const int64_t *region;
   // configuration
   int32_t S, ip_C, ip_lp_rounds, rep_random, rep_bfs, rep_ggg, fm_passes, fm_stop;
   int32_t conv_num, conv_den;
@@ -1456,7 +1456,8 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   const ItemDesc D = A.items[it];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (D.n == 0) return;
-  Bump B{A.scratch + (int64_t)blockIdx.x * A.slot, A.slot, 0, false};
+  const int64_t region = A.region[blockIdx.x];
+  Bump B{A.scratch + region, A.region[blockIdx.x + 1] - region, 0, false};
   int32_t n0 = D.n;
   int32_t *x0 = B.take(n0 + 1);
   if (B.oom) {
@@ -1768,13 +1769,13 @@ __global__ void __launch_bounds__(IPT, 3) k_ip_items(const __grid_constant__ IPA
   __shared__ int32_t s_it;
   extern __shared__ __align__(16) int32_t ipdyn[];  // working state, then the warps' tables
   int32_t *wkeys = ipdyn + A.dyn_words, *wvals = wkeys + IPW * A.wtab;
-  for (;;) {
-    if (threadIdx.x == 0) s_it = atomicAdd(A.queue, 1);
-    __syncthreads();
-    int32_t q = s_it;
-    __syncthreads();
-    if (q >= A.nitems) break;
+  // item b of the order first: the CTA's region is sized for it, and later ones are smaller
+  for (int32_t q = blockIdx.x; q < A.nitems;) {
     run_item<MULTI>(A, A.order[q], wkeys, wvals, ipdyn);
+    if (threadIdx.x == 0) s_it = gridDim.x + atomicAdd(A.queue, 1);
+    __syncthreads();
+    q = s_it;
+    __syncthreads();
   }
 }
 
@@ -2079,33 +2080,28 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
   DBuf<int32_t> side(n);
   side.zero();
   if (!items.empty()) {
-    // largest items first (work queue order does not change results)
-    std::vector<int32_t> order(items.size());
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b2) {
-      return (int64_t)items[a].n + items[a].m > (int64_t)items[b2].n + items[b2].m;
-    });
     DBuf<int32_t> dorder(items.size()), q(2);
-    to_dev(dorder.p, order.data(), order.size());
     bool learned = cfg.learned && proposer().W;
     int64_t mult = 1;
-    // one wave of CTAs that take items from the queue; each has one scratch
-    // region, sized for the largest item and reused, so that what the CTAs touch
-    // stays in L2 (a region per item spread 8192 items of 2048 nodes over 36 GB)
+    // One wave of CTAs that take items from the queue, largest first (the order does
+    // not change results); each has one scratch region and reuses it, so that what
+    // the CTAs touch stays in L2 (a region per item spread 8192 items of 2048 nodes
+    // over 36 GB).
     int64_t maxn = 0;
-    for (auto &d : items) maxn = std::max<int64_t>(maxn, d.n);
+    std::vector<int64_t> words;
+    for (auto &d : items) {
+      maxn = std::max<int64_t>(maxn, d.n);
+      words.push_back(ip_scratch_words(d.n, d.m, learned ? 2 * MF + 3 * MH + 4 : 0));
+    }
     const int per_sm = std::min<int>(C.tune.ip_blocks_per_sm, 3);
     const int gridip = (int)std::min<int64_t>((int64_t)items.size(), (int64_t)C.sms * per_sm);
     for (int attempt = 0; attempt < 6; ++attempt, mult *= 4) {
-      int64_t slot = 0;
-      for (auto &d : items) {
-        int64_t nP = next_pow2((uint64_t)std::max(d.n, 2));
-        int64_t mP = next_pow2((uint64_t)std::max(d.m, 2));
-        slot = std::max<int64_t>(slot, mult * (104ll * d.n + 64ll * nP + 16ll * d.m + 8ll * mP + 2048 +
-                                      (learned ? (int64_t)(2 * MF + 3 * MH + 4) * d.n + 64 : 0)));
-      }
+      const IPRegions plan = ip_regions(words, gridip, mult);
       DBuf<ItemDesc> ditems(items.size());
-      DBuf<int32_t> scratch(slot * gridip);
+      DBuf<int64_t> dregion(plan.region.size());
+      DBuf<int32_t> scratch(plan.region.back());
+      to_dev(dorder.p, plan.order.data(), plan.order.size());
+      to_dev(dregion.p, plan.region.data(), plan.region.size());
       to_dev(ditems.p, items.data(), items.size());
       q.zero();
       IPArgs A;
@@ -2120,7 +2116,7 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
       A.svw = svw;
       A.side_out = side;
       A.scratch = scratch;
-      A.slot = slot;
+      A.region = dregion;
       A.S = cfg.subrounds;
       A.ip_C = cfg.ip_C;
       A.ip_lp_rounds = cfg.ip_lp_rounds;
