@@ -1099,18 +1099,32 @@ void project(int32_t n_fine, const int32_t *map, const int32_t *part_c, int32_t 
   KMP_LAUNCHED("project");
 }
 
-// Block weights node by node, then the cut by equal shares of the entries: a warp
-// takes CUT_TILE consecutive entries, finds the row they start in by one search,
-// and reads the ends and blocks of 32 rows at a time; an entry's row is the number
-// of those that end at or before it.  So a hub's row is shared by many warps and
-// a short row costs no round trip of its own (rows one after the other on the
-// warp that held their 32 nodes: R-MAT 2^22 1.48 ms, mesh of 2^24 nodes 1.41 ms;
-// for the cut alone).  Tiles start at xadj[0]: entries before it belong to no row and
-// are not read.  Weights are summed in shared memory when k is small.  bad (nullable)
-// is set when a block id lies outside [0, k); such ids index nothing.
+// Block weights node by node, then the cut by equal shares of rows and entries: a warp
+// takes CUT_TILE consecutive ones (a row counts for one more than its entries),
+// finds the row they start in, and reads the ends and blocks of 32 rows at a time; an
+// entry's row is the number of those that end at or before it.  So a hub's row is
+// shared by many warps, and a short row costs no round trip of its own (rows one
+// after the other on the warp that held their 32 nodes: R-MAT 2^22 1.48 ms, mesh of
+// 2^24 nodes 1.41 ms; for the cut alone).  Shares of the entries alone let one warp
+// walk all rows without entries between two of its own: 2^24 isolated nodes took
+// 293 ms, every 64th of 2^20 nodes joined 2.0 ms.  Entries before xadj[0] belong
+// to no row and are not read.  Weights are summed in shared memory when k is small.
+// bad (nullable) is set when a block id lies outside [0, k); such ids index nothing.
 constexpr int CUT_SBW = 2048;
-constexpr int CUT_TILE = 2048;
+constexpr int CUT_TILE = 2304;  // 2048 entries in rows of 8, with their rows
 constexpr int CUT_U = 4;
+// The last row v with v + xadj[v] - xadj[0] <= d (d >= 0), by a warp, 32 positions a read
+__device__ __forceinline__ int64_t share_row(const int64_t *__restrict__ xadj, int32_t n, int64_t d) {
+  const int lane = threadIdx.x & 31;
+  int64_t st = 1, v = 0;
+  while (32 * st < n) st *= 32;
+  d += xadj[0];
+  for (; st > 0; st /= 32) {
+    const int64_t p = v + st * (lane + 1);
+    v += st * __popc(__ballot_sync(0xFFFFFFFFu, p < n && p + xadj[p] <= d));  // rises with p
+  }
+  return v;
+}
 __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k, const int64_t *__restrict__ xadj,
                                                 const int32_t *__restrict__ adj, const int32_t *__restrict__ vw,
                                                 const int32_t *__restrict__ ew, const int32_t *__restrict__ part,
@@ -1135,16 +1149,11 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   unsigned long long c = 0;
-  const int64_t m0 = xadj[0];
-  for (int64_t tile = gw; m0 + tile * CUT_TILE < m; tile += nw) {
-    int64_t e = m0 + tile * CUT_TILE;
-    const int64_t e1 = e + CUT_TILE < m ? e + CUT_TILE : m;
-    int64_t v0 = 0, hi = n - 1;  // the last row that starts at or before e
-    while (v0 < hi) {
-      const int64_t mid = (v0 + hi + 1) >> 1;
-      if (xadj[mid] <= e) v0 = mid;
-      else hi = mid - 1;
-    }
+  const int64_t m0 = xadj[0], total = n + m - m0;
+  for (int64_t tile = gw; tile * CUT_TILE < total; tile += nw) {
+    const int64_t d = tile * CUT_TILE, d1 = d + CUT_TILE;
+    int64_t v0 = share_row(xadj, n, d), e = m0 + d - v0, e1 = m;
+    if (d1 < total) e1 = m0 + d1 - share_row(xadj, n, d1);
     while (e < e1) {
       const int64_t v = v0 + lane;
       const int64_t end = v < n ? xadj[v + 1] : m;
@@ -1223,7 +1232,7 @@ void block_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw_d
 // bad, status (nullable): as in k_cut_bw; the status word goes behind bad
 static void launch_cut(const Graph &g, const int32_t *part, int32_t k, int64_t *bw, int64_t *cut, int64_t *bad,
                        const int *status) {
-  const int64_t work = std::max<int64_t>(g.n, ceil_div(g.m, CUT_TILE) * 32);
+  const int64_t work = std::max<int64_t>(g.n, ceil_div(g.n + g.m, CUT_TILE) * 32);
   k_cut_bw<<<grid_for(work, 256, 8), 256, 0, ctx().stream>>>(
       g.n, g.m, k, g.xadj, g.adj, g.vw, g.ew, part, reinterpret_cast<unsigned long long *>(bw),
       reinterpret_cast<unsigned long long *>(cut), reinterpret_cast<unsigned long long *>(bad), status);
