@@ -604,12 +604,11 @@ int kmp_cut(const kmp_graph *g, const kmp_vid *part, int32_t k, int64_t *cut_out
   return guarded([&] {
     if (!g || !part) fail(KMP_ERR_ARG, "NULL argument");
     if (k < 1) fail(KMP_ERR_ARG, "k < 1");
-    std::vector<int64_t> r;
-    cut_to_host(g->g, part, k, r);
-    if (r[k + 2]) sync_and_check("cut");  // clears the word and reports it
-    if (r[k + 1]) fail(KMP_ERR_ARG, "part: value out of range");
-    if (bw_out) memcpy(bw_out, r.data(), (size_t)k * sizeof(int64_t));
-    if (cut_out) *cut_out = r[k];
+    int64_t r[3];
+    cut_to_host(g->g, part, k, r, bw_out);
+    if (r[2]) sync_and_check("cut");  // clears the word and reports it
+    if (r[1]) fail(KMP_ERR_ARG, "part: value out of range");
+    if (cut_out) *cut_out = r[0];
   });
 }
 

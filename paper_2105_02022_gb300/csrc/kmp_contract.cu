@@ -20,6 +20,7 @@
 // Also: projection (Algorithm 1), cut and block weights (Section 2), and the
 // per-graph facts the other kernels need (max degree, isolated nodes, weights).
 #include <climits>
+#include <cstring>
 
 #include "kmp_internal.cuh"
 #include "kmp_plan.h"
@@ -1249,16 +1250,26 @@ void cut_and_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw
   KMP_LAUNCHED("half");
 }
 
-// Block weights, cut, the range check of the block ids and the status word in
-// one buffer: one clear, one kernel, one copy and one wait.
-void cut_to_host(const Graph &g, const int32_t *part, int32_t k, std::vector<int64_t> &out) {
+// Cut, the range check of the block ids, the status word and the block weights behind
+// them in one buffer: one clear, one kernel, one copy and one wait while the weights
+// are few.  Many go straight to the caller's array in a copy of their own, none are
+// copied when not asked for (k = 2^20 on a mesh of 2^21 nodes: 0.94 ms through a second
+// host buffer, 0.32 like this).
+constexpr int32_t CUT_ONE_COPY = 4096;
+void cut_to_host(const Graph &g, const int32_t *part, int32_t k, int64_t head[3], int64_t *bw) {
   Context &C = ctx();
   DBuf<int64_t> d((size_t)k + 3);
   d.zero();
-  launch_cut(g, part, k, d.p, d.p + k, d.p + k + 1, C.d_status);
-  out.resize((size_t)k + 3);
-  to_host(out.data(), d.p, out.size());
-  out[k] /= 2;
+  launch_cut(g, part, k, d.p + 3, d.p, d.p + 1, C.d_status);
+  const bool one = bw && k <= CUT_ONE_COPY;
+  std::vector<int64_t> h(3 + (one ? (size_t)k : 0));
+  to_host(h.data(), d.p, h.size());
+  head[0] = h[0] / 2;
+  head[1] = h[1];
+  head[2] = h[2];
+  if (!bw || head[1] || head[2]) return;
+  if (one) memcpy(bw, h.data() + 3, (size_t)k * sizeof(int64_t));
+  else to_host(bw, d.p + 3, (size_t)k);
 }
 
 }  // namespace kmp

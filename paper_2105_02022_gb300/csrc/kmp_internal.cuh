@@ -273,9 +273,9 @@ void project(int32_t n_fine, const int32_t *map, const int32_t *part_c, int32_t 
 // cut and block weights (device out arrays: bw int64[k], cut int64[1])
 void cut_and_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw_dev,
                      int64_t *cut_dev);
-// the same to the host, out: block weights [k], cut, nonzero when a block id is
-// outside [0, k) (weights and cut then unspecified), device status word
-void cut_to_host(const Graph &g, const int32_t *part, int32_t k, std::vector<int64_t> &out);
+// the same to the host: head holds the cut, nonzero when a block id is outside [0, k), and
+// the device status word; bw (nullable) gets the weights when both of those are 0
+void cut_to_host(const Graph &g, const int32_t *part, int32_t k, int64_t head[3], int64_t *bw);
 // block weights only (device out int64[k])
 void block_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw_dev);
 // refinement wrapper: caps host int32[k]; returns the cut when want_cut, else 0
