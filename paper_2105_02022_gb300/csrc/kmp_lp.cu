@@ -1458,7 +1458,14 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
 // dependent reads a sub-round on one SM.  Partition of a 32,768-node mesh, whose
 // four coarse levels run here: 9.6 -> 6.9 ms.  The order of the node list inside a
 // (sub-round, bin) is arbitrary here; nothing depends on it.
+// One SM rates about 32 entries a round trip of its warps, so the bound on entries
+// is what keeps dense graphs with the kernels of all SMs.  Clustering and 8-way
+// refinement in one launch over the separate kernels, 4096 nodes: meshes of 32,000
+// entries 0.52..0.82 of the time, of 63,000 0.64..1.18, of 125,000 0.93..1.58; random
+// graphs of 33,000 0.70..1.07, of 130,000 1.67, of 516,000 2.8..3.3.  Break-even moves
+// to 60,000..90,000 entries at 500..2000 nodes.
 constexpr int32_t SMALL_N = 4096;
+constexpr int64_t SMALL_M = 32768;
 constexpr int64_t SMALL_DEG = 256;
 constexpr int SMALL_T = 1024;
 constexpr size_t SMALL_SMEM = (size_t)(SMALL_T / 32) * (2 * WARP_TAB * sizeof(int32_t) + WARP_TAB / 2 * sizeof(uint16_t));
@@ -1869,7 +1876,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
       }
     }
   };
-  if (n <= SMALL_N && g.maxdeg <= SMALL_DEG && !C.profile) {
+  if (n <= SMALL_N && g.m <= SMALL_M && g.maxdeg <= SMALL_DEG && !C.profile) {
     std::vector<LPRound> hr(rounds);
     for (int r = 0; r < rounds; ++r) {
       const uint64_t rk = key_step(basekey, (uint64_t)r);
