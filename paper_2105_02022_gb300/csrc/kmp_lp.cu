@@ -120,6 +120,7 @@ struct LPArgs {
   int64_t huge_deg;            // largest degree of bin 5 (many labels: <= HUGE_DEG_MAX)
   int64_t mid_deg;             // largest degree of bin 6; above it a node is a hub
   int64_t hub_chunk;           // edges per hub insert work unit
+  int32_t apply_row;           // longest row that k_apply marks itself
   int32_t nlab;
   int32_t S;
   LPRound *R;                  // current round (written by k_round_begin)
@@ -1359,14 +1360,21 @@ __global__ void __launch_bounds__(256) k_resolve(LPArgs A) {
   if (nslots > 0) resolve_slots(A, nslots, blockIdx.x, gridDim.x);
 }
 
-// A warp takes 32 list entries.  The rows of its moved nodes (up to APPLY_ROW
-// entries each) are walked together, an entry per lane: the entry's owner comes
-// from a prefix sum of the row lengths, so consecutive lanes read consecutive
-// entries and mark close-by neighbours in few sectors.  One row a thread cost a
-// sector per lane and entry.  What is left is the random sectors of labels and
-// weights.  Partition of a 2^24-node mesh, degree 16, k = 2^14, all k_apply
-// launches: 16.6 -> 13.3 ms.
-constexpr int APPLY_ROW = 256;
+// A warp takes 32 list entries.  The rows of its moved nodes (up to A.apply_row
+// entries each; longer ones go to k_scatter_big) are walked together, an entry per
+// lane: the entry's owner comes from a prefix sum of the row lengths, so consecutive
+// lanes read consecutive entries and mark close-by neighbours in few sectors.  One
+// row a thread cost a sector per lane and entry.  What is left is the random sectors
+// of labels and weights.  Partition of a 2^24-node mesh, degree 16, k = 2^14, all
+// k_apply launches: 16.6 -> 13.3 ms.
+// A warp walks its rows alone, so long rows pay only where a sub-round's list fills
+// the chip with warps: up to 256 entries from APPLY_MANY nodes on (8 sub-rounds of
+// 2048 warps), else 96, and a CTA for each longer row.  Clustering of random graphs
+// of 100 neighbours, 64 / 256 entries: 4096 nodes 1.85 / 2.06 ms, 65,536 nodes 3.02 /
+// 3.38, 262,144 nodes 4.73 / 4.98, 1 M nodes 12.4 / 12.3 (a mesh 8.2 / 7.7); of 50
+// neighbours, 65,536 nodes 2.57 / 2.47, hence 96.
+constexpr int APPLY_ROW = 96, APPLY_ROW_MANY = 256;
+constexpr int32_t APPLY_MANY = 1 << 19;
 // first: the list entry of the warp's lane 0
 __device__ __forceinline__ void apply_range(const LPArgs &A, int64_t first, int64_t hi, int64_t stride) {
   uint8_t *__restrict__ nxt = act_nxt(A);
@@ -1388,7 +1396,7 @@ __device__ __forceinline__ void apply_range(const LPArgs &A, int64_t first, int6
         ++moved;
         beg = A.xadj[u];
         const int64_t d = A.xadj[u + 1] - beg;
-        if (d > APPLY_ROW) A.bigmove[atomicAdd(&A.ctr[2], 1)] = u;  // neighbours marked by k_scatter_big
+        if (d > A.apply_row) A.bigmove[atomicAdd(&A.ctr[2], 1)] = u;  // neighbours marked by k_scatter_big
         else deg = (int32_t)d;
       } else if (A.fav) {
         A.fav[u] = T;
@@ -1742,6 +1750,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   A.huge_deg = huge;
   A.mid_deg = mid;
   A.hub_chunk = C.tune.hub_chunk;
+  A.apply_row = n < APPLY_MANY ? APPLY_ROW : APPLY_ROW_MANY;
   A.nlab = nlab;
   A.S = S;
 
@@ -1835,7 +1844,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
       KMP_LAUNCHED("resolve");
       k_apply<<<grid_commit, 256, 0, st>>>(A, s);
       KMP_LAUNCHED("apply");
-      if (g.maxdeg > APPLY_ROW) {
+      if (g.maxdeg > A.apply_row) {
         k_scatter_big<<<4 * C.sms, 256, 0, st>>>(A);
         KMP_LAUNCHED("scatter_big");
       }
@@ -1889,6 +1898,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
       KMP_CUDA(cudaFuncSetAttribute(k_lp_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
       attr = true;
     }
+    A.apply_row = (int32_t)SMALL_DEG;  // it marks every row itself
     k_lp_small<<<1, SMALL_T, SMALL_SMEM, stream>>>(A, dr, rounds);
     KMP_LAUNCHED("lp_small");
   } else if (C.tune.lp_graphs) {
