@@ -61,7 +61,10 @@ def build_kmp(verbose: bool = False, extra=()) -> str:
 
     def compile_one(src):
         obj = os.path.join(BUILD, os.path.basename(src) + ".o")
-        if _stale(obj, [src] + hdrs):
+        with open(src) as f:  # a second build of another source includes it
+            text = f.read()
+        included = [x for x in srcs if f'#include "{os.path.basename(x)}"' in text]
+        if _stale(obj, [src] + included + hdrs):
             cmd = [nvcc, *ARCH, *NVCC_FLAGS, *extra, "-c", src, "-o", obj + ".tmp"]
             if verbose:
                 cmd.insert(1, "-Xptxas=-v")

@@ -35,6 +35,7 @@ struct BalArgs {
   const int32_t *adj;
   const int32_t *vw;
   const int32_t *ew;
+  int32_t multi;         // the graph may hold parallel entries
   int32_t *part;
   int64_t *bw;
   const int32_t *cap;
@@ -604,8 +605,8 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
   __shared__ uint32_t s_adj[BM_W], s_mask[BM_W], s_toff[BM_W + 1];
   __shared__ unsigned long long s_best[BM_W];
   __shared__ int32_t mk[MEMB], mv[MEMB];
-  // weight from member to member of a small batch, summed over the entries that join them
-  // (parallel ones count together), where s_adj has the bit; zero between batches
+  // weight from member to member of a small batch, where s_adj has the bit; parallel entries
+  // (A.multi) are summed, and their sums are zero between batches
   __shared__ int32_t adjw[32][33];
   __shared__ int32_t s_nb, s_B, s_ob, s_i, s_phase, s_done, s_large, s_hint;
   constexpr unsigned ALL = 0xFFFFFFFFu;
@@ -778,7 +779,8 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
               const int32_t ib = memb_find(mk, mv, uu[r]);
               if (ib >= 0) {
                 atomicOr(&s_adj[jm[r]], 1u << ib);
-                atomicAdd(&adjw[jm[r]][ib], wt[r]);
+                if (A.multi) atomicAdd(&adjw[jm[r]][ib], wt[r]);
+                else adjw[jm[r]][ib] = wt[r];
               }
               ht_add(wk + s_toff[jm[r]], wv + s_toff[jm[r]], s_mask[jm[r]], bk[r], wt[r]);
             }
@@ -817,7 +819,8 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
           wk[x] = HT_EMPTY;
           wv[x] = 0;
         }
-        for (uint32_t x = madj; x; x &= x - 1) adjw[lane][__ffs(x) - 1] = 0;
+        if (A.multi)
+          for (uint32_t x = madj; x; x &= x - 1) adjw[lane][__ffs(x) - 1] = 0;
         mk[lane] = HT_EMPTY;
         mk[lane + 32] = HT_EMPTY;
         if (lane == 0 && left != need) {
@@ -993,6 +996,7 @@ int64_t balance(const Graph &g, int32_t k, const int32_t *caps_host, int32_t *pa
   A.k = k;
   A.xadj = g.xadj;
   A.adj = g.adj;
+  A.multi = g.multi ? 1 : 0;
   A.vw = g.vw;
   A.ew = g.ew;
   A.part = part;

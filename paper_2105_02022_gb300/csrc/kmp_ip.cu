@@ -25,6 +25,10 @@
 #include "kmp_mpnn.cuh"
 #include "kmp_plan.h"
 
+#ifndef KMP_IP_MULTI
+#define KMP_IP_MULTI 0
+#endif
+
 namespace kmp {
 
 constexpr int IPT = 256;
@@ -81,6 +85,10 @@ struct IPArgs {
   int32_t dyn_words;  // words of the phases' working state in shared memory
 };
 
+#if KMP_IP_MULTI
+namespace multi {
+#endif
+
 // A level of an item.  Neighbour ids take 16 bits and unit weights are not
 // stored, so the 2048-node items of a degree-16 mesh take 64 KB each instead of
 // 250: what the resident items read again and again stays in L2.
@@ -94,18 +102,28 @@ struct LG {
 };
 __device__ __forceinline__ int32_t lg_w(const LG &g, int32_t q) { return g.ew ? g.ew[q] : 1; }
 
-struct Bump {
+// The CTA's scratch region: base and words, in shared memory, so that a take holds no
+// registers for them (4096 items of 200..4000 nodes: 32.3 ms with both in registers,
+// 560 bytes of spill loads a thread; 30.4 like this, 288)
+struct Region {
   int32_t *base;
-  int64_t cap, top;
+  int64_t cap;
+};
+__device__ __forceinline__ Region &region() {
+  __shared__ Region r;
+  return r;
+}
+struct Bump {
+  int64_t top;
   bool oom;
   __device__ int32_t *take(int64_t cnt) {
     int64_t t = (top + 1) & ~1ll;
-    if (oom || t + cnt > cap) {
+    if (oom || t + cnt > region().cap) {
       oom = true;
-      return base;  // never dereferenced: callers check oom
+      return region().base;  // never dereferenced: callers check oom
     }
     top = t + cnt;
-    return base + t;
+    return region().base + t;
   }
 };
 
@@ -885,15 +903,16 @@ __device__ __forceinline__ bool fm_less(int32_t ia, int64_t oa, int64_t ca, int3
   return ca < cb;
 }
 
-// MULTI: the input graph's rows may hold parallel entries, so lanes that walk a row
-// may change one node's key or gain at once and add atomically.  4096 items of
-// 200..4000 nodes: 31.8 ms with plain updates, 32.5 with atomics, so graphs whose
-// rows strictly increase (known from their creation) keep the plain ones.
-template <bool MULTI>
-__device__ __forceinline__ void fm_add(int32_t *x, int32_t d) {
-  if (MULTI) atomicAdd(x, d);
-  else *x += d;
-}
+// A graph whose rows may hold parallel entries (Graph::multi) has a build of these
+// kernels of its own (kmp_ip_multi.cu): lanes that walk a row may change one node's
+// key or gain at once, so they add atomically.  With atomics everywhere 4096 items of
+// 200..4000 nodes take 32.5 ms instead of 31.8; as template variants in this file the
+// plain kernel took 2 % longer on small items, for its registers.
+#if KMP_IP_MULTI
+#define FM_ADD(x, k, d) atomicAdd(&(x), d)
+#else
+#define FM_ADD(x, k, d) ((x) = (k) + (d))
+#endif
 
 // The moves of one FM pass by one warp, from keys already set: repeatedly the
 // better feasible top of the two sides (gain desc, id asc), until no unlocked
@@ -910,7 +929,7 @@ __device__ __forceinline__ void fm_add(int32_t *x, int32_t d) {
 // Measured a step in place: 780 cycles with all of a level of up to 256 nodes in
 // shared memory (about 1900 with 64-bit selection keys reduced by shuffles), 2200
 // for 2048 nodes with the entries in L2 (3800).
-template <int GRAPH, bool MULTI>
+template <int GRAPH>
 __device__ __forceinline__ int32_t fm_pass_packed(int32_t fm_stop, int32_t n, const FMState F, int32_t idbits,
                                                   int32_t bias, int32_t L0, int32_t L1, int32_t &W0, int32_t &W1,
                                                   int32_t &cut) {
@@ -969,7 +988,7 @@ __device__ __forceinline__ int32_t fm_pass_packed(int32_t fm_stop, int32_t n, co
     const int32_t sg = from0 ? 1 << (idbits + 1) : -(1 << (idbits + 1));
     for (int32_t q = qb + lane; q < qe; q += 32) {
       const int32_t x = adj[q], d = (unit ? 1 : ew[q]) * sg, k = key[x];
-      if (k) fm_add<MULTI>(&key[x], d);
+      if (k) FM_ADD(key[x], k, d);
     }
     if (lane == 0) {
       key[v] = 0;
@@ -1002,7 +1021,6 @@ __device__ __forceinline__ int32_t fm_pass_packed(int32_t fm_stop, int32_t n, co
 }
 
 // the same pass from plain gains, for levels whose keys do not pack
-template <bool MULTI>
 __device__ __noinline__ int32_t fm_pass_plain(int32_t fm_stop, int32_t n, const FMState F, int64_t L0, int64_t L1,
                                               int32_t &W0, int32_t &W1, int32_t &cut) {
   constexpr unsigned ALL = 0xFFFFFFFFu;
@@ -1045,7 +1063,7 @@ __device__ __noinline__ int32_t fm_pass_plain(int32_t fm_stop, int32_t n, const 
     const int32_t v = from0 ? v0 : v1, to = from0 ? 1 : 0;
     for (int32_t q = F.xadj[v] + lane; q < F.xadj[v + 1]; q += 32) {
       const int32_t x = F.adj[q], d = 2 * (F.ew ? F.ew[q] : 1), k = F.key[x];
-      if (k != FM_LOCKED) fm_add<MULTI>(&F.key[x], fm_side(F.bits, x) == to ? -d : d);
+      if (k != FM_LOCKED) FM_ADD(F.key[x], k, fm_side(F.bits, x) == to ? -d : d);
     }
     if (lane == 0) {
       F.key[v] = FM_LOCKED;
@@ -1076,19 +1094,17 @@ __device__ __noinline__ int32_t fm_pass_plain(int32_t fm_stop, int32_t n, const 
   return best_step;
 }
 
-template <bool MULTI>
 __device__ __forceinline__ int32_t pass_moves(int32_t fm_stop, int32_t n, const FMState F, int32_t idbits,
                                               int32_t bias, int32_t L0, int32_t L1, int32_t &W0, int32_t &W1,
                                               int32_t &cut) {
-  if (idbits < 0) return fm_pass_plain<MULTI>(fm_stop, n, F, L0, L1, W0, W1, cut);
-  if (F.eoff >= 0) return fm_pass_packed<2, MULTI>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
-  if (F.off >= 0) return fm_pass_packed<1, MULTI>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
-  return fm_pass_packed<0, MULTI>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+  if (idbits < 0) return fm_pass_plain(fm_stop, n, F, L0, L1, W0, W1, cut);
+  if (F.eoff >= 0) return fm_pass_packed<2>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+  if (F.off >= 0) return fm_pass_packed<1>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+  return fm_pass_packed<0>(fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
 }
 
 // 2-way FM by one warp (same decisions as the oracle) from the sides in
 // F.bits, which it improves; returns the final cut, W0 and W1 the side weights
-template <bool MULTI>
 __device__ int32_t warp_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, const FMState F, int32_t &W0,
                            int32_t &W1) {
   const int lane = threadIdx.x & 31;
@@ -1128,7 +1144,7 @@ __device__ int32_t warp_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, c
       }
     }
     __syncwarp();
-    if (pass_moves<MULTI>(A.fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut) == 0) break;
+    if (pass_moves(A.fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut) == 0) break;
   }
   return cut;
 }
@@ -1136,7 +1152,6 @@ __device__ int32_t warp_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, c
 // the same FM with the whole CTA: cut, keys and weights by all warps (a
 // half-warp per node and four nodes at a time, so the loads of four rows are in
 // flight together), the moves by warp 0
-template <bool MULTI>
 __device__ void cta_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, const FMState F) {
   __shared__ int32_t s_kept;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1204,7 +1219,7 @@ __device__ void cta_fm(const IPArgs &A, int32_t n, int32_t L0, int32_t L1, const
     }
     __syncthreads();  // the keys are complete
     if (w == 0) {
-      const int32_t kept = pass_moves<MULTI>(A.fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
+      const int32_t kept = pass_moves(A.fm_stop, n, F, idbits, bias, L0, L1, W0, W1, cut);
       if (lane == 0) s_kept = kept;
     }
     __syncthreads();
@@ -1266,7 +1281,6 @@ __device__ FMState cta_fm_state(const LG &g, int32_t *dyn, int32_t dyn_words, in
 // portfolio initial bipartition by one warp: algo 0 random, 1 BFS, 2 GGG
 // algo 0 random, 1 BFS, 2 greedy graph growing, 3 learned (first fit in the
 // order of `score`, like random with a learned order)
-template <bool MULTI>
 __device__ void warp_initial(int algo, const LG &g, int32_t t0, uint64_t key, int32_t *side,
                              uint64_t *oh, int32_t *ov, int32_t *gain, int32_t *vis, int32_t *queue,
                              const float *score) {
@@ -1335,7 +1349,8 @@ __device__ void warp_initial(int algo, const LG &g, int32_t t0, uint64_t key, in
       if (v >= 0) {
         if (lane == 0) side[v] = 0;
         W0 += g.vw[v];
-        for (int32_t q = g.xadj[v] + lane; q < g.xadj[v + 1]; q += 32) fm_add<MULTI>(&gain[g.adj[q]], 2 * lg_w(g, q));
+        for (int32_t q = g.xadj[v] + lane; q < g.xadj[v + 1]; q += 32)
+          FM_ADD(gain[g.adj[q]], gain[g.adj[q]], 2 * lg_w(g, q));
         __syncwarp();
       }
       uint64_t best = 0;
@@ -1402,7 +1417,6 @@ __device__ void record_sample(const SampleSink &K, const LG &h, const int32_t *s
 // the item graph with the finest level's caps.  1: feasible, written to
 // side_out; 0: a cap is broken (the caller runs the plain method); -1: the
 // item's scratch is too small.
-template <bool MULTI>
 __device__ int item_learned(const IPArgs &A, const ItemDesc &D, const LG &g, Bump &B, int32_t *dyn) {
   const int w = threadIdx.x >> 5;
   const int32_t n = g.n;
@@ -1420,13 +1434,13 @@ __device__ int item_learned(const IPArgs &A, const ItemDesc &D, const LG &g, Bum
   mp_features(G, key_step(D.key, DOM_LEARNED), X, d1, d2);
   mp_forward_cta(G, A.W, X, scr, sc);
   __syncthreads();
-  if (w == 0) warp_initial<MULTI>(3, g, D.t0, 0, side, oh, ov, nullptr, nullptr, nullptr, sc);
+  if (w == 0) warp_initial(3, g, D.t0, 0, side, oh, ov, nullptr, nullptr, nullptr, sc);
   __syncthreads();
   const int32_t c0 = level_cap(D.L0, D.t0, g.maxc), c1 = level_cap(D.L1, D.t1, g.maxc);
   const FMState F = cta_fm_state(g, dyn, A.dyn_words, fmbuf);
   cta_set_bits(F.bits, n, [&](int32_t v) { return side[v]; });
   __syncthreads();
-  cta_fm<MULTI>(A, n, c0, c1, F);
+  cta_fm(A, n, c0, c1, F);
   __syncthreads();
   int64_t W0 = 0, W1 = 0;
   for (int32_t v = threadIdx.x; v < n; v += IPT) {
@@ -1441,7 +1455,6 @@ __device__ int item_learned(const IPArgs &A, const ItemDesc &D, const LG &g, Bum
   return 1;
 }
 
-template <bool MULTI>
 __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *wvals, int32_t *dyn) {
   __shared__ LG lv[IP_MAXL + 1];
   __shared__ int32_t *maps[IP_MAXL + 1];
@@ -1456,8 +1469,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   const ItemDesc D = A.items[it];
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (D.n == 0) return;
-  const int64_t region = A.region[blockIdx.x];
-  Bump B{A.scratch + region, A.region[blockIdx.x + 1] - region, 0, false};
+  Bump B{0, false};
   int32_t n0 = D.n;
   int32_t *x0 = B.take(n0 + 1);
   if (B.oom) {
@@ -1491,7 +1503,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   __syncthreads();
   if (A.learned_item) {
     const int64_t mark = B.top;
-    const int r = item_learned<MULTI>(A, D, lv[0], B, dyn);
+    const int r = item_learned(A, D, lv[0], B, dyn);
     if (r < 0) {
       if (threadIdx.x == 0) atomicExch(A.oom, 1);
       return;
@@ -1675,14 +1687,14 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
           if (phase == 1) r += first[a];
         }
         uint64_t key = a == 3 ? 0 : key_step(key_step(D.key, doms[a]), (uint64_t)r);
-        warp_initial<MULTI>(a, h, D.t0, key, side, oh, ov, F.key, vis, queue, score);
+        warp_initial(a, h, D.t0, key, side, oh, ov, F.key, vis, queue, score);
         for (int32_t v = lane; v < fm_pad(nH); v += 32) {
           const unsigned m = __ballot_sync(0xFFFFFFFFu, v < nH && side[v] != 0);
           if (lane == 0) F.bits[v >> 5] = m;
         }
         __syncwarp();
         int32_t W0, W1;
-        const int64_t cut = warp_fm<MULTI>(A, nH, hL0, hL1, F, W0, W1);
+        const int64_t cut = warp_fm(A, nH, hL0, hL1, F, W0, W1);
         int64_t o0 = (int64_t)W0 - hL0, o1 = (int64_t)W1 - hL1;
         int64_t o = o0 > o1 ? o0 : o1;
         int32_t inf = o > 0;
@@ -1753,7 +1765,7 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
     const FMState F = cta_fm_state(g, dyn, A.dyn_words, fmbuf);
     cta_set_bits(F.bits, g.n, [&](int32_t v) { return cur[map[v]]; });
     __syncthreads();
-    cta_fm<MULTI>(A, g.n, level_cap(D.L0, D.t0, g.maxc), level_cap(D.L1, D.t1, g.maxc), F);
+    cta_fm(A, g.n, level_cap(D.L0, D.t0, g.maxc), level_cap(D.L1, D.t1, g.maxc), F);
     __syncthreads();
     for (int32_t v = threadIdx.x; v < g.n; v += IPT) fine[v] = fm_side(F.bits, v);
     __syncthreads();
@@ -1764,20 +1776,44 @@ __device__ void run_item(const IPArgs &A, int32_t it, int32_t *wkeys, int32_t *w
   if (A.sink.counters && A.sink.item_level) record_sample(A.sink, lv[0], cur, D.key);
 }
 
-template <bool MULTI>
+#if KMP_IP_MULTI
+#define k_ip_items k_ip_items_multi
+#endif
 __global__ void __launch_bounds__(IPT, 3) k_ip_items(const __grid_constant__ IPArgs A) {
   __shared__ int32_t s_it;
   extern __shared__ __align__(16) int32_t ipdyn[];  // working state, then the warps' tables
   int32_t *wkeys = ipdyn + A.dyn_words, *wvals = wkeys + IPW * A.wtab;
   // item b of the order first: the CTA's region is sized for it, and later ones are smaller
-  for (int32_t q = blockIdx.x; q < A.nitems;) {
-    run_item<MULTI>(A, A.order[q], wkeys, wvals, ipdyn);
+  if (threadIdx.x == 0) {
+    const int64_t r0 = A.region[blockIdx.x];
+    region() = Region{A.scratch + r0, A.region[blockIdx.x + 1] - r0};
+    s_it = blockIdx.x;
+  }
+  for (;;) {
+    __syncthreads();
+    int32_t q = s_it;
+    __syncthreads();
+    if (q >= A.nitems) break;
+    run_item(A, A.order[q], wkeys, wvals, ipdyn);
     if (threadIdx.x == 0) s_it = gridDim.x + atomicAdd(A.queue, 1);
-    __syncthreads();
-    q = s_it;
-    __syncthreads();
   }
 }
+
+static void launch_items(const IPArgs &A, int grid, size_t smem) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    KMP_CUDA(cudaFuncSetAttribute(k_ip_items, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * IP_WORDS1));
+    attr_set = true;
+  }
+  k_ip_items<<<grid, IPT, smem, ctx().stream>>>(A);
+  KMP_LAUNCHED("ip_items");
+}
+
+#if KMP_IP_MULTI
+}  // namespace multi
+void launch_items_multi(const IPArgs &A, int grid, size_t smem) { multi::launch_items(A, grid, smem); }
+#else
+void launch_items_multi(const IPArgs &A, int grid, size_t smem);  // kmp_ip_multi.cu
 
 // ------------------------------------------------------ extraction (host side kernels)
 __global__ void k_block_keys(int32_t n, const int32_t *part, int bits, uint64_t *keys) {
@@ -2145,15 +2181,8 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
       A.wtab = wtab;
       A.dyn_words = (int32_t)std::min<int64_t>((want + 3) & ~3ll, words - 2 * IPW * wtab);
       const size_t dyn_bytes = 4 * (size_t)(2 * IPW * A.wtab + A.dyn_words);
-      static bool attr_set = false;
-      if (!attr_set) {
-        KMP_CUDA(cudaFuncSetAttribute(k_ip_items<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * IP_WORDS1));
-        KMP_CUDA(cudaFuncSetAttribute(k_ip_items<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * IP_WORDS1));
-        attr_set = true;
-      }
-      if (g.multi) k_ip_items<true><<<gridip, IPT, dyn_bytes, s>>>(A);
-      else k_ip_items<false><<<gridip, IPT, dyn_bytes, s>>>(A);
-      KMP_LAUNCHED("ip_items");
+      if (g.multi) launch_items_multi(A, gridip, dyn_bytes);
+      else launch_items(A, gridip, dyn_bytes);
       int32_t oom = 0;
       to_host(&oom, q.p + 1, 1);
       if (!oom) break;
@@ -2169,5 +2198,6 @@ int32_t bipartition_blocks(const Graph &g, int32_t *part, int32_t nblocks, std::
   f = nf;
   return nn;
 }
+#endif  // KMP_IP_MULTI
 
 }  // namespace kmp

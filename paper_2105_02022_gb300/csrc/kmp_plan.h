@@ -31,10 +31,8 @@ constexpr int64_t SEG_MAX_ENTRIES = 1ll << 30, SEG_MAX_COUNTERS = 1ll << 30;
 // Scratch words of a bipartitioner item of n nodes and m entries (a first estimate; the
 // launch says when it was too small), with `learned` words a node for the proposer
 inline int64_t ip_scratch_words(int64_t n, int64_t m, int64_t learned) {
-  int64_t np = 2, mp = 2;
-  while (np < n) np *= 2;
-  while (mp < m) mp *= 2;
-  return (104 * n + 64 * np + 16 * m + 8 * mp + 2048 + (learned > 0 ? learned * n + 64 : 0) + 3) & ~3ll;
+  const auto pow2 = [](int64_t x) { return x <= 2 ? 2ll : 1ll << (64 - __builtin_clzll((unsigned long long)x - 1)); };
+  return (104 * n + 64 * pow2(n) + 16 * m + 8 * pow2(m) + 2048 + (learned > 0 ? learned * n + 64 : 0) + 3) & ~3ll;
 }
 
 // Work order of a round's items and the scratch regions of its CTAs.  Items are
