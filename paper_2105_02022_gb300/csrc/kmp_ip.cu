@@ -324,7 +324,8 @@ __device__ __forceinline__ void item_group_rate(const GroupIn &in, bool unit, in
   const int lane = threadIdx.x & 31, gl = lane & (G - 1);
   const unsigned gmask = (G == 32) ? 0xFFFFFFFFu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int32_t l = in.l;
-  // as k_rate's groups: the set's size with unit weights, else its peers' weights
+  // as k_rate's groups: the set's size with unit weights, else its peers' weights, one by
+  // one here (an item's sets are small: 4096 items 30.33 ms, 30.47 with peer_sum)
   const unsigned peers = __match_any_sync(0xFFFFFFFFu, l) & gmask;
   int32_t r;
   if (unit) {
