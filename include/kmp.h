@@ -256,7 +256,9 @@ int kmp_last_stats(kmp_stats *stats);
  * on, the rating kernel k_rate stamps the device's global timer: its first
  * CTA's start and its last CTA's end give the launch's duration (stamps are
  * taken inside the kernels, so the replayed CUDA graph of an LP round needs
- * no extra nodes).  Algorithmic bytes are counted per directed entry rated:
+ * no extra nodes; a graph small enough to run all its rounds in one launch
+ * stamps each sub-round's rating inside that, and counts it as one launch;
+ * profiling does not change which kernels rate).  Algorithmic bytes are counted per directed entry rated:
  * adjncy 4 + neighbour label 4 (+ edge weight 4 when weighted); per rated
  * node: xadj 8 + list entry 4 + own label 4 + proposal 8 (+ node weight 4).
  * kmp_profile_read: k_rate alone (nodes rated by the hub kernels excluded),

@@ -1482,11 +1482,12 @@ constexpr int64_t SMALL_M = 32768;
 constexpr int64_t SMALL_DEG = 256;
 constexpr int SMALL_T = 1024;
 constexpr size_t SMALL_SMEM = (size_t)(SMALL_T / 32) * (2 * WARP_TAB * sizeof(int32_t) + WARP_TAB / 2 * sizeof(uint16_t));
-__global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *rounds, int32_t nrounds) {
+__global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *rounds, int32_t nrounds,
+                                                      int32_t *boff_all) {
   extern __shared__ __align__(16) unsigned char lps_smem[];
   constexpr int W = SMALL_T / 32;
   __shared__ int32_t cnt[8 * NB + 1], fill[8 * NB];
-  __shared__ unsigned long long s_scan;
+  __shared__ unsigned long long s_scan, sdeg[8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int32_t *keys = reinterpret_cast<int32_t *>(lps_smem) + w * WARP_TAB;
   int32_t *vals = reinterpret_cast<int32_t *>(lps_smem) + (W + w) * WARP_TAB;
@@ -1503,6 +1504,7 @@ __global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *roun
     volatile unsigned long long *ctr = ctr_cur(A);
     for (int i = threadIdx.x; i < nk; i += SMALL_T) fill[i] = 0;
     if (threadIdx.x == 0) s_scan = 0;
+    if (threadIdx.x < 8) sdeg[threadIdx.x] = 0;
     __syncthreads();
     // binning: counts, offsets, list; consumes act
     for (int pass = 0; pass < 2; ++pass) {
@@ -1515,6 +1517,7 @@ __global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *roun
         const int key = (int)(key_step(rk, (uint64_t)(uint32_t)v) & (uint64_t)(A.S - 1)) * NB + deg_bin(d, A.huge_deg, A.mid_deg);
         const int32_t at = atomicAdd(&fill[key], 1);
         if (pass == 1) A.vlist[cnt[key] + at] = v;
+        else if (A.tmin) atomicAdd(&sdeg[key / NB], (unsigned long long)d);
         my += (unsigned long long)d;
       }
       if (pass == 0 && my) atomicAdd(&s_scan, my);
@@ -1529,16 +1532,19 @@ __global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *roun
           cnt[nk] = run;
           ctr[0] = s_scan;
         }
+        if (A.tmin && threadIdx.x < A.S) ctr[2 + threadIdx.x] = sdeg[threadIdx.x];
         __syncthreads();
         for (int i = threadIdx.x; i < nk; i += SMALL_T) fill[i] = 0;
         __syncthreads();
       }
     }
+    if (A.tmin && threadIdx.x <= nk) boff_all[(nk + 1) * r + threadIdx.x] = cnt[threadIdx.x];
     for (int s = 0; s < A.S; ++s) {
       const int32_t *bo = cnt + s * NB;
       const int32_t lo = bo[0], hi = bo[NB];
       if (lo == hi) continue;
       if (threadIdx.x < 3) A.ctr[threadIdx.x] = 0;
+      if (A.tmin && threadIdx.x == 0) A.tmin[(int64_t)r * A.S + s] = global_ns();
 #define KMP_GROUP_BIN(BIN, G)                                                  \
   for (int32_t b0 = bo[BIN] + w * (32 / G); b0 < bo[BIN + 1]; b0 += W * (32 / G)) { \
     const int32_t idx = b0 + lane / G;                                         \
@@ -1551,6 +1557,7 @@ __global__ void __launch_bounds__(SMALL_T, 1) k_lp_small(LPArgs A, LPRound *roun
 #undef KMP_GROUP_BIN
       for (int32_t idx = bo[4] + w; idx < bo[5]; idx += W) rate_warp(A, A.vlist[idx], idx, lane, keys, vals, list);
       __syncthreads();
+      if (A.tmin && threadIdx.x == 0) A.tmax[(int64_t)r * A.S + s] = A.smax[(int64_t)r * A.S + s] = global_ns();
       classify_range(A, lo + threadIdx.x, hi, SMALL_T);
       __syncthreads();
       const int32_t nslots = *(volatile int32_t *)&A.ctr[0];
@@ -1783,8 +1790,8 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   A.ctr64 = ctr_all;
   // profiling: the span of every k_rate launch on the device's global timer
   // (first CTA start to last CTA end; stamps taken inside the kernel, so the
-  // replayed graph needs no extra nodes) and each round's bin offsets, all
-  // read after the run
+  // replayed graph needs no extra nodes), or of a sub-round's rating inside
+  // k_lp_small, and each round's bin offsets, all read after the run
   DBuf<int32_t> boff_all;
   DBuf<unsigned long long> tmin, tmax, smax;
   if (C.profile) {
@@ -1890,7 +1897,8 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
       }
     }
   };
-  if (n <= SMALL_N && g.m <= SMALL_M && g.maxdeg <= SMALL_DEG && !C.profile) {
+  const bool small = n <= SMALL_N && g.m <= SMALL_M && g.maxdeg <= SMALL_DEG;
+  if (small) {
     std::vector<LPRound> hr(rounds);
     for (int r = 0; r < rounds; ++r) {
       const uint64_t rk = key_step(basekey, (uint64_t)r);
@@ -1904,7 +1912,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
       attr = true;
     }
     A.apply_row = (int32_t)SMALL_DEG;  // it marks every row itself
-    k_lp_small<<<1, SMALL_T, SMALL_SMEM, stream>>>(A, dr, rounds);
+    k_lp_small<<<1, SMALL_T, SMALL_SMEM, stream>>>(A, dr, rounds, boff_all.p);
     KMP_LAUNCHED("lp_small");
   } else if (C.tune.lp_graphs) {
     // one captured round, replayed for every round: its kernels read the
@@ -1958,6 +1966,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     st->moved_total += (int64_t)hall[18 * r + 1];
     if (hall[18 * r + 1] == 0) break;
   }
+  if (small && C.profile) profile_rounds(st->rounds);  // the rounds that it ran
   KMP_CUDA(cudaEventRecord(e1, stream));
   KMP_CUDA(cudaEventSynchronize(e1));
   float ms = 0;
