@@ -87,7 +87,8 @@ __device__ __forceinline__ int64_t mp_wdeg(const GView<XT, AT> &G, bool take, in
 }
 
 // Features of one graph by one CTA; d1, d2: scratch of n ints (local index).
-// The sums are whole numbers below 2^53, so their doubles are exact.
+// The sums are whole numbers of magnitude below 2^53, so their doubles are exact; they
+// are added as unsigned words and read as signed (a batch's weights may be negative).
 template <class XT, class AT>
 __device__ void mp_features(const GView<XT, AT> &G, uint64_t key, float *X, int32_t *d1, int32_t *d2) {
   __shared__ unsigned long long s_c, s_w, s_md;
@@ -175,7 +176,7 @@ __device__ void mp_features(const GView<XT, AT> &G, uint64_t key, float *X, int3
     }
   }
   int32_t s_D1 = s_D[0], s_D2 = s_D[1];
-  double meanc = (double)s_c / (n > 0 ? n : 1), meanw = (double)s_w / (n > 0 ? n : 1);
+  double meanc = (double)(int64_t)s_c / (n > 0 ? n : 1), meanw = (double)(int64_t)s_w / (n > 0 ? n : 1);
   for (int32_t v = threadIdx.x; v < n; v += blockDim.x) {
     const double wd = (double)*reinterpret_cast<const int64_t *>(X + (int64_t)v * MF + 6);
     double deg = (double)(G.xadj[v + 1] - G.xadj[v]);
