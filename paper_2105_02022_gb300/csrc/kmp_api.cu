@@ -766,11 +766,11 @@ int kmp_set_profiling(int on) {
 int kmp_profile_read(double *rate_ms, double *rate_bytes, int64_t *rate_launches, int reset) {
   return guarded([&] {
     Context &C = ctx();
-    if (rate_ms) *rate_ms = C.prof_rate_ms;
+    if (rate_ms) *rate_ms = (double)C.prof_rate_ns * 1e-6;
     if (rate_bytes) *rate_bytes = C.prof_rate_bytes;
     if (rate_launches) *rate_launches = C.prof_rate_launches;
     if (reset) {
-      C.prof_rate_ms = 0;
+      C.prof_rate_ns = 0;
       C.prof_rate_bytes = 0;
       C.prof_rate_launches = 0;
     }
@@ -780,11 +780,11 @@ int kmp_profile_read(double *rate_ms, double *rate_bytes, int64_t *rate_launches
 int kmp_profile_read_stage(double *stage_ms, double *stage_bytes, int64_t *spans, int reset) {
   return guarded([&] {
     Context &C = ctx();
-    if (stage_ms) *stage_ms = C.prof_stage_ms;
+    if (stage_ms) *stage_ms = (double)C.prof_stage_ns * 1e-6;
     if (stage_bytes) *stage_bytes = C.prof_stage_bytes;
     if (spans) *spans = C.prof_stage_spans;
     if (reset) {
-      C.prof_stage_ms = 0;
+      C.prof_stage_ns = 0;
       C.prof_stage_bytes = 0;
       C.prof_stage_spans = 0;
     }

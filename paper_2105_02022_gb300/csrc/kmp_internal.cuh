@@ -43,9 +43,11 @@ struct Context {
   // live profiling of the LP rating launches (CUDA events on `stream`)
   bool profile = false;
   cudaStream_t capture_stream = nullptr;  // created on first use: CUDA graph capture of LP rounds
-  double prof_rate_ms = 0, prof_rate_bytes = 0;
+  uint64_t prof_rate_ns = 0;
+  double prof_rate_bytes = 0;
   int64_t prof_rate_launches = 0;
-  double prof_stage_ms = 0, prof_stage_bytes = 0;  // whole rating stage per sub-round
+  uint64_t prof_stage_ns = 0;  // whole rating stage per sub-round
+  double prof_stage_bytes = 0;
   int64_t prof_stage_spans = 0;
 };
 Context &ctx();

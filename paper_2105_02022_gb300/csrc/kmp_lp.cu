@@ -1877,6 +1877,8 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     to_host(t2.data(), smax.p, t2.size());
     bool hubs_outside = many || dense_hubs;
     const double per_entry = 8.0 + (g.ew ? 4.0 : 0.0), per_node = 24.0 + (g.vw ? 4.0 : 0.0);
+    // whole nanoseconds until the end, so that a stage's sum is never below its k_rate's
+    unsigned long long rate_ns = 0, stage_ns = 0;
     for (int r = 0; r < nr; ++r) {
       const int32_t *hboff = hb.data() + (size_t)(S * NB + 1) * r;
       for (int s = 0; s < S; ++s) {
@@ -1888,14 +1890,16 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
           D -= (double)h[18 * r + 10 + s];
         }
         size_t i = (size_t)S * r + s;
-        C.prof_rate_ms += t1[i] > t0[i] ? (double)(t1[i] - t0[i]) * 1e-6 : 0.0;
+        rate_ns += t1[i] > t0[i] ? t1[i] - t0[i] : 0;
         C.prof_rate_launches += 1;
         C.prof_rate_bytes += D * per_entry + V * per_node;
-        C.prof_stage_ms += t2[i] > t0[i] ? (double)(t2[i] - t0[i]) * 1e-6 : 0.0;
+        stage_ns += t2[i] > t0[i] ? t2[i] - t0[i] : 0;
         C.prof_stage_spans += 1;
         C.prof_stage_bytes += Dall * per_entry + Vall * per_node;
       }
     }
+    C.prof_rate_ns += rate_ns;
+    C.prof_stage_ns += stage_ns;
   };
   const bool small = n <= SMALL_N && g.m <= SMALL_M && g.maxdeg <= SMALL_DEG;
   if (small) {
