@@ -35,7 +35,6 @@ struct BalArgs {
   const int32_t *adj;
   const int32_t *vw;
   const int32_t *ew;
-  int32_t multi;         // the graph may hold parallel entries
   int32_t *part;
   int64_t *bw;
   const int32_t *cap;
@@ -394,8 +393,8 @@ __global__ void __launch_bounds__(BAL_T) k_bal_spec(BalArgs A) {
 // memory while k fits, and the blocks of the neighbours, the one gather from
 // global memory left per batch.  A batch with at most WS_E entries and WS_T table
 // slots is evaluated by warp 0 alone, in shared-memory tables; a larger one by
-// the CTA, in shared memory too while its tables fit beside the windows or over them.  Mesh of 2^20 nodes, 8192 blocks of 128 nodes brought from
-// 10% to 3% imbalance, the whole call: 97.0 -> 58.4 ms with the windows and rooms,
+// the CTA, in shared memory too while its tables fit beside the windows or over them.
+// Mesh of 2^20 nodes, 8192 blocks of 128 nodes brought from 10% to 3% imbalance, the whole call: 97.0 -> 58.4 ms with the windows and rooms,
 // 30.8 ms with small batches decided to their end (a batch used to stop at the
 // first member next to an earlier move, and its tables were built again).
 constexpr int WS_E = 256;
@@ -592,9 +591,14 @@ constexpr int32_t BAL_ROOM_K = 26000;  // rooms in shared memory: 104 KB beside 
 // more lies over the windows, which are then read again, or in global memory).
 // With all large batches over the windows, 32 windows were read again for each:
 // partition of R-MAT 2^22, k = 4096, 368.4 ms, and 353.1 like this.
+// A batch of BAL_FIT members or more that fits is preferred to one that does not: a
+// random graph of 30,000 nodes of 300 neighbours in 300 blocks 45.6 -> 13.6 ms (39.5
+// before the windows, whose reloads it paid for), 60,000 nodes of 250 in 20,000 blocks
+// 23.3 -> 11.5 (with 8 instead of 4 members 23.3).
 constexpr size_t BAL_SMEM_MAX = 224000;
+constexpr int32_t BAL_FIT = 4;
 
-template <bool SROOM>
+template <bool SROOM, bool MULTI>
 __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, int32_t slots) {
   extern __shared__ __align__(16) unsigned char bal_smem[];
   BalWindow *const win = reinterpret_cast<BalWindow *>(bal_smem);
@@ -606,7 +610,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
   __shared__ unsigned long long s_best[BM_W];
   __shared__ int32_t mk[MEMB], mv[MEMB];
   // weight from member to member of a small batch, where s_adj has the bit; parallel entries
-  // (A.multi) are summed, and their sums are zero between batches
+  // (MULTI: the graph may hold them) are summed, and their sums are zero between batches
   __shared__ int32_t adjw[32][33];
   __shared__ int32_t s_nb, s_B, s_ob, s_i, s_phase, s_done, s_large, s_hint;
   constexpr unsigned ALL = 0xFFFFFFFFu;
@@ -618,7 +622,8 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
   }
   for (int32_t x = threadIdx.x; x < A.k; x += BM_T) room[x] = (int32_t)((int64_t)A.cap[x] - A.bw[x]);
   if (threadIdx.x < MEMB) mk[threadIdx.x] = HT_EMPTY;
-  for (int x = threadIdx.x; x < 32 * 33; x += BM_T) (&adjw[0][0])[x] = 0;
+  if (MULTI)
+    for (int x = threadIdx.x; x < 32 * 33; x += BM_T) (&adjw[0][0])[x] = 0;
   if (threadIdx.x == 0) {
     s_ob = 0;
     s_i = -1;
@@ -728,9 +733,17 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
         }
         if (lane == 0) s_toff[0] = 0;
         ++n_batches;
-        n_cands += nb;
-        n_entries += E;
         if (E > WS_E || TT > (uint32_t)WS_T) {
+          // Members whose tables do not fit beside the windows are left to the next batch
+          // while BAL_FIT or more do fit: on dense graphs a batch stops at a neighbour of
+          // an earlier move after a few members, and tables in global memory, cleared and
+          // filled for all 32, cost more than the batches that this adds.
+          if (TT > (uint32_t)slots) {
+            const int32_t fit = __popc(__ballot_sync(ALL, lane < nb && tpre <= (uint32_t)slots));
+            if (fit >= BAL_FIT) nb = fit;
+          }
+          n_cands += nb;
+          n_entries += W.epre[a + nb] - e0;
           if (lane < nb) {
             s_v[lane] = v;
             s_c[lane] = c;
@@ -746,6 +759,8 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
           large = true;
           break;  // the whole CTA evaluates this batch
         }
+        n_cands += nb;
+        n_entries += E;
         __syncwarp();
         // ---- warp 0 alone: connectivity tables in shared memory
         for (int32_t t0 = 0; t0 < (int32_t)E; t0 += 32 * WS_R) {
@@ -779,7 +794,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
               const int32_t ib = memb_find(mk, mv, uu[r]);
               if (ib >= 0) {
                 atomicOr(&s_adj[jm[r]], 1u << ib);
-                if (A.multi) atomicAdd(&adjw[jm[r]][ib], wt[r]);
+                if (MULTI) atomicAdd(&adjw[jm[r]][ib], wt[r]);
                 else adjw[jm[r]][ib] = wt[r];
               }
               ht_add(wk + s_toff[jm[r]], wv + s_toff[jm[r]], s_mask[jm[r]], bk[r], wt[r]);
@@ -819,7 +834,7 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
           wk[x] = HT_EMPTY;
           wv[x] = 0;
         }
-        if (A.multi)
+        if (MULTI)
           for (uint32_t x = madj; x; x &= x - 1) adjw[lane][__ffs(x) - 1] = 0;
         mk[lane] = HT_EMPTY;
         mk[lane + 32] = HT_EMPTY;
@@ -948,6 +963,16 @@ __global__ void __launch_bounds__(BM_T) k_bal_moves(BalArgs A, int32_t *groom, i
   }
 }
 
+template <bool SROOM, bool MULTI>
+static void launch_moves(const BalArgs &A, int32_t *room, int32_t slots) {
+  static bool attr = false;
+  if (!attr) {
+    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<SROOM, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAL_SMEM_MAX));
+    attr = true;
+  }
+  k_bal_moves<SROOM, MULTI><<<1, BM_T, BAL_SMEM_MAX, ctx().stream>>>(A, room, slots);
+}
+
 int64_t balance(const Graph &g, int32_t k, const int32_t *caps_host, int32_t *part, BalStats *bs) {
   Context &C = ctx();
   cudaStream_t s = C.stream;
@@ -996,7 +1021,6 @@ int64_t balance(const Graph &g, int32_t k, const int32_t *caps_host, int32_t *pa
   A.k = k;
   A.xadj = g.xadj;
   A.adj = g.adj;
-  A.multi = g.multi ? 1 : 0;
   A.vw = g.vw;
   A.ew = g.ew;
   A.part = part;
@@ -1066,17 +1090,13 @@ int64_t balance(const Graph &g, int32_t k, const int32_t *caps_host, int32_t *pa
   A.gtab = gtab1;
   const size_t fixed = BAL_WINDOWS + BAL_TABS + (k <= BAL_ROOM_K ? (size_t)k * sizeof(int32_t) : 0);
   const int32_t slots = (int32_t)((BAL_SMEM_MAX - fixed) / (2 * sizeof(int32_t))) & ~31;
-  static bool attr = false;
-  if (!attr) {
-    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAL_SMEM_MAX));
-    KMP_CUDA(cudaFuncSetAttribute(k_bal_moves<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BAL_SMEM_MAX));
-    attr = true;
-  }
+  if (k > BAL_ROOM_K) room.alloc(k);
   if (k <= BAL_ROOM_K) {
-    k_bal_moves<true><<<1, BM_T, BAL_SMEM_MAX, s>>>(A, nullptr, slots);
+    if (g.multi) launch_moves<true, true>(A, nullptr, slots);
+    else launch_moves<true, false>(A, nullptr, slots);
   } else {
-    room.alloc(k);
-    k_bal_moves<false><<<1, BM_T, BAL_SMEM_MAX, s>>>(A, room, slots);
+    if (g.multi) launch_moves<false, true>(A, room, slots);
+    else launch_moves<false, false>(A, room, slots);
   }
   KMP_LAUNCHED("bal_moves");
   unsigned long long hm[5];
