@@ -1471,14 +1471,19 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
 // dependent reads a sub-round on one SM.  Partition of a 32,768-node mesh, whose
 // four coarse levels run here: 9.6 -> 6.9 ms.  The order of the node list inside a
 // (sub-round, bin) is arbitrary here; nothing depends on it.
-// One SM rates about 32 entries a round trip of its warps, so the bound on entries
-// is what keeps dense graphs with the kernels of all SMs.  Clustering and 8-way
-// refinement in one launch over the separate kernels, 4096 nodes: meshes of 32,000
-// entries 0.52..0.82 of the time, of 63,000 0.64..1.18, of 125,000 0.93..1.58; random
-// graphs of 33,000 0.70..1.07, of 130,000 1.67, of 516,000 2.8..3.3.  Break-even moves
-// to 60,000..90,000 entries at 500..2000 nodes.
+// One SM rates about 32 entries a round trip of its warps, so a bound on entries keeps
+// dense graphs with the kernels of all SMs.  Time in one launch over the separate
+// kernels at 4000 and 4096 nodes, unit to weighted meshes, then unit random graphs:
+//   entries      clustering               8-way refinement
+//   31,000       0.69..0.82, 0.70         0.52..0.62, 1.07
+//   47,000       0.79..0.96               0.59..0.71
+//   63,000       0.91..1.18, 1.11         0.64..0.83, 1.31
+//   92,000       1.03..1.40               0.73..1.04
+//   130,000      1.31..1.58, 1.67         0.93..1.24, 1.67
+// Break-even of random graphs moves to 60,000..90,000 entries at 500..2000 nodes.
+// Refinement starts near its end (a projected partition), as the meshes do here.
 constexpr int32_t SMALL_N = 4096;
-constexpr int64_t SMALL_M = 32768;
+constexpr int64_t SMALL_M_CLUSTER = 49152, SMALL_M_REFINE = 65536;
 constexpr int64_t SMALL_DEG = 256;
 constexpr int SMALL_T = 1024;
 constexpr size_t SMALL_SMEM = (size_t)(SMALL_T / 32) * (2 * WARP_TAB * sizeof(int32_t) + WARP_TAB / 2 * sizeof(uint16_t));
@@ -1901,7 +1906,7 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
     C.prof_rate_ns += rate_ns;
     C.prof_stage_ns += stage_ns;
   };
-  const bool small = n <= SMALL_N && g.m <= SMALL_M && g.maxdeg <= SMALL_DEG;
+  const bool small = n <= SMALL_N && g.m <= (cap ? SMALL_M_REFINE : SMALL_M_CLUSTER) && g.maxdeg <= SMALL_DEG;
   if (small) {
     std::vector<LPRound> hr(rounds);
     for (int r = 0; r < rounds; ++r) {

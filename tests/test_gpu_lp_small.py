@@ -1,5 +1,5 @@
-"""GPU tests of the one-launch LP run's bound on entries: bit-exact against the oracle on
-both sides of it, and a dense graph of as few nodes takes the kernels of all SMs."""
+"""GPU tests of the one-launch LP run's bounds on entries: bit-exact against the oracle on
+both sides of them, and a dense graph of as few nodes takes the kernels of all SMs."""
 import numpy as np
 import pytest
 import torch
@@ -9,7 +9,7 @@ from paper_2105_02022_gb300 import graphgen as gg
 
 pytestmark = pytest.mark.gpu
 
-ENTRIES = 32768
+ENTRIES = [49152, 65536]  # clustering, refinement
 
 
 @pytest.fixture(scope="module")
@@ -37,8 +37,8 @@ def _random(n, edges, seed):
     return gg.Graph(n, xadj, c[order].astype(np.int32), None, None, "random")
 
 
-@pytest.mark.parametrize("n", [400, 1500, 4096])
-@pytest.mark.parametrize("edges", [ENTRIES // 2, ENTRIES // 2 + 1])
+@pytest.mark.parametrize("n", [500, 1500, 4096])
+@pytest.mark.parametrize("edges", [e // 2 + x for e in ENTRIES for x in (0, 1)])
 @pytest.mark.parametrize("weighted", [False, True])
 def test_both_sides_of_the_bound(kmp, n, edges, weighted):
     g = _random(n, edges, n)
