@@ -1101,18 +1101,23 @@ void project(int32_t n_fine, const int32_t *map, const int32_t *part_c, int32_t 
 }
 
 // Block weights node by node, then the cut by equal shares of rows and entries: a warp
-// takes CUT_TILE consecutive ones (a row counts for one more than its entries),
-// finds the row they start in, and reads the ends and blocks of 32 rows at a time; an
+// takes one run of them (a row counts for one more than its entries), CUT_SHARE at
+// least, finds the row they start in, and reads the ends and blocks of 32 rows at a time; an
 // entry's row is the number of those that end at or before it.  So a hub's row is
 // shared by many warps, and a short row costs no round trip of its own (rows one
 // after the other on the warp that held their 32 nodes: R-MAT 2^22 1.48 ms, mesh of
 // 2^24 nodes 1.41 ms; for the cut alone).  Shares of the entries alone let one warp
 // walk all rows without entries between two of its own: 2^24 isolated nodes took
-// 293 ms, every 64th of 2^20 nodes joined 2.0 ms.  Entries before xadj[0] belong
+// 293 ms, every 64th of 2^20 nodes joined 2.0 ms.  One run a warp, since runs of a
+// fixed length leave a last wave nearly empty on large graphs and most warps without
+// any on small ones (kernel alone, runs of 2048 entries against this: mesh of 2^15
+// nodes, degree 12, 44 -> 21 us; of 2^21, weighted, 209 -> 172; R-MAT 2^21 324 -> 260);
+// below 512 the search for its rows costs more.  Entries before xadj[0] belong
 // to no row and are not read.  Weights are summed in shared memory when k is small.
 // bad (nullable) is set when a block id lies outside [0, k); such ids index nothing.
 constexpr int CUT_SBW = 2048;
-constexpr int CUT_TILE = 2304;  // 2048 entries in rows of 8, with their rows
+constexpr int CUT_SHARE = 512;
+constexpr int CUT_TILE = 2048;  // entries of a window taken together
 constexpr int CUT_U = 4;
 // The last row v with v + xadj[v] - xadj[0] <= d (d >= 0), by a warp, 32 positions a read
 __device__ __forceinline__ int64_t share_row(const int64_t *__restrict__ xadj, int32_t n, int64_t d) {
@@ -1126,6 +1131,9 @@ __device__ __forceinline__ int64_t share_row(const int64_t *__restrict__ xadj, i
   }
   return v;
 }
+// WEIGHTED: ew is not null (with the test in the loop 60 us instead of 44 for 100,000
+// entries in runs of 2304)
+template <bool WEIGHTED>
 __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k, const int64_t *__restrict__ xadj,
                                                 const int32_t *__restrict__ adj, const int32_t *__restrict__ vw,
                                                 const int32_t *__restrict__ ew, const int32_t *__restrict__ part,
@@ -1151,16 +1159,16 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   unsigned long long c = 0;
   const int64_t m0 = xadj[0], total = n + m - m0;
-  for (int64_t tile = gw; tile * CUT_TILE < total; tile += nw) {
-    const int64_t d = tile * CUT_TILE, d1 = d + CUT_TILE;
+  const int64_t share = max((total + nw - 1) / nw, (int64_t)CUT_SHARE), d = gw * share;
+  if (d < total) {
     int64_t v0 = share_row(xadj, n, d), e = m0 + d - v0, e1 = m;
-    if (d1 < total) e1 = m0 + d1 - share_row(xadj, n, d1);
+    if (d + share < total) e1 = m0 + d + share - share_row(xadj, n, d + share);
     while (e < e1) {
       const int64_t v = v0 + lane;
       const int64_t end = v < n ? xadj[v + 1] : m;
       const int32_t pv = v < n ? part[v] : -1;
       const int64_t top = (int64_t)__shfl_sync(0xFFFFFFFFu, (unsigned long long)end, 31);
-      const int64_t lim = top < e1 ? top : e1;
+      const int64_t lim = min(min(top, e1), e + CUT_TILE);
       const int32_t rel = (int32_t)(end - e < 2 * CUT_TILE ? end - e : 2 * CUT_TILE);  // row ends from e on
       const int32_t len = (int32_t)(lim - e);
       for (int32_t t0 = 0; t0 < len; t0 += 32 * CUT_U) {
@@ -1169,7 +1177,7 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
         for (int r = 0; r < CUT_U; ++r) {
           const int32_t t = t0 + 32 * r + lane;
           u[r] = t < len ? adj[e + t] : -1;
-          wt[r] = t < len && ew ? ew[e + t] : 1;
+          wt[r] = WEIGHTED && t < len ? ew[e + t] : 1;
         }
 #pragma unroll
         for (int r = 0; r < CUT_U; ++r) u[r] = u[r] >= 0 ? part[u[r]] : INT32_MIN;
@@ -1186,8 +1194,8 @@ __global__ void __launch_bounds__(256) k_cut_bw(int32_t n, int64_t m, int32_t k,
           if (t < len && u[r] != own) c += (unsigned long long)wt[r];
         }
       }
+      if (lim == top) v0 += 32;
       e = lim;
-      v0 += 32;
     }
   }
 #pragma unroll
@@ -1233,8 +1241,11 @@ void block_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw_d
 // bad, status (nullable): as in k_cut_bw; the status word goes behind bad
 static void launch_cut(const Graph &g, const int32_t *part, int32_t k, int64_t *bw, int64_t *cut, int64_t *bad,
                        const int *status) {
-  const int64_t work = std::max<int64_t>(g.n, ceil_div(g.n + g.m, CUT_TILE) * 32);
-  k_cut_bw<<<grid_for(work, 256, 8), 256, 0, ctx().stream>>>(
+  const int64_t work = std::max<int64_t>(g.n, ceil_div(g.n + g.m, CUT_SHARE) * 32);
+  const auto kernel = g.ew ? k_cut_bw<true> : k_cut_bw<false>;
+  // one wave: 5 CTAs an SM with 48 registers a thread, 6 with 40 (8 asked for, a weighted
+  // R-MAT graph of 2^19 nodes takes 107 us, one of 2^21 345)
+  kernel<<<grid_for(work, 256, g.ew ? 5 : 6), 256, 0, ctx().stream>>>(
       g.n, g.m, k, g.xadj, g.adj, g.vw, g.ew, part, reinterpret_cast<unsigned long long *>(bw),
       reinterpret_cast<unsigned long long *>(cut), reinterpret_cast<unsigned long long *>(bad), status);
   KMP_LAUNCHED("cut_bw");
@@ -1254,8 +1265,9 @@ void cut_and_weights(const Graph &g, const int32_t *part, int32_t k, int64_t *bw
 // them in one buffer: one clear, one kernel, one copy and one wait while the weights
 // are few.  Many go straight to the caller's array in a copy of their own, none are
 // copied when not asked for (k = 2^20 on a mesh of 2^21 nodes: 0.94 ms through a second
-// host buffer, 0.32 like this).
-constexpr int32_t CUT_ONE_COPY = 4096;
+// host buffer, 0.32 like this; at 4097..12,000 one copy is 4..10 us faster, at 32,768
+// two are 8).
+constexpr int32_t CUT_ONE_COPY = 16384;
 void cut_to_host(const Graph &g, const int32_t *part, int32_t k, int64_t head[3], int64_t *bw) {
   Context &C = ctx();
   DBuf<int64_t> d((size_t)k + 3);

@@ -13,7 +13,7 @@ from paper_2105_02022_gb300 import graphgen as gg
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("k", [1, 2, 4095, 4096, 4097, 1 << 20])
+@pytest.mark.parametrize("k", [1, 2, 4097, 16383, 16384, 16385, 1 << 20])
 @pytest.mark.parametrize("weighted", [False, True])
 def test_cut_and_weights(k, weighted):
     from paper_2105_02022_gb300 import _build, kmp
