@@ -132,19 +132,16 @@ __global__ void __launch_bounds__(BAL_T) k_bal_cand(BalArgs A, int32_t *big, int
     int64_t cown = conn_table(A, (int32_t)v, K, V, mask);
     int64_t c = bw_node(A, (int32_t)v);
     int64_t best = -1;
-    int32_t nadj = 0;
     for (uint32_t i = lane; i <= mask; i += 32) {
       int32_t b = K[i];
       if (b == HT_EMPTY || b == B) continue;
       if (A.bw[b] + c > A.cap[b]) continue;
-      ++nadj;
       if (V[i] > best) best = V[i];
     }
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) {
       int64_t o = (int64_t)shfl_xor64((uint64_t)best, m);
       best = o > best ? o : best;
-      nadj += __shfl_xor_sync(0xFFFFFFFFu, nadj, m);
     }
     if (best < 0 && room_somewhere(A, c)) best = 0;  // an admissible block without neighbours
     if (lane == 0 && best >= 0) {
@@ -161,7 +158,6 @@ __global__ void __launch_bounds__(BAL_T) k_bal_cand(BalArgs A, int32_t *big, int
 // (2 * gcap words; the node uses the power of two >= 2 min(degree, k)).
 __global__ void __launch_bounds__(BAL_T) k_bal_cand_big(BalArgs A, const int32_t *big, const int32_t *nbig) {
   __shared__ int64_t s_best[BAL_W];
-  __shared__ int32_t s_nadj[BAL_W];
   __shared__ int64_t s_cown;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int32_t *K = A.gtab + (int64_t)blockIdx.x * 2 * A.gcap, *V = K + A.gcap;
@@ -189,7 +185,6 @@ __global__ void __launch_bounds__(BAL_T) k_bal_cand_big(BalArgs A, const int32_t
     __syncthreads();
     const int64_t c = bw_node(A, v);
     int64_t best = -1;
-    int32_t nadj = 0;
     for (uint32_t x = threadIdx.x; x < cap; x += BAL_T) {
       const int32_t blk = K[x];
       if (blk == HT_EMPTY) continue;
@@ -198,26 +193,21 @@ __global__ void __launch_bounds__(BAL_T) k_bal_cand_big(BalArgs A, const int32_t
         continue;
       }
       if (A.bw[blk] + c > A.cap[blk]) continue;
-      ++nadj;
       if (V[x] > best) best = V[x];
     }
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) {
       int64_t o = (int64_t)shfl_xor64((uint64_t)best, m);
       best = o > best ? o : best;
-      nadj += __shfl_xor_sync(0xFFFFFFFFu, nadj, m);
     }
     if (lane == 0) {
       s_best[w] = best;
-      s_nadj[w] = nadj;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
       int64_t bb = -1;
-      int32_t na = 0;
       for (int x = 0; x < BAL_W; ++x) {
         bb = s_best[x] > bb ? s_best[x] : bb;
-        na += s_nadj[x];
       }
       if (bb < 0 && room_somewhere(A, c)) bb = 0;  // an admissible block without neighbours
       if (bb >= 0) {

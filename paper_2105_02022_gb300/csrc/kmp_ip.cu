@@ -305,10 +305,6 @@ __device__ void item_rate(const LG &g, int32_t u, const uint16_t *label, const i
   __syncwarp();
 }
 
-// rating of 32 / G nodes by one warp, G lanes per node (degree <= G, one
-// neighbour per lane; u < 0: no node): lanes of a group holding the same
-// label form a peer set whose weight sum is that label's rating.  Same
-// decision as item_rate.
 // inputs of one group node: neighbour label and edge weight of this lane, own
 // label and node weight (u < 0: no node)
 struct GroupIn {
@@ -1279,7 +1275,7 @@ __device__ FMState cta_fm_state(const LG &g, int32_t *dyn, int32_t dyn_words, in
   return F;
 }
 
-// portfolio initial bipartition by one warp: algo 0 random, 1 BFS, 2 GGG
+// portfolio initial bipartition by one warp:
 // algo 0 random, 1 BFS, 2 greedy graph growing, 3 learned (first fit in the
 // order of `score`, like random with a learned order)
 __device__ void warp_initial(int algo, const LG &g, int32_t t0, uint64_t key, int32_t *side,

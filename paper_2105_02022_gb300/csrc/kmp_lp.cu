@@ -98,7 +98,6 @@ struct LPArgs {
   // into bucket order and aggregated one bucket per warp in shared memory
   const int32_t *hubs;         // hub node ids, ascending
   const int32_t *hpos;         // per node, its index among them (when it is one)
-  int32_t nhubs;
   unsigned long long *hkc;     // best admissible key per hub
   unsigned long long *hku;     // best key per hub
   int32_t *hrown;              // rating of the hub's own cluster
@@ -1745,7 +1744,6 @@ void lp_run(const Graph &g, int32_t *label, int32_t *wt, int32_t nlab, const int
   A.bigmove = bigmove;
   A.hubs = hubs.p;
   A.hpos = hpos.p;
-  A.nhubs = nhubs;
 
   A.hkc = hkc.p;
   A.hku = hku.p;
