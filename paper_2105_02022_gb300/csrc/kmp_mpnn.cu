@@ -145,9 +145,11 @@ __device__ __forceinline__ void mp_load_tile(float *dst, const float *__restrict
 // shared memory as floats, input-major, for the whole launch; a thread keeps a
 // 4 x 4 block of outputs in registers, so 32 multiply-adds take six 16-byte
 // shared reads instead of a global read each.  READOUT: the scores of the
-// tile's nodes as well, from the tile in shared memory.  Bound by FP32
-// issue (layer 2 of 325,000 nodes: 5.3 GFLOP).  Both layers with the read-out:
-// 8.9 ms with one output a thread and strided weight reads, 0.24 ms now.
+// tile's nodes as well, from the tile in shared memory.  Bound by
+// latency: layer 2 of 325,000 nodes, 5.3 GFLOP in 0.21 ms, keeps the FMA pipe 34 % busy
+// and issues in 42 % of cycles; the eight warps of each of two CTAs an SM wait for the
+// tile's global loads and for shared reads.  Both layers with the read-out: 8.9 ms with
+// one output a thread and strided weight reads, 0.24 ms now.
 template <int DIN, bool READOUT>
 constexpr size_t mp_layer_smem() {
   return sizeof(float) * (2 * DIN * MH + 2 * MP_TILE * (DIN + 4) + (READOUT ? MP_TILE * MP_LD : 0));
@@ -272,8 +274,9 @@ __global__ void k_mp_loss(int32_t ng, const int32_t *noff, const float *S, const
 // gA2 = relu'(h2) gS w_o in shared memory only; the read-out's and layer 2's
 // weight gradients; and the layer's input gradients gH1[v][i] = sum_o
 // W2s[o][i] gA2[v][o], gM1 likewise with W2n.  Threads hold 4 x 4 blocks as in
-// k_mp_layer.  Bound by FP32 issue (325,000 nodes: 10.6 GFLOP); 1.8 ms as five
-// kernels with gA2 in global memory, 0.41 ms now.
+// k_mp_layer.  Bound by latency too (325,000 nodes, 10.6 GFLOP: FMA pipe 40 %, issue
+// 52 % of cycles; waits for the tile's loads); 1.8 ms as five kernels with gA2 in
+// global memory, 0.41 ms now.
 constexpr size_t MP_BW2_SMEM = sizeof(float) * (4 * MP_TILE * MP_LD + 2 * MH * MH + MP_TILE + MH);
 __global__ void __launch_bounds__(MP_T) k_mp_bw2(int32_t N, const __nv_bfloat16 *__restrict__ W,
                                                  const float *__restrict__ gS, const float *__restrict__ H2,
